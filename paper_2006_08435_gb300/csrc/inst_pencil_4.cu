@@ -1,0 +1,8 @@
+// Pencil kernels (pencil.cuh) of the plannable edges of rank 4 modulo 8.
+#include "pencil.cuh"
+
+namespace fft3d {
+PencilKernel pencil_kernel_unit4(int L, int dir, int kind) {
+  return pc::unit_kernel<4>(L, dir, kind);
+}
+}  // namespace fft3d

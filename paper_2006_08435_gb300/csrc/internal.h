@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
 #include <vector>
 
 #include "fft3d.h"
@@ -91,94 +92,64 @@ struct FastDiv {
 };
 FastDiv make_fastdiv(unsigned d);
 
-// One pencil length, planned on the host: the radices of its
-// decimation-in-frequency stages and the device tables (W_L^m, m < L, FP64
-// rounded to FP32; the position each output K holds after the stages).
-struct AxisTable {
-  int L = 0, nst = 0;
-  int radix[kAxisMaxStages] = {};
-  float2* d_tw = nullptr;
-  unsigned short* d_pos = nullptr;
-};
 int axis_stages(int L, int* radix);                              // 0: not plannable
 void axis_positions(int L, int nst, const int* radix, int* pos);  // pos[K], K < L
 
-// Which pencils a pass transforms.  contiguous: `rows` rows of L points
-// packed back to back (the x pass).  Strided: for each of `outer` slices,
-// the nx pencils at base + x (x < nx), element i at + i * pi, with
-// base = (outer / d1) * s1 + (outer % d1) * s0.
-struct AxisGeom {
-  int contiguous = 0;
-  long long rows = 0;
-  long long outer = 0;
-  int nx = 0, d1 = 1;
-  long long s1 = 0, s0 = 0, pi = 0;
-  float scale = 1.0f;
-  int do_scale = 0;
-};
-
-// Kernel arguments of one pass (axis.cu).
-struct AxisArgs {
-  const float2* in;  // may equal out (a tile is read before it is written)
+// Register-first pencil passes (pencil.cuh).  np pencils; strided kind:
+// pencil p starts at (p / nx) * so + p % nx, its points pi apart; the other
+// kinds: rows packed back to back.  tw[k * A + n1] = W_L^(n1 k) (k < L / A);
+// real rows: twr[k] = W_2L^k, k <= L.
+enum { kEvictNormal = 0, kEvictFirst = 1, kEvictLast = 2 };
+struct PencilArgs {
+  const float2* in;  // may equal out (complex kinds)
   float2* out;
   const float2* tw;
-  const unsigned short* pos;
-  int L, nst, W, lw;  // W = 2^lw pencils per tile
-  int radix[kAxisMaxStages], span[kAxisMaxStages], sub[kAxisMaxStages], twst[kAxisMaxStages];
-  FastDiv divsub[kAxisMaxStages];  // division by sub[t], the span M of a stage's sub-blocks
-  FastDiv divL;
-  int swsh, swmask;  // tile slot of (i, c): i * (W + 1) + (c ^ ((i >> swsh) & swmask))
-  int contiguous;
-  unsigned ntiles;
-  long long rows;
-  long long outer;     // strided: slices in all
-  int nx, xtiles, d1;  // strided: tile -> (slice group, x0 = 16 * (tile % xtiles))
-  FastDiv divx, divd1;
-  long long s1, s0, pi;
+  const float2* twr;
+  unsigned np, nx;
+  FastDiv divn;  // by nx
+  long long so, pi;
   float scale;
   int do_scale;
+  int pol_in, pol_out;  // L2 policies of the loads and the stores
 };
-// The x and y passes fused for planes that fit shared memory (axis.cu):
-// one nx x ny plane per block at a time, x stages over its rows, y stages
-// over its columns, one read and one write of the plane.
-struct AxisStages {
-  int L, nst;
-  int radix[kAxisMaxStages], span[kAxisMaxStages], sub[kAxisMaxStages], twst[kAxisMaxStages];
-  FastDiv divsub[kAxisMaxStages];
-};
-struct PlaneArgs {
-  const float2* in;
-  float2* out;
-  const float2 *twx, *twy;
-  const unsigned short *posx, *posy;
-  AxisStages sx, sy;
-  int nx, ny, px;      // row pitch px: odd, >= nx
-  int rsh, rmask;      // element x of a row sits at x ^ ((x >> rsh) & rmask)
-  FastDiv divnx, divny;
-  unsigned nplanes;
-};
-struct PlaneLaunch {
-  PlaneArgs args{};
-  int dir = -1;
-  int grid = 0, threads = 0;
+struct PencilKernel {
+  cudaError_t (*launch)(const PencilArgs&, cudaStream_t) = nullptr;
+  const void* func = nullptr;
+  int A = 0, width = 0;  // split L = A * B; pencils per block
   size_t smem = 0;
 };
-// Shared memory a plane pass of an nx x ny plane needs (0 if it does not fit).
-size_t plane_pass_smem(int nx, int ny);
-int prepare_plane_pass(const AxisTable& tx, const AxisTable& ty, int dir, long long planes, int sms,
-                       PlaneLaunch* out);
-cudaError_t launch_plane_pass(const PlaneLaunch& l, const float2* in, float2* out,
-                              cudaStream_t stream);
+// kind: 0 strided, 1 rows, 2 real rows of 2 L points forward (dir -1), 3 the
+// same inverse (dir 1); launch is null for an edge that is not plannable.
+PencilKernel pencil_kernel_info(int L, int dir, int kind);
 
-struct AxisLaunch {
-  AxisArgs args{};
-  int dir = -1;
-  int nbuf = 1;  // tile buffers per block
-  int grid = 0;
-  size_t smem = 0;
+// A 3D transform as three pencil passes (passes.cu): complex grids (x, y, z,
+// out of place or in place), real grids to half spectra (x, y, z) or back
+// (z into a workspace of work_points() complex points, y, x).
+constexpr int kMaxChains = 2;
+enum PassKind { kPassC2C = 0, kPassR2C = 1, kPassC2R = 2 };
+struct AxisPasses {
+  PassKind kind = kPassC2C;
+  int nx = 0, ny = 0, nz = 0, hx = 0, batch = 0;  // hx: complex columns of a row
+  long long chunk = 0;  // grids per chunk
+  long long sub = 0;    // planes per launch of the x and y passes
+  PencilKernel k[3];
+  int chains = 1;       // streams the chunks alternate between
+  cudaStream_t side = nullptr;
+  cudaEvent_t fork = nullptr, join = nullptr;
+  std::mutex* mu = nullptr;
+  float2* d_tab = nullptr;
+  const float2* tw[3] = {nullptr, nullptr, nullptr};
+  const float2* twr = nullptr;
+  float scale = 1.0f;
+  int do_scale = 0;
+  int create(PassKind kind, int nx, int ny, int nz, int batch, int dir, float scale, int do_scale,
+             int l2_bytes);
+  void destroy();
+  long long work_points() const;
+  cudaError_t execute(const void* in, void* out, float2* work, cudaStream_t s) const;
+  cudaError_t chunk_passes(long long g, const void* in, void* out, float2* work,
+                           cudaStream_t s) const;
 };
-int prepare_axis_pass(const AxisTable& tab, int dir, const AxisGeom& g, int sms, AxisLaunch* out);
-cudaError_t launch_axis_pass(const AxisLaunch& l, const float2* in, float2* out, cudaStream_t stream);
 
 // Defined in the inst_*.cu translation units.
 KernelInfo fused_kernel_info(int n, int dir, int variant);   // single-size kernel

@@ -1,0 +1,440 @@
+// Register-first 1D transforms of pencils for every edge L, 2 <= L <= 512,
+// with prime factors 2, 3, 5: the passes of the general path (the 1D FFTs
+// along x, then y, then z of the paper's section "Approach").
+//
+// L = A * B, both register codelets (B >= A as close as they come).  With
+// n = n1 + A n2 and k = k2 + B k1:
+//   phase 1: thread (pencil, n1) loads the B points n1 + A n2 straight from
+//            global memory into registers, DFT_B, times W_L^(n1 k2), to
+//            shared memory;
+//   phase 2: thread (pencil, k2) reads its A values, DFT_A, and stores the
+//            outputs k2 + B k1 straight to global memory, in natural order.
+// One round trip through shared memory (16 bytes per point) and one barrier
+// per tile, every index of a butterfly a compile-time constant; B loads of
+// every thread are in flight at once.  The kernels before staged a tile by
+// cp.async and ran two or more in-place stages and a digit-reversed read
+// there (32 bytes and more of shared-memory traffic per point, run-time
+// radices): 96 x 128 x 64, 64 grids 524 -> 412 us by the kernels alone, 261
+// with the launches and chunks of passes.cu; 256^3 x 4 827 -> 396; 100^3 x
+// 16 174 -> 94.  A pass is bound by its 16 bytes of traffic per point: 256^3
+// passes run at the HBM copy rate, L2-resident ones of 50 MB take 16 us of
+// which a copy kernel takes 12 (its ramp and drain 4).
+//
+// A block waits for nothing but its predecessor launch: passes are
+// programmatic dependent launches (launch_dependents at the start, wait
+// before the first read), so a pass's blocks are resident when the pass
+// before it drains (96 x 128 x 64, 64 grids, one chain: 412 -> 372 us).
+// L2 policies: inputs read once and final outputs evict first, the
+// intermediate last (256^3 x 4 455 -> 418 us, small ones 1-2%).
+//
+// Strided pencils (y and z): lanes are consecutive pencils.  The pencils of
+// a pass are numbered p = o * nx + x and start at o * so + x, so that a run
+// of lanes crosses row ends without idle lanes whatever nx is (the half
+// spectra of real grids have n/2 + 1 columns); the z pass takes a whole
+// plane as one row (nx = plane, so = grid).  Contiguous pencils (x): lanes
+// are consecutive n1 (loads) and k2 (stores) of a row.
+//
+// Real rows of n = 2 L points (kinds kR2C, kC2R) are contiguous pencils of
+// z[m] = r[2m] + i r[2m+1] with Z[k] = E[k] + i O[k], E and O the transforms
+// of the even and odd samples, X[k] = E[k] + W_n^k O[k], k = 0 .. L.  The
+// split needs Z[k] and Z[L-k], which are outputs of the phase-2 items k2 and
+// B - k2: one thread takes both and splits in registers.  The inverse undoes
+// the split as it loads, one thread taking the points of n1 and A - n1.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include <utility>
+
+#include "codelets.cuh"
+#include "internal.h"
+
+namespace fft3d {
+namespace pc {
+
+enum { kStrided = 0, kContig = 1, kR2C = 2, kC2R = 3, kKinds = 4 };
+
+constexpr bool smooth(int n) {
+  if (n < 2) return false;
+  while (n % 2 == 0) n /= 2;
+  while (n % 3 == 0) n /= 3;
+  while (n % 5 == 0) n /= 5;
+  return n == 1;
+}
+constexpr bool codelet(int r) {
+  return r == 1 || r == 2 || r == 3 || r == 4 || r == 5 || r == 6 || r == 8 || r == 9 || r == 10 ||
+         r == 12 || r == 15 || r == 16 || r == 18 || r == 20 || r == 24 || r == 25 || r == 27 ||
+         r == 32;
+}
+// The smaller factor A of the split; B = L / A.  Strided pencils of a
+// codelet's length stay in one thread (no exchange); rows are split from 8
+// points up so that the lanes of a warp share rows.
+constexpr int split_a(int L, int kind) {
+  if (codelet(L) && (kind == kStrided || L < 8)) return 1;
+  int best = 0;
+  for (int a = 1; a * a <= L; ++a)
+    if (L % a == 0 && codelet(a) && codelet(L / a)) best = a;
+  return best;
+}
+// Threads of a block: the multiple of 32 up to 512 that leaves the fewest
+// lanes idle over the two phases (n1 items of work w1, then n2 of w2), at
+// most four items per thread and phase.
+constexpr int block_threads(int n1, int w1, int n2, int w2) {
+  int best = 0;
+  long best_cost = 0;
+  const int need = n1 > n2 ? n1 : n2;
+  for (int t = 512; t >= 128; t -= 32) {
+    if (t - 31 > need && t > 128) continue;
+    const int i1 = (n1 + t - 1) / t, i2 = (n2 + t - 1) / t;
+    if (i1 > 4 || i2 > 4) continue;
+    const long cost = (long)t * ((long)i1 * w1 + (long)i2 * w2);
+    if (!best || cost * 100 < best_cost * 98) {
+      best = t;
+      best_cost = cost;
+    }
+  }
+  return best ? best : 512;
+}
+// Pencils per block: 16 (a 128-byte run of columns) at the long edges, more
+// at the short ones, about 2048 points.
+constexpr int tile_pencils(int L, int A) {
+  if (A == 1) return 64;
+  int w = 16;
+  while (w < 64 && 2 * w * L <= 2048) w *= 2;
+  return w;
+}
+
+// Pitch of staged rows of R points written by lanes that walk `run`
+// consecutive points of a row, then the next row: odd rows are packed (one
+// run of memory), even ones padded (to an even pitch: 16-byte copies) so
+// that the next row's banks follow on.
+constexpr int stage_pitch(int R, int run) {
+  if (R % 2) return R;
+  int p = R;
+  while (p % 16 != (run + 1) / 2 * 2 % 16) p += 2;
+  return p;
+}
+
+// Registers a thread may use (complex kinds), so that the compiler aims at
+// 32 warps and more: 256^3 x 4 419 -> 395, 100^3 x 16 102 -> 94 us.
+constexpr int reg_budget(int B) { return B <= 8 ? 48 : B <= 12 ? 56 : B <= 16 ? 64 : 96; }
+
+template <int L, int KIND>
+struct Cfg {
+  static constexpr int A = split_a(L, KIND), B = L / A;
+  static constexpr int W = tile_pencils(L, A);
+  // items of the two phases (real rows: mirrored pairs where the split is)
+  static constexpr int N1 = W * (KIND == kC2R && A > 1 ? A / 2 + 1 : A);
+  static constexpr int N2 = A == 1 ? 0 : W * (KIND == kR2C ? B / 2 + 1 : B);
+  static constexpr int T = block_threads(N1, KIND == kC2R ? 2 * B : B, N2, KIND == kR2C ? 2 * A : A);
+  static constexpr int I1 = (N1 + T - 1) / T, I2 = (N2 + T - 1) / T;
+  // contiguous kinds: exchange slot of (pencil, k2, n1); odd pitch of k2
+  static constexpr int AP = A | 1, RP = B * AP;
+  static constexpr int exchange = A == 1 ? 0 : KIND == kStrided ? W * L : W * RP;
+  // Half spectra leave through shared memory, as packed rows of L + 1 points,
+  // where the direct stores' runs of B / 2 + 1 points would split most
+  // sectors: forward 96^3 (B = 8) 135 -> 117 us, 160^3 (B = 10) 76 -> 69,
+  // but 256^3 (B = 16) 129 -> 143.
+  static constexpr bool staged = KIND == kR2C && B <= 10;
+  static constexpr int OP = stage_pitch(L + 1, A == 1 ? 1 : B / 2 + 1);
+  static constexpr size_t smem =
+      sizeof(float2) * (size_t)(exchange + (staged ? W * OP : 0));
+  static constexpr int blocks = KIND == kStrided || KIND == kContig ? 65536 / (T * reg_budget(B)) : 1;
+  static_assert(A >= 1, "no split into two codelets");
+  static_assert(KIND == kStrided || KIND == kContig || L <= 256, "real rows hold 2 L points");
+};
+
+__device__ __forceinline__ unsigned fdiv(unsigned n, FastDiv d) {
+  return (unsigned)(((unsigned long long)__umulhi(n, d.mul) + n) >> d.shift);
+}
+
+// L2 policy of a pass's loads or stores (kEvictNormal, kEvictFirst, kEvictLast).
+__device__ __forceinline__ uint64_t l2_policy(int which) {
+  uint64_t n, f, l;
+  asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(n));
+  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(f));
+  asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(l));
+  return which == kEvictFirst ? f : which == kEvictLast ? l : n;
+}
+__device__ __forceinline__ float2 ldg(const float2* p, uint64_t pol) {
+  float2 v;
+  asm volatile("ld.global.L2::cache_hint.v2.f32 {%0, %1}, [%2], %3;"
+               : "=f"(v.x), "=f"(v.y) : "l"(p), "l"(pol));
+  return v;
+}
+__device__ __forceinline__ void stg(float2* p, float2 v, uint64_t pol) {
+  asm volatile("st.global.L2::cache_hint.v2.f32 [%0], {%1, %2}, %3;"
+               ::"l"(p), "f"(v.x), "f"(v.y), "l"(pol) : "memory");
+}
+
+// `rows` consecutive rows of R points from pitch P in shared memory, packed
+// at g.  Even R: every row starts on 16 bytes (the grids do).  Odd R: the
+// packed run may start on 8 bytes.
+__device__ __forceinline__ void stg16(float2* g, const float2* s, float sc, uint64_t pol) {
+  float4 v = *reinterpret_cast<const float4*>(s);
+  asm volatile("st.global.L2::cache_hint.v4.f32 [%0], {%1, %2, %3, %4}, %5;"
+               ::"l"(g), "f"(v.x * sc), "f"(v.y * sc), "f"(v.z * sc), "f"(v.w * sc), "l"(pol) : "memory");
+}
+template <int R, int P, int T>
+__device__ __forceinline__ void rows_out(float2* g, const float2* s, int rows, float sc, uint64_t pol) {
+  if constexpr (R % 2 == 0) {
+    for (int u = threadIdx.x; u < rows * (R / 2); u += T)
+      stg16(g + 2 * u, s + u / (R / 2) * P + 2 * (u % (R / 2)), sc, pol);
+  } else if ((reinterpret_cast<uintptr_t>(g) & 15) == 0) {
+    const int n = rows * R;
+    for (int u = threadIdx.x; u < n / 2; u += T) stg16(g + 2 * u, s + 2 * u, sc, pol);
+    if ((n & 1) && threadIdx.x == 0) stg(g + n - 1, cscale(s[n - 1], sc), pol);
+  } else {
+    for (int u = threadIdx.x; u < rows * R; u += T) stg(g + u, cscale(s[u], sc), pol);
+  }
+}
+
+// Half spectrum of a real row of 2 L points from Z: X[k] = E + W_n^k O and
+// X[L-k] = conj(E - W_n^k O), E = (Z[k] + conj Z[L-k]) / 2,
+// O = -i (Z[k] - conj Z[L-k]) / 2.  z[k1] = Z[k2 + B k1]; mz holds the
+// mirrors: mz[A-1-k1] = Z[L-k2-B k1], or, for k2 = 0, z itself with
+// Z[L - B k1] = z[(A - k1) % A].  A = 1 (L = B): z and mz are the row.
+template <int L, int A, bool STAGED>
+__device__ __forceinline__ void split_store(const PencilArgs& a, float2* dst, const float2* z,
+                                            const float2* mz, int k2, uint64_t pout) {
+  constexpr int B = L / A, N = A == 1 ? L : A, S = A == 1 ? 1 : B;
+#pragma unroll
+  for (int k1 = 0; k1 < N; ++k1) {
+    const int k = k2 + S * k1;
+    const float2 u = z[k1], m = k2 == 0 ? z[(N - k1) % N] : mz[N - 1 - k1];
+    const float2 E = make_float2(0.5f * (u.x + m.x), 0.5f * (u.y - m.y));
+    const float2 O = make_float2(0.5f * (u.y + m.y), 0.5f * (m.x - u.x));
+    const float2 t = cmul_tw<-1>(O, __ldg(a.twr + k));
+    float2 lo = cadd(E, t), hi = make_float2(E.x - t.x, t.y - E.y);
+    if constexpr (STAGED) {
+      dst[k] = lo;
+      dst[L - k] = hi;
+    } else {
+      if (a.do_scale) {
+        lo = cscale(lo, a.scale);
+        hi = cscale(hi, a.scale);
+      }
+      stg(dst + k, lo, pout);
+      stg(dst + L - k, hi, pout);
+    }
+  }
+}
+
+template <int L, int DIR, int KIND>
+__global__ void __launch_bounds__(Cfg<L, KIND>::T, Cfg<L, KIND>::blocks) pencil_kernel(const PencilArgs a) {
+  using C = Cfg<L, KIND>;
+  constexpr int A = C::A, B = C::B, W = C::W, T = C::T;
+  extern __shared__ __align__(16) float2 sm[];
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const unsigned p0 = blockIdx.x * (unsigned)W;
+  const float sc = a.scale;
+  const uint64_t pin = l2_policy(a.pol_in), pout = l2_policy(a.pol_out);
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+
+  // first point of pencil p (in: input side, else output side)
+  auto base = [&](unsigned p, bool in) -> long long {
+    if constexpr (KIND == kStrided) {
+      const unsigned o = fdiv(p, a.divn);
+      return (long long)o * a.so + (long long)(p - o * a.nx);
+    } else {
+      const int pitch = KIND == kR2C && !in ? L + 1 : KIND == kC2R && in ? L + 1 : L;
+      return (long long)p * pitch;
+    }
+  };
+
+  // phase 1
+#pragma unroll 1
+  for (int it = 0; it < C::I1; ++it) {
+    const int e = threadIdx.x + it * T;
+    if (e >= C::N1) break;
+    if constexpr (KIND == kC2R) {
+      // Z[k] = 2 E + i 2 O and Z[L-k] = conj(2 E) + i conj(2 O) with
+      // 2 E = X[k] + conj X[L-k], 2 O = (X[k] - conj X[L-k]) W_n^-k: the item
+      // of n1 makes the points n1 + A j and their mirrors, A - n1 + A j (its
+      // own points for n1 = 0 and A / 2).  Of X[0] and X[L] only the real
+      // parts count.
+      constexpr int H = A > 1 ? A / 2 + 1 : 1;
+      const int c = e / H, n1 = e % H;
+      const unsigned p = p0 + (unsigned)c;
+      if (p >= a.np) continue;
+      const float2* src = a.in + base(p, true);
+      float2 u[B], m[B];
+#pragma unroll
+      for (int j = 0; j < B; ++j) {
+        u[j] = ldg(src + n1 + A * j, pin);
+        m[j] = ldg(src + L - n1 - A * j, pin);
+      }
+      if (n1 == 0) u[0].y = m[0].y = 0.0f;
+#pragma unroll
+      for (int j = 0; j < B; ++j) {
+        const float2 s = make_float2(u[j].x + m[j].x, u[j].y - m[j].y);
+        const float2 d = make_float2(u[j].x - m[j].x, u[j].y + m[j].y);
+        const float2 t = cmul_tw<1>(d, __ldg(a.twr + n1 + A * j));
+        u[j] = make_float2(s.x - t.y, s.y + t.x);
+        m[j] = make_float2(s.x + t.y, t.x - s.y);
+      }
+      DFT<B, DIR>::run(u);
+      if constexpr (A > 1) {
+#pragma unroll
+        for (int k = 0; k < B; ++k)
+          sm[c * C::RP + k * C::AP + n1] = k ? cmul_tw<DIR>(u[k], __ldg(a.tw + k * A + n1)) : u[k];
+        if (n1 != 0 && 2 * n1 != A) {
+          float2 v[B];
+#pragma unroll
+          for (int j = 0; j < B; ++j) v[j] = m[B - 1 - j];
+          DFT<B, DIR>::run(v);
+          const int n2 = A - n1;
+#pragma unroll
+          for (int k = 0; k < B; ++k)
+            sm[c * C::RP + k * C::AP + n2] = k ? cmul_tw<DIR>(v[k], __ldg(a.tw + k * A + n2)) : v[k];
+        }
+      } else {
+        float2* dst = a.out + base(p, false);
+#pragma unroll
+        for (int k = 0; k < B; ++k) stg(dst + k, a.do_scale ? cscale(u[k], sc) : u[k], pout);
+      }
+    } else {
+      const int c = KIND == kStrided ? e % W : e / A;
+      const int n1 = KIND == kStrided ? e / W : e % A;
+      const unsigned p = p0 + (unsigned)c;
+      if (p >= a.np) continue;
+      const float2* src = a.in + base(p, true);
+      const long long step = KIND == kStrided ? (long long)A * a.pi : A;
+      src += KIND == kStrided ? (long long)n1 * a.pi : n1;
+      float2 v[B];
+#pragma unroll
+      for (int j = 0; j < B; ++j) v[j] = ldg(src + j * step, pin);
+      DFT<B, DIR>::run(v);
+      if constexpr (A > 1) {
+#pragma unroll
+        for (int k = 0; k < B; ++k) {
+          const float2 y = k ? cmul_tw<DIR>(v[k], __ldg(a.tw + k * A + n1)) : v[k];
+          sm[KIND == kStrided ? (k * A + n1) * W + c : c * C::RP + k * C::AP + n1] = y;
+        }
+      } else if constexpr (KIND == kR2C) {
+        split_store<L, 1, true>(a, sm + c * C::OP, v, v, 0, pout);
+      } else {
+        float2* dst = a.out + base(p, false);
+        const long long ostep = KIND == kStrided ? a.pi : 1;
+#pragma unroll
+        for (int k = 0; k < B; ++k) stg(dst + k * ostep, a.do_scale ? cscale(v[k], sc) : v[k], pout);
+      }
+    }
+  }
+
+  // phase 2
+  if constexpr (A > 1) {
+    __syncthreads();
+#pragma unroll 1
+    for (int it = 0; it < C::I2; ++it) {
+      const int e = threadIdx.x + it * T;
+      if (e >= C::N2) break;
+      constexpr int H = KIND == kR2C ? B / 2 + 1 : B;  // items of a row
+      const int c = KIND == kStrided ? e % W : e / H;
+      const int k2 = KIND == kStrided ? e / W : e % H;
+      const unsigned p = p0 + (unsigned)c;
+      if (p >= a.np) continue;
+      float2 v[A];
+#pragma unroll
+      for (int j = 0; j < A; ++j)
+        v[j] = sm[KIND == kStrided ? (k2 * A + j) * W + c : c * C::RP + k2 * C::AP + j];
+      DFT<A, DIR>::run(v);
+      if constexpr (KIND == kR2C) {
+        float2* row = C::staged ? sm + C::exchange + c * C::OP : a.out + base(p, false);
+        // the mirrors of this item's outputs are those of B - k2
+        if (k2 == 0 || 2 * k2 == B) {
+          split_store<L, A, C::staged>(a, row, v, v, k2, pout);
+        } else {
+          float2 w[A];
+#pragma unroll
+          for (int j = 0; j < A; ++j) w[j] = sm[c * C::RP + (B - k2) * C::AP + j];
+          DFT<A, DIR>::run(w);
+          split_store<L, A, C::staged>(a, row, v, w, k2, pout);
+        }
+      } else {
+        float2* dst = a.out + base(p, false);
+        if (a.do_scale) {
+#pragma unroll
+          for (int k = 0; k < A; ++k) v[k] = cscale(v[k], sc);
+        }
+        const long long step = KIND == kStrided ? (long long)B * a.pi : B;
+        dst += KIND == kStrided ? (long long)k2 * a.pi : k2;
+#pragma unroll
+        for (int k = 0; k < A; ++k) stg(dst + k * step, v[k], pout);
+      }
+    }
+  }
+
+  if constexpr (C::staged) {
+    __syncthreads();
+    const int rows = (int)min((unsigned)W, a.np - p0);
+    rows_out<L + 1, C::OP, T>(a.out + (size_t)p0 * (L + 1), sm + C::exchange, rows,
+                              a.do_scale ? sc : 1.0f, pout);
+  }
+}
+
+template <int L, int DIR, int KIND>
+cudaError_t launch(const PencilArgs& a, cudaStream_t s) {
+  using C = Cfg<L, KIND>;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((a.np + C::W - 1) / C::W, 1, 1);
+  cfg.blockDim = dim3(C::T, 1, 1);
+  cfg.dynamicSmemBytes = C::smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, &pencil_kernel<L, DIR, KIND>, a);
+}
+
+template <int L, int DIR, int KIND>
+PencilKernel entry() {
+  using C = Cfg<L, KIND>;
+  PencilKernel k;
+  k.launch = &launch<L, DIR, KIND>;
+  k.func = (const void*)&pencil_kernel<L, DIR, KIND>;
+  k.A = C::A;
+  k.smem = C::smem;
+  k.width = C::W;
+  return k;
+}
+
+template <int L>
+PencilKernel entry_of(int dir, int kind) {
+  if (kind == kStrided) return dir < 0 ? entry<L, -1, kStrided>() : entry<L, 1, kStrided>();
+  if (kind == kContig) return dir < 0 ? entry<L, -1, kContig>() : entry<L, 1, kContig>();
+  if constexpr (L <= 256) {
+    if (kind == kR2C && dir < 0) return entry<L, -1, kR2C>();
+    if (kind == kC2R && dir > 0) return entry<L, 1, kC2R>();
+  }
+  return PencilKernel{};
+}
+
+// The plannable edges are shared out over kUnits translation units by their
+// rank, so that they compile in parallel.
+constexpr int kUnits = 8;
+constexpr int rank_of(int L) {
+  int r = 0;
+  for (int n = 2; n < L; ++n) r += smooth(n);
+  return r;
+}
+template <int UNIT, int L>
+void pick(int want, int dir, int kind, PencilKernel& k) {
+  if constexpr (smooth(L) && rank_of(L) % kUnits == UNIT)
+    if (L == want) k = entry_of<L>(dir, kind);
+}
+template <int UNIT, int... I>
+PencilKernel unit_kernel(int L, int dir, int kind, std::integer_sequence<int, I...>) {
+  PencilKernel k;
+  (pick<UNIT, I>(L, dir, kind, k), ...);
+  return k;
+}
+template <int UNIT>
+PencilKernel unit_kernel(int L, int dir, int kind) {
+  return unit_kernel<UNIT>(L, dir, kind, std::make_integer_sequence<int, kAxisMaxLen + 1>{});
+}
+
+}  // namespace pc
+}  // namespace fft3d

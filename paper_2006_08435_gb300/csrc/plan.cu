@@ -304,15 +304,8 @@ struct fft3d_plan_s {
   // device buffers shared by the units (owned)
   long long* d_off = nullptr;
   unsigned* d_status = nullptr;
-  // general path (variant kGeneralVariant): one pass per axis over chunks of
-  // `chunk` grids (the last chunk `tail` grids); pass[axis][0] for a full
-  // chunk, pass[axis][1] for the tail
-  bool general = false;
-  std::vector<AxisTable> tables;
-  AxisLaunch pass[3][2];
-  bool xy_fused = false;  // x and y in one plane pass (the plane fits shared memory)
-  PlaneLaunch plane[2];
-  int chunk = 0, nchunks = 0, tail = 0;
+  bool general = false;  // variant kGeneralVariant
+  AxisPasses passes;
 };
 
 namespace {
@@ -346,12 +339,7 @@ void free_plan_buffers(fft3d_plan p) {
   p->side.clear();
   p->join.clear();
   p->fork = nullptr;
-  for (AxisTable& t : p->tables) {
-    cudaFree(t.d_tw);
-    cudaFree(t.d_pos);
-    t.d_tw = nullptr;
-    t.d_pos = nullptr;
-  }
+  p->passes.destroy();
 }
 
 int check_device() {
@@ -529,23 +517,11 @@ int validate_common(int precision, int direction, int norm, fft3d_plan* out_plan
   return FFT3D_SUCCESS;
 }
 
-// General path: per chunk of grids, the x pass (in -> out), then y and z in
-// place on out; a chunk's intermediate (at most 40% of L2 when the grids
-// allow) stays in L2 between its passes.
+// General path (passes.cu): x, y, z passes over chunks of grids.
 int launch_general(fft3d_plan p, const float2* in, float2* out, cudaStream_t stream) {
-  const long long grid_pts = (long long)p->nx * p->ny * p->nz;
-  for (int c = 0; c < p->nchunks; ++c) {
-    const int w = (c == p->nchunks - 1 && p->tail != p->chunk) ? 1 : 0;
-    const long long off = (long long)c * p->chunk * grid_pts;
-    const bool xy_ok =
-        p->xy_fused
-            ? launch_plane_pass(p->plane[w], in + off, out + off, stream) == cudaSuccess
-            : launch_axis_pass(p->pass[0][w], in + off, out + off, stream) == cudaSuccess &&
-                  launch_axis_pass(p->pass[1][w], out + off, out + off, stream) == cudaSuccess;
-    if (!xy_ok || launch_axis_pass(p->pass[2][w], out + off, out + off, stream) != cudaSuccess) {
-      cudaGetLastError();
-      return FFT3D_ERR_CUDA;
-    }
+  if (p->passes.execute(in, out, nullptr, stream) != cudaSuccess) {
+    cudaGetLastError();
+    return FFT3D_ERR_CUDA;
   }
   return FFT3D_SUCCESS;
 }
@@ -629,90 +605,13 @@ int launch(fft3d_plan p, const float2* in, float2* out, const float2* const* in_
   return FFT3D_SUCCESS;
 }
 
-// W_L^m = exp(-2 pi i m / L), m < L, evaluated in FP64 by the host math
-// library and rounded to nearest FP32: the twiddle table of the general
-// path's passes.
-void root_table(int L, float* out /* 2 * L */) {
-  for (int m = 0; m < L; ++m) {
-    const double a = 2.0 * 3.14159265358979323846 * (double)m / (double)L;
-    out[2 * m] = (float)std::cos(a);
-    out[2 * m + 1] = (float)(-std::sin(a));
-  }
-}
-
-// Plan of the general path: tables for each distinct edge, chunking by the
-// L2 budget, the three passes prepared for a full chunk and for the tail.
+// Plan of the general path.
 int create_general(fft3d_plan p) {
-  int rc;
-  const int lens[3] = {p->nx, p->ny, p->nz};
-  int tab_of[3];
-  for (int a = 0; a < 3; ++a) {
-    tab_of[a] = -1;
-    for (size_t t = 0; t < p->tables.size(); ++t)
-      if (p->tables[t].L == lens[a]) tab_of[a] = (int)t;
-    if (tab_of[a] >= 0) continue;
-    AxisTable t;
-    t.L = lens[a];
-    t.nst = axis_stages(t.L, t.radix);
-    if (!t.nst) return FFT3D_ERR_UNSUPPORTED_SIZE;
-    std::vector<float> tw(2 * (size_t)t.L);
-    root_table(t.L, tw.data());
-    std::vector<int> pos(t.L);
-    axis_positions(t.L, t.nst, t.radix, pos.data());
-    std::vector<unsigned short> pos16(pos.begin(), pos.end());
-    p->tables.push_back(t);
-    AxisTable& tt = p->tables.back();
-    if ((rc = upload(&tt.d_tw, reinterpret_cast<const float2*>(tw.data()), (size_t)t.L))) return rc;
-    if ((rc = upload(&tt.d_pos, pos16.data(), pos16.size()))) return rc;
-    tab_of[a] = (int)p->tables.size() - 1;
-  }
-  int sms = 0, l2_bytes = 0;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device) != cudaSuccess ||
-      cudaDeviceGetAttribute(&l2_bytes, cudaDevAttrL2CacheSize, p->device) != cudaSuccess)
+  int l2_bytes = 0;
+  if (cudaDeviceGetAttribute(&l2_bytes, cudaDevAttrL2CacheSize, p->device) != cudaSuccess)
     return FFT3D_ERR_CUDA;
-  const long long nx = p->nx, ny = p->ny, nz = p->nz;
-  const double grid_bytes = 8.0 * (double)(nx * ny * nz);
-  long long chunk = (long long)(0.4 * (double)l2_bytes / grid_bytes);
-  // a pass's tile count stays below 2^31 (every pass has fewer tiles than
-  // pencils, at most max(ny nz, nz nx, ny nx) per grid)
-  const long long cap = std::max(1LL, (1LL << 30) / std::max({ny * nz, nz * nx, ny * nx}));
-  chunk = std::max(1LL, std::min({chunk, (long long)p->batch, cap}));
-  p->chunk = (int)chunk;
-  p->nchunks = (int)((p->batch + chunk - 1) / chunk);
-  // x and y in one pass where a plane fits shared memory and holds enough
-  // points for a block's iteration (measured: 64^3 x 256 0.20 -> 0.24,
-  // 96 x 128 x 64 0.19 -> 0.24 of the roofline; 16^3 planes of 256 points
-  // 0.22 -> 0.09, so small planes keep the separate passes' larger tiles)
-  p->xy_fused = (long long)p->nx * p->ny >= 4096 && plane_pass_smem(p->nx, p->ny) != 0;
-  p->tail = p->batch - (p->nchunks - 1) * p->chunk;
-  for (int w = 0; w < 2; ++w) {
-    const long long c = w == 0 ? p->chunk : p->tail;
-    AxisGeom gx, gy, gz;
-    gx.contiguous = 1;
-    gx.rows = c * ny * nz;
-    gy.outer = c * nz;  // (grid, z) slices: base = outer * ny * nx
-    gy.nx = (int)nx;
-    gy.d1 = 1;
-    gy.s1 = ny * nx;
-    gy.pi = nx;
-    gz.outer = c * ny;  // (grid, y) slices: base = grid * nz ny nx + y nx
-    gz.nx = (int)nx;
-    gz.d1 = (int)ny;
-    gz.s1 = nz * ny * nx;
-    gz.s0 = nx;
-    gz.pi = nx * ny;
-    gz.scale = p->scale;
-    gz.do_scale = p->do_scale;
-    const AxisGeom* gs[3] = {&gx, &gy, &gz};
-    for (int a = p->xy_fused ? 2 : 0; a < 3; ++a)
-      if ((rc = prepare_axis_pass(p->tables[tab_of[a]], p->direction, *gs[a], sms, &p->pass[a][w])))
-        return rc;
-    if (p->xy_fused &&
-        (rc = prepare_plane_pass(p->tables[tab_of[0]], p->tables[tab_of[1]], p->direction, c * nz,
-                                 sms, &p->plane[w])))
-      return rc;
-  }
-  return FFT3D_SUCCESS;
+  return p->passes.create(kPassC2C, p->nx, p->ny, p->nz, p->batch, p->direction, p->scale,
+                          p->do_scale, l2_bytes);
 }
 
 // Validated arguments -> plan (variant < 0: environment override, tuning
