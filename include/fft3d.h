@@ -97,7 +97,8 @@ enum {
 int fft3d_size_supported(int n);
 
 /*
- * Host-only view of the general path's 1D plan for edge n (needs no GPU):
+ * Host-only mixed-radix plan of edge n (needs no GPU; a reference for
+ * digit-reversed layouts, the kernels transform in natural order):
  * the radices R_0 .. R_(s-1) (product n) of its decimation-in-frequency
  * stages, *nstages = s <= 12, and the digit-reversal map: after the stages
  * output K = k_0 + R_0 (k_1 + R_1 (k_2 + ...)), k_t < R_t, sits at position
@@ -287,12 +288,12 @@ int fft3d_selftest_wait_timeout(int64_t timeout_ns);
  * multiprocessor), with the buffer requirements of the tensor-TMA FP32
  * variants; the block-floating-point and FP8 kinds exist on 9 only.  10:
  * the general path (every plan that is not cubic with a fused edge;
- * selectable for those too): per chunk of grids that fits 40% of L2, the x
- * pass (in -> out) and the y and z passes in place on out, each a batched
- * 1D transform of the pencils of one axis in shared-memory tiles (mixed
- * radices 2, 3, 4, 5, 6, 8, 9, 10, 12, 15, 16; fft3d_axis_digit_map);
- * where a plane of at least 4096 points fits shared memory, x and y run as
- * one plane pass (two launches per chunk instead of three).  Mixed plans:
+ * selectable for those too): per chunk of grids that fits L2, the x pass
+ * (in -> out) and the y and z passes in place on out, each a batched 1D
+ * transform of the pencils of one axis, split into two register codelets;
+ * the launches of a batch above 40 MB alternate between the caller's stream
+ * and a side stream of the plan, forked and joined by events (in a captured
+ * graph, parallel branches). Mixed plans:
  * 0 one launch of the mixed-edge kernel, 1 one launch per distinct edge (the
  * tensor-TMA kernels of 128^3 and 32^3 .. 96^3 take one pair of
  * tensor maps per grid, up to 32 grids of an edge; an edge whose default is
@@ -437,10 +438,13 @@ int fft3d_complex_to_real(const void* in, float* re, int64_t count, void* stream
  * block transforms a whole grid, at 64 and 128 one pass runs over the real
  * grids and one over the half spectra; each grid's error is relative to
  * itself.
- * Elsewhere two grids of the batch share one complex transform (c = a + i b;
- * the pair is separated with the symmetry above), so a grid's rounding error
- * is relative to the larger of its pair; cost per pair: a packing pass, one
- * complex transform of the plan's precision, a separating pass.
+ * At the other edges above 2 they run in FP32 as one pass per axis (x on real
+ * rows, y and z on the half spectra), each grid on its own as well.  At n = 2
+ * and in the tensor-core precisions two grids of the batch share one complex
+ * transform (c = a + i b; the pair is separated with the symmetry above), so
+ * a grid's rounding error is relative to the larger of its pair; cost per
+ * pair: a packing pass, one complex transform of the plan's precision, a
+ * separating pass.
  * ---------------------------------------------------------------------------
  */
 typedef struct fft3d_real_plan_s* fft3d_real_plan;
@@ -457,8 +461,11 @@ typedef struct fft3d_real_plan_s* fft3d_real_plan;
  * Validates its arguments before touching the GPU.  Owns its device memory,
  * allocated here and freed by fft3d_real_plan_destroy: at n = 64 and 128
  * in FP32 a schedule, counters and (forward) batch * n * n/2 complex64
- * points of workspace, at n = 16 and 32 a status word only; elsewhere a complex plan of ceil(batch/2) grids and a workspace
- * of ceil(batch/2) * n^3 complex64 points.  The environment variable
+ * points of workspace, at n = 16 and 32 a status word only; at the other
+ * edges above 2 in FP32 twiddle tables and (inverse) the half spectra of the
+ * grids in flight (about 75 MB, or two grids if those are larger); elsewhere
+ * a complex plan of ceil(batch/2) grids and a workspace of ceil(batch/2) *
+ * n^3 complex64 points.  The environment variable
  * FFT3D_REAL_PATH=pairs selects the pair scheme everywhere (for testing).
  */
 int fft3d_real_plan_create(int n, int batch, int precision, int direction, int norm,
@@ -469,10 +476,10 @@ int fft3d_real_plan_create(int n, int batch, int precision, int direction, int n
  * 16-byte aligned, not overlapping (forward: in = real grids, out = half
  * spectra; inverse: the other way round).  Asynchronous on `stream`,
  * allocates nothing, capturable in a CUDA graph (one kernel at n = 16 and
- * 32, a counter reset and one kernel at n = 64 and 128 in FP32; elsewhere a packing
- * or rebuilding kernel, the complex plan's launch, a separating or splitting
- * kernel).  A plan may run
- * on one stream at a time.
+ * 32, a counter reset and one kernel at n = 64 and 128 in FP32, one kernel
+ * per pass and chunk at the other edges; in the pair scheme a packing or
+ * rebuilding kernel, the complex plan's launch, a separating or splitting
+ * kernel).  A plan may run on one stream at a time.
  */
 int fft3d_real_execute(fft3d_real_plan plan, const void* in, void* out, void* stream);
 

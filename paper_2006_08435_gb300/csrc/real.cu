@@ -21,11 +21,15 @@
 // with half-length row transforms: at 16^3 and 32^3 a whole grid per block
 // (rwholegrid.cuh), at 64^3 and 128^3 two phases (rgrid.cuh: one pass over
 // the real grid and one over the half spectrum, a workspace of n^2/2
-// complex per grid for the Nyquist column of the forward transform); everywhere else the
-// pair scheme above, whose kernels here move data only (pack, separate,
-// rebuild, split) and whose transforms are the library's complex plans.
-// Packing two grids into one makes each grid's rounding error relative to
-// the larger of the pair.
+// complex per grid for the Nyquist column of the forward transform), at the
+// other edges above 2 as one pencil pass per axis (passes.cu): 24 bytes per
+// real point through L2 where the pair scheme moves about 60 and makes the
+// passes of a whole complex transform (96^3 x 32, forward + inverse 333 ->
+// 214 us, 100^3 x 16 286 -> 124, 20^3 x 500 373 -> 45).  The pair scheme
+// remains for n = 2 and the tensor-core precisions; its kernels here move
+// data only (pack, separate, rebuild, split) and its transforms are the
+// library's complex plans.  Packing two grids into one makes each grid's
+// rounding error relative to the larger of the pair.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -44,6 +48,9 @@ struct fft3d_real_plan_s {
   // pair scheme
   fft3d_plan inner = nullptr;  // complex plan of `pairs` n^3 grids
   float2* d_work = nullptr;    // pairs * n^3 complex points
+  // pencil passes (passes.cu); the inverse keeps a chunk of spectra in d_work
+  bool pencils = false;
+  fft3d::AxisPasses passes;
   // dedicated kernels (rgrid.cuh)
   bool fused = false;
   fft3d::KernelInfo kern;
@@ -295,6 +302,42 @@ int create_fused_real(int n, int batch, int direction, int norm, const KernelInf
   return FFT3D_SUCCESS;
 }
 
+// Plan of the pencil passes: every even edge above 2 without a dedicated kernel.
+int create_pencil_real(int n, int batch, int direction, int norm, fft3d_real_plan* out_plan) {
+  int dev = -1, l2 = 0, major = 0, minor = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess) {
+    cudaGetLastError();
+    return FFT3D_ERR_NO_DEVICE;
+  }
+  if (major != 10 || minor != 3) return FFT3D_ERR_NO_DEVICE;
+  auto* p = new (std::nothrow) fft3d_real_plan_s();
+  if (!p) return FFT3D_ERR_ALLOC;
+  p->n = n;
+  p->batch = batch;
+  p->direction = direction;
+  p->pencils = true;
+  set_real_norm(p, norm, n);
+  const bool fwd = direction == FFT3D_FORWARD;
+  int rc = p->passes.create(fwd ? kPassR2C : kPassC2R, n, n, n, batch, fwd ? -1 : 1, p->scale,
+                            p->do_scale, l2);
+  if (!rc && !fwd &&
+      cudaMalloc(&p->d_work, sizeof(float2) * (size_t)p->passes.work_points()) != cudaSuccess) {
+    cudaGetLastError();
+    p->d_work = nullptr;
+    rc = FFT3D_ERR_ALLOC;
+  }
+  if (rc) {
+    p->passes.destroy();
+    delete p;
+    return rc;
+  }
+  *out_plan = p;
+  return FFT3D_SUCCESS;
+}
+
 int execute_fused_real(fft3d_real_plan p, const void* in, void* out, cudaStream_t s) {
   if (p->kern.uses_work &&
       cudaMemsetAsync(p->d_count, 0, sizeof(unsigned) * (size_t)(p->batch + 1), s) != cudaSuccess) {
@@ -339,6 +382,8 @@ int fft3d_real_plan_create(int n, int batch, int precision, int direction, int n
     const fft3d::KernelInfo k = fft3d::real_kernel_info(n, direction == FFT3D_FORWARD ? -1 : 1);
     if (k.launch) return fft3d::create_fused_real(n, batch, direction, norm, k, out_plan);
   }
+  if (precision == FFT3D_FP32 && !pairs_only && n > 2)
+    return fft3d::create_pencil_real(n, batch, direction, norm, out_plan);
   const int pairs = (batch + 1) / 2;
   fft3d_plan inner = nullptr;
   int rc = fft3d_plan_create(n, n, n, pairs, precision, direction, norm, &inner);
@@ -370,6 +415,13 @@ int fft3d_real_execute(fft3d_real_plan plan, const void* in, void* out, void* st
   if (!aligned16(in) || !aligned16(out)) return FFT3D_ERR_MISALIGNED;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (plan->fused) return execute_fused_real(plan, in, out, s);
+  if (plan->pencils) {
+    if (plan->passes.execute(in, out, plan->d_work, s) != cudaSuccess) {
+      cudaGetLastError();
+      return FFT3D_ERR_CUDA;
+    }
+    return FFT3D_SUCCESS;
+  }
   const int n = plan->n, batch = plan->batch, pairs = plan->pairs;
   const int q = n * n * n / 4, h = n / 2 + 1;
   if (plan->direction == FFT3D_FORWARD) {
@@ -395,11 +447,12 @@ int fft3d_real_execute(fft3d_real_plan plan, const void* in, void* out, void* st
 
 int fft3d_real_get_device_status(fft3d_real_plan plan, void* stream) {
   if (!plan) return FFT3D_ERR_NULL_PTR;
-  if (!plan->fused) return fft3d_get_device_status(plan->inner, stream);
+  if (plan->inner) return fft3d_get_device_status(plan->inner, stream);
   if (cudaStreamSynchronize(static_cast<cudaStream_t>(stream)) != cudaSuccess) {
     cudaGetLastError();
     return FFT3D_ERR_CUDA;
   }
+  if (plan->pencils) return FFT3D_SUCCESS;  // no waits between blocks
   unsigned st = 0;
   if (cudaMemcpy(&st, plan->d_status, sizeof(unsigned), cudaMemcpyDeviceToHost) != cudaSuccess ||
       cudaMemset(plan->d_status, 0, sizeof(unsigned)) != cudaSuccess)
@@ -415,6 +468,11 @@ int fft3d_real_plan_destroy(fft3d_real_plan plan) {
     return FFT3D_SUCCESS;
   }
   cudaFree(plan->d_work);
+  if (plan->pencils) {
+    plan->passes.destroy();
+    delete plan;
+    return FFT3D_SUCCESS;
+  }
   const int rc = fft3d_plan_destroy(plan->inner);
   delete plan;
   return rc;
