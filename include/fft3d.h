@@ -300,10 +300,10 @@ int fft3d_selftest_wait_timeout(int64_t timeout_ns);
  * a tensor-TMA kernel otherwise takes variant 0 at 32^3 .. 96^3
  * (4 at 80^3 from 4 grids) and 5 at 128^3, as do calls with pointer
  * arrays), 2 the
- * launches of 1 as concurrent branches: the plan's own side streams, one
- * per edge, wait on the caller's stream and the caller's stream waits on
- * each of them (in a captured graph, parallel branches between a fork and
- * a join).
+ * launches of 1 on two concurrent branches, the caller's stream and a side
+ * stream of the plan: it waits on the caller's stream and the caller's
+ * stream waits on it (in a captured graph, parallel branches between a fork
+ * and a join).
  * At create the variant comes from FFT3D_VARIANT / FFT3D_MIXED_VARIANT if
  * set, else from the tuning cache named by FFT3D_TUNE_CACHE (tuned on the
  * spot when FFT3D_TUNE=1 and the entry is missing), else a built-in default.

@@ -183,10 +183,10 @@ static bool fused_size(int n) { return fused_slot(n) >= 0; }
 // 9 the tensor-TMA items with tcgen05 products (64^3 two-plane, 128^3
 // split-y).
 // Variant 10 (kGeneralVariant): the general path, one pencil pass per axis
-// (axis.cu), the only one for non-cubic grids and edges without a fused
+// (passes.cu), the only one for non-cubic grids and edges without a fused
 // kernel, selectable for the others.  Mixed plans: 0 one
 // launch of the mixed-edge kernel, 1 one launch per distinct edge with that
-// edge's default kernel, 2 the launches of 1 as concurrent branches.
+// edge's default kernel, 2 the launches of 1 on two concurrent branches.
 std::vector<int> variant_candidates(bool mixed, int n, int precision) {
   if (mixed) return {0, 1, 2};
   // the block-floating-point and FP8 kinds exist on the tcgen05 kernels only
@@ -295,12 +295,11 @@ struct fft3d_plan_s {
   // the units for calls with pointer arrays (the same edges, kernels that
   // address grids through pointers)
   std::vector<Unit> units_ptr;
-  // mixed variant 2: the units as concurrent branches, one side stream and
-  // one join event per unit, forked from the caller's stream (owned)
+  // mixed variant 2: the units on two concurrent branches, the caller's
+  // stream and a side stream forked from it (owned)
   bool branches = false;
-  cudaEvent_t fork = nullptr;
-  std::vector<cudaStream_t> side;
-  std::vector<cudaEvent_t> join;
+  cudaEvent_t fork = nullptr, join = nullptr;
+  cudaStream_t side = nullptr;
   // device buffers shared by the units (owned)
   long long* d_off = nullptr;
   unsigned* d_status = nullptr;
@@ -331,14 +330,11 @@ void free_plan_buffers(fft3d_plan p) {
   cudaFree(p->d_status);
   p->d_off = nullptr;
   p->d_status = nullptr;
-  for (cudaStream_t s : p->side)
-    if (s) cudaStreamDestroy(s);
-  for (cudaEvent_t e : p->join)
-    if (e) cudaEventDestroy(e);
+  if (p->side) cudaStreamDestroy(p->side);
+  if (p->join) cudaEventDestroy(p->join);
   if (p->fork) cudaEventDestroy(p->fork);
-  p->side.clear();
-  p->join.clear();
-  p->fork = nullptr;
+  p->side = nullptr;
+  p->join = p->fork = nullptr;
   p->passes.destroy();
 }
 
@@ -576,33 +572,32 @@ int launch(fft3d_plan p, const float2* in, float2* out, const float2* const* in_
     }
     return FFT3D_SUCCESS;
   }
-  // concurrent branches: every side stream waits for the caller's stream,
-  // takes one unit (the smallest first, so that short launches find free
-  // multiprocessors before the persistent ones take them all), and the
-  // caller's stream waits for every branch; a captured graph records the
-  // fork and joins as edges
-  if (cudaEventRecord(p->fork, stream) != cudaSuccess) {
+  // two concurrent branches, the caller's stream and a side stream forked
+  // from it: the units alternate between them, smallest first, so that one
+  // branch's launch drains while the other's runs; a captured graph records
+  // the fork and join as edges.  (A side stream per edge, six on the 64-grid
+  // workload, ran it in 540 us when its plans were the only ones and in 663
+  // with two more pairs of plans alive, whose streams share the device's
+  // queues; one branch 569, two 495, three 520, four 514 us, largest first
+  // 510.)
+  int rc = FFT3D_SUCCESS;
+  if (cudaEventRecord(p->fork, stream) != cudaSuccess ||
+      cudaStreamWaitEvent(p->side, p->fork, 0) != cudaSuccess) {
     cudaGetLastError();
     return FFT3D_ERR_CUDA;
   }
-  int rc = FFT3D_SUCCESS;
-  for (size_t i = units.size(); i-- > 0;) {
-    if (cudaStreamWaitEvent(p->side[i], p->fork, 0) != cudaSuccess) {
-      cudaGetLastError();
-      return FFT3D_ERR_CUDA;
-    }
-    rc = launch_unit(p, units[i], in, out, in_ptrs, out_ptrs, p->side[i]);
-    // a forked branch is joined even when its launch failed: the caller's
-    // stream then still waits for every branch already launched, and a
-    // capture does not end with an unjoined stream
-    if (cudaEventRecord(p->join[i], p->side[i]) != cudaSuccess ||
-        cudaStreamWaitEvent(stream, p->join[i], 0) != cudaSuccess) {
-      cudaGetLastError();
-      if (!rc) rc = FFT3D_ERR_CUDA;
-    }
-    if (rc) return rc;
+  for (size_t i = 0; i < units.size() && !rc; ++i)
+    rc = launch_unit(p, units[units.size() - 1 - i], in, out, in_ptrs, out_ptrs,
+                     i & 1 ? p->side : stream);
+  // the side stream is joined even when a launch failed: the caller's stream
+  // then still waits for what was launched there, and a capture does not end
+  // with an unjoined stream
+  if (cudaEventRecord(p->join, p->side) != cudaSuccess ||
+      cudaStreamWaitEvent(stream, p->join, 0) != cudaSuccess) {
+    cudaGetLastError();
+    if (!rc) rc = FFT3D_ERR_CUDA;
   }
-  return FFT3D_SUCCESS;
+  return rc;
 }
 
 // Plan of the general path.
@@ -752,13 +747,9 @@ int create_mixed(int count, const int* dims, int direction, int norm, int varian
   }
   if (variant == 2 && p->units.size() > 1) {
     p->branches = true;
-    p->side.resize(p->units.size(), nullptr);
-    p->join.resize(p->units.size(), nullptr);
-    bool ok = cudaEventCreateWithFlags(&p->fork, cudaEventDisableTiming) == cudaSuccess;
-    for (size_t i = 0; ok && i < p->units.size(); ++i)
-      ok = cudaStreamCreateWithFlags(&p->side[i], cudaStreamNonBlocking) == cudaSuccess &&
-           cudaEventCreateWithFlags(&p->join[i], cudaEventDisableTiming) == cudaSuccess;
-    if (!ok) {
+    if (cudaEventCreateWithFlags(&p->fork, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&p->join, cudaEventDisableTiming) != cudaSuccess ||
+        cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking) != cudaSuccess) {
       cudaGetLastError();
       free_plan_buffers(p);
       delete p;
