@@ -203,16 +203,12 @@ std::vector<int> variant_candidates(bool mixed, int n, int precision) {
 }
 
 // The fastest variant measured on the GB300 for each edge and batch
-// (back-to-back executes; one grid also with L2 flushed):
+// (back-to-back executes):
 //   16^3: cluster-fused below 128 grids, whole grid per block from 128;
-//   32^3: cluster-fused below 128 grids, thread pairs from 128;
-//   48^3: plain persistent below 32 grids, thread pairs from 32;  80^3:
-//     plain persistent for one grid, the
-//     double-buffered persistent kernel from 4, the thread-pair kernel from
-//     8;  96^3: plain persistent below 4 grids, the thread-pair kernel from 4;
-//   64^3: warp-owned for one grid, the persistent kernel with twice the
-//     threads below 16, thread-per-pencil below 64, two-plane from 64;
-//   128^3: warp-owned for one grid, split-y from 2;
+//   32^3: cluster-fused below 48 grids, pencil passes below 300, thread pairs;
+//   48^3, 64^3, 80^3, 96^3, 128^3: pencil passes for few grids (below 36, 20,
+//     18, 8 and 3), then thread pairs (48, 80, 96), thread-per-pencil and from
+//     64 grids two-plane (64), split-y (128);
 //   tensor-core precisions: the plain persistent kernel (mma.sync) for few
 //     grids, the tcgen05 kernels from 16 (64^3) and 2 (128^3) grids.
 int builtin_default_variant(bool mixed, int n, int batch, int precision) {
@@ -230,22 +226,42 @@ int builtin_default_variant(bool mixed, int n, int batch, int precision) {
     // the whole-grid kernel from 128 (x 256: 0.29 against 0.15; x 4096:
     // 0.53 against 0.17)
     case 16: return batch >= 128 ? 12 : 3;
-    // 32^3: the cluster-fused kernel (16 blocks per grid) below 128 grids
-    // (one grid, L2 flushed: 10.9 us against 11.9; 2-64 grids: 11.6-23.2 us
-    // against 13.0-26.6 for the persistent kernel), the thread-pair kernel
-    // (four-plane items of 32 KB) from 128 (x 256: 0.46; x 1024: 0.51)
+    // Pencil passes (three dependent launches) fill the GPU with small blocks
+    // where the ticket kernels' large items leave it idle; their 48 bytes
+    // per point through L2 lose to the two-phase kernels once those fill it.
+    // us, pencil passes / the kernels before:
+    // 32^3 x 16 8.9 / 10.5, x 32 13.1 / 12.2 (3), x 64 15.7 / 18.8, x 127 24.5 /
+    // 31.5, x 200 35.9 / 39.5 (13), x 400 67.6 / 66.5
+    case 32: return batch >= 300 ? 13 : batch >= 48 ? kGeneralVariant : 3;
+    // 48^3 x 1 8.9 / 11.8 (0), x 4 8.6 / 14.1, x 24 19.7 / 25.3, x 32 24.6 / 25.3
+    // (13), x 48 33.3 / 30.2
+    case 48: return batch >= 36 ? 13 : kGeneralVariant;
+    // 64^3 x 1 8.8 / 11.7 (5), x 4 12.2 / 18.4 (1), x 16 25.2 / 29.0 (7), x 24
+    // 35.1 / 33.8, x 48 68.3 / 61.6, x 64 89.1 / 77.0 (8)
+    case 64: return batch >= 64 ? 8 : batch >= 20 ? 7 : kGeneralVariant;
+    // 80^3 x 1 8.6 / 14.9 (0), x 4 15.7 / 25.1 (4), x 8 26.0 / 32.4 (13), x 16
+    // 48.1 / 52.2
+    case 80: return batch >= 18 ? 13 : kGeneralVariant;
+    // 96^3 x 1 12.6 / 17.1 (0), x 4 24.1 / 33.9 (13), x 6 30.8 / 35.0, x 8 43.1 /
+    // 42.7
+    case 96: return batch >= 8 ? 13 : kGeneralVariant;
+    // 128^3 x 1 17.0 / 20.9 (5), x 2 27.7 / 32.6 (6), x 3 42.4 / 40.3
+    case 128: return batch >= 3 ? 6 : kGeneralVariant;
+    default: return 0;
+  }
+}
+
+// The kernel of an edge's `batch` grids in a mixed plan, whose grids lie
+// anywhere in the buffers: the fastest of the kernels that address grids
+// through a map or per-grid tensor maps.
+static int unit_variant(int n, int batch) {
+  switch (n) {
+    case 16: return batch >= 128 ? 12 : 3;
     case 32: return batch >= 128 ? 13 : 3;
-    case 64: return batch == 1 ? 5 : batch < 16 ? 1 : batch < 64 ? 7 : 8;
-    // 80^3, 96^3: the thread-pair kernel from 8 (80) and 4 (96) grids (x 256:
-    // 0.57 / 0.62 of the roofline against 0.30 / 0.25; x 12-14: 0.41-0.43
-    // against 0.25-0.27); below, the double-buffered kernel (80) or the
-    // plain persistent one
+    case 48: return batch >= 32 ? 13 : 0;
+    case 64: return batch == 1 ? 5 : batch < 16 ? 1 : 0;
     case 80: return batch >= 8 ? 13 : batch >= 4 ? 4 : 0;
     case 96: return batch >= 4 ? 13 : 0;
-    // 48^3: the thread-pair kernel (two-plane items of 36 KB) from 32 grids
-    // (x 64: 0.39 against 0.28; x 256: 0.52 against 0.30), the plain kernel
-    // below
-    case 48: return batch >= 32 ? 13 : 0;
     case 128: return batch == 1 ? 5 : 6;
     default: return 0;
   }
@@ -718,20 +734,20 @@ int create_mixed(int count, const int* dims, int direction, int norm, int varian
       Unit u;
       for (int g = 0; g < count; ++g)
         if (p->dims[g] == n) u.grids.push_back(g);
-      // the edge's default kernel.  The tensor-map kernels read a packed
+      // the edge's kernel (unit_variant).  The tensor-map kernels read a packed
       // batch: at 128^3 the split-y kernel (6) takes one pair of tensor maps
       // per grid with the launch (up to kMixMaps grids) on packed buffers,
       // and calls with pointer arrays use the warp-owned kernel (5) in a
-      // unit of their own; at 64^3 (7, 8) the plain persistent kernel (0),
-      // as fast at the grid counts of a mixed batch
+      // unit of their own; at 64^3 no tensor-map kernel is used,
+      // the plain persistent ones are as fast at a mixed batch's grid counts
       const int ng = (int)u.grids.size();
-      int v = builtin_default_variant(false, n, ng, FFT3D_FP32);
+      int v = unit_variant(n, ng);
       // the tensor-map kernels with per-grid maps: split-y (128^3) and the
       // thread-pair kernel (80^3, 96^3); for pointer arrays a kernel that
       // addresses grids through the plan's map
       const bool maps = (v == 6 || v == 13) && ng <= kMixMaps;
       const int v_ptr = n == 128 ? 5 : (n == 80 && ng >= 4) ? 4 : n == 32 ? 3 : 0;
-      if ((n == 64 && (v == 7 || v == 8)) || ((v == 6 || v == 13) && !maps)) v = n == 64 ? 0 : v_ptr;
+      if ((v == 6 || v == 13) && !maps) v = v_ptr;
       u.kernel = fused_kernel_info(n, direction, v);
       Unit w = u;
       if (maps) {
