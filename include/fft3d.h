@@ -472,6 +472,15 @@ int fft3d_real_plan_create(int n, int batch, int precision, int direction, int n
                            fft3d_real_plan* out_plan);
 
 /*
+ * As fft3d_real_plan_create with FFT3D_FORWARD and FFT3D_NORM_NONE in FP32,
+ * for spectra whose bits must not depend on the library's choice of kernel:
+ * the dedicated kernels at n = 16, 32, 64 and 128, elsewhere the pair scheme
+ * over complex transforms of one fixed arithmetic order.  The Hartree energy,
+ * which is returned in FP64, is taken from these.
+ */
+int fft3d_real_plan_create_fixed(int n, int batch, fft3d_real_plan* out_plan);
+
+/*
  * Transform every grid of the plan.  `in` and `out` are DEVICE pointers,
  * 16-byte aligned, not overlapping (forward: in = real grids, out = half
  * spectra; inverse: the other way round).  Asynchronous on `stream`,

@@ -2,7 +2,7 @@
 // with prime factors 2, 3, 5: the passes of the general path (the 1D FFTs
 // along x, then y, then z of the paper's section "Approach").
 //
-// L = A * B, both register codelets (B >= A as close as they come).  With
+// L = A * B, both register codelets.  With
 // n = n1 + A n2 and k = k2 + B k1:
 //   phase 1: thread (pencil, n1) loads the B points n1 + A n2 straight from
 //            global memory into registers, DFT_B, times W_L^(n1 k2), to
@@ -61,18 +61,38 @@ constexpr bool smooth(int n) {
   while (n % 5 == 0) n /= 5;
   return n == 1;
 }
+// Lengths of a step's transform in registers (transform below).
 constexpr bool codelet(int r) {
   return r == 1 || r == 2 || r == 3 || r == 4 || r == 5 || r == 6 || r == 8 || r == 9 || r == 10 ||
          r == 12 || r == 15 || r == 16 || r == 18 || r == 20 || r == 24 || r == 25 || r == 27 ||
-         r == 32;
+         r == 30 || r == 32;
 }
-// The smaller factor A of the split; B = L / A.  Strided pencils of a
-// codelet's length stay in one thread (no exchange); rows are split from 8
-// points up so that the lanes of a warp share rows.
+// The factor A of the split; B = L / A.
+// Edges without a fused kernel: B is the first radix of the edge's mixed-radix
+// plan (fft3d_axis_digit_map: the largest of 16, 15, 12, 10, 9, 8, ...) where
+// the rest is a codelet (all but 486 and 500).  The sums, twiddles and order
+// are then those of the plan's decimation-in-frequency stages, and the bits
+// those of the stage-by-stage passes before: the Hartree energy is returned
+// in FP64 and keeps its value.
+// Fused edges and 512, whose Hartree spectra come from other kernels, and real
+// rows: the closest pair (64^3 x 4 12.2 us, with 16 * 4 16.8; 48^3 x 12 12.0,
+// with 16 * 3 16.2; 512^3 1060, with 16 * 2 * 16 1255).
+// Pencils of a codelet's length stay in one thread (no exchange), rows only
+// below 16 points (real ones up to 6): the lanes of a warp share longer ones.
+constexpr int first_radix(int L) {
+  const int radices[] = {16, 15, 12, 10, 9, 8, 6, 5, 4, 3, 2};
+  for (int r : radices)
+    if (L % r == 0) return r;
+  return 0;
+}
 constexpr int split_a(int L, int kind) {
-  if (codelet(L) && (kind == kStrided || L < 8)) return 1;
+  const bool real = kind == kR2C || kind == kC2R;
+  const bool closest = real || L == 16 || L == 32 || L == 48 || L == 64 || L == 80 || L == 96 || L == 512;
+  if (codelet(L) && L <= (real ? 6 : kind == kContig ? 15 : 32)) return 1;
+  int a = L / first_radix(L);
+  if (!closest && codelet(a)) return a;
   int best = 0;
-  for (int a = 1; a * a <= L; ++a)
+  for (a = 1; a * a <= L; ++a)
     if (L % a == 0 && codelet(a) && codelet(L / a)) best = a;
   return best;
 }
@@ -139,10 +159,50 @@ struct Cfg {
   static constexpr int OP = stage_pitch(L + 1, A == 1 ? 1 : B / 2 + 1);
   static constexpr size_t smem =
       sizeof(float2) * (size_t)(exchange + (staged ? W * OP : 0));
-  static constexpr int blocks = KIND == kStrided || KIND == kContig ? 65536 / (T * reg_budget(B)) : 1;
+  static constexpr int blocks = KIND == kStrided || KIND == kContig ? 65536 / (T * reg_budget(A > B ? A : B)) : 1;
   static_assert(A >= 1, "no split into two codelets");
   static_assert(KIND == kStrided || KIND == kContig || L <= 256, "real rows hold 2 L points");
 };
+
+// a * w (forward) or a * conj w, w a forward table twiddle.  The order of the
+// fused operations is written out: left to the compiler it differs from one
+// kernel to the next, and results are to keep their bits.
+template <int DIR>
+FFT3D_HD float2 twiddle(float2 a, float2 w) {
+  const float s = DIR < 0 ? w.y : -w.y;
+  return make_float2(fmaf(a.x, w.x, -(a.y * s)), fmaf(a.y, w.x, a.x * s));
+}
+
+// The R-point transform of a step.  Above 16 points (but 32, which only fused
+// edges and 512 have), R = R1 * R2 with R1 = first_radix(R): the two decimation-in-frequency stages of the mixed-radix
+// plan in registers, R1 points R2 apart, the twiddles W_R^(j k) as the table
+// has them, then R2 points.
+template <int R, int DIR>
+FFT3D_HD void transform(float2* v) {
+  if constexpr (R <= 16 || R == 32) {
+    DFT<R, DIR>::run(v);
+  } else {
+    constexpr int R1 = first_radix(R), R2 = R / R1;
+    float2 t[R2][R1];
+    static_for<0, R2>([&](auto J) {
+      constexpr int j = decltype(J)::value;
+      static_for<0, R1>([&](auto I) { t[j][decltype(I)::value] = v[j + R2 * decltype(I)::value]; });
+      DFT<R1, DIR>::run(t[j]);
+      static_for<1, R1>([&](auto K) {
+        constexpr int k = decltype(K)::value;
+        if constexpr (j > 0)
+          t[j][k] = twiddle<DIR>(t[j][k], make_float2((float)turn_cos(j * k, R), (float)-turn_sin(j * k, R)));
+      });
+    });
+    static_for<0, R1>([&](auto K) {
+      constexpr int k = decltype(K)::value;
+      float2 u[R2];
+      static_for<0, R2>([&](auto J) { u[decltype(J)::value] = t[decltype(J)::value][k]; });
+      DFT<R2, DIR>::run(u);
+      static_for<0, R2>([&](auto M) { v[k + R1 * decltype(M)::value] = u[decltype(M)::value]; });
+    });
+  }
+}
 
 __device__ __forceinline__ unsigned fdiv(unsigned n, FastDiv d) {
   return (unsigned)(((unsigned long long)__umulhi(n, d.mul) + n) >> d.shift);
@@ -273,20 +333,20 @@ __global__ void __launch_bounds__(Cfg<L, KIND>::T, Cfg<L, KIND>::blocks) pencil_
         u[j] = make_float2(s.x - t.y, s.y + t.x);
         m[j] = make_float2(s.x + t.y, t.x - s.y);
       }
-      DFT<B, DIR>::run(u);
+      transform<B, DIR>(u);
       if constexpr (A > 1) {
 #pragma unroll
         for (int k = 0; k < B; ++k)
-          sm[c * C::RP + k * C::AP + n1] = k ? cmul_tw<DIR>(u[k], __ldg(a.tw + k * A + n1)) : u[k];
+          sm[c * C::RP + k * C::AP + n1] = k ? twiddle<DIR>(u[k], __ldg(a.tw + k * A + n1)) : u[k];
         if (n1 != 0 && 2 * n1 != A) {
           float2 v[B];
 #pragma unroll
           for (int j = 0; j < B; ++j) v[j] = m[B - 1 - j];
-          DFT<B, DIR>::run(v);
+          transform<B, DIR>(v);
           const int n2 = A - n1;
 #pragma unroll
           for (int k = 0; k < B; ++k)
-            sm[c * C::RP + k * C::AP + n2] = k ? cmul_tw<DIR>(v[k], __ldg(a.tw + k * A + n2)) : v[k];
+            sm[c * C::RP + k * C::AP + n2] = k ? twiddle<DIR>(v[k], __ldg(a.tw + k * A + n2)) : v[k];
         }
       } else {
         float2* dst = a.out + base(p, false);
@@ -304,11 +364,11 @@ __global__ void __launch_bounds__(Cfg<L, KIND>::T, Cfg<L, KIND>::blocks) pencil_
       float2 v[B];
 #pragma unroll
       for (int j = 0; j < B; ++j) v[j] = ldg(src + j * step, pin);
-      DFT<B, DIR>::run(v);
+      transform<B, DIR>(v);
       if constexpr (A > 1) {
 #pragma unroll
         for (int k = 0; k < B; ++k) {
-          const float2 y = k ? cmul_tw<DIR>(v[k], __ldg(a.tw + k * A + n1)) : v[k];
+          const float2 y = k ? twiddle<DIR>(v[k], __ldg(a.tw + k * A + n1)) : v[k];
           sm[KIND == kStrided ? (k * A + n1) * W + c : c * C::RP + k * C::AP + n1] = y;
         }
       } else if constexpr (KIND == kR2C) {
@@ -338,7 +398,7 @@ __global__ void __launch_bounds__(Cfg<L, KIND>::T, Cfg<L, KIND>::blocks) pencil_
 #pragma unroll
       for (int j = 0; j < A; ++j)
         v[j] = sm[KIND == kStrided ? (k2 * A + j) * W + c : c * C::RP + k2 * C::AP + j];
-      DFT<A, DIR>::run(v);
+      transform<A, DIR>(v);
       if constexpr (KIND == kR2C) {
         float2* row = C::staged ? sm + C::exchange + c * C::OP : a.out + base(p, false);
         // the mirrors of this item's outputs are those of B - k2
@@ -348,7 +408,7 @@ __global__ void __launch_bounds__(Cfg<L, KIND>::T, Cfg<L, KIND>::blocks) pencil_
           float2 w[A];
 #pragma unroll
           for (int j = 0; j < A; ++j) w[j] = sm[c * C::RP + (B - k2) * C::AP + j];
-          DFT<A, DIR>::run(w);
+          transform<A, DIR>(w);
           split_store<L, A, C::staged>(a, row, v, w, k2, pout);
         }
       } else {

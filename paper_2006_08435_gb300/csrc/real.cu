@@ -366,6 +366,44 @@ int execute_fused_real(fft3d_real_plan p, const void* in, void* out, cudaStream_
 
 }  // namespace fft3d
 
+namespace fft3d {
+namespace {
+
+// Plan of the pair scheme around a complex plan of `pairs` grids.
+int create_pair_real(int n, int batch, int direction, fft3d_plan inner, fft3d_real_plan* out_plan) {
+  auto* p = new (std::nothrow) fft3d_real_plan_s();
+  if (!p) {
+    fft3d_plan_destroy(inner);
+    return FFT3D_ERR_ALLOC;
+  }
+  p->n = n;
+  p->batch = batch;
+  p->pairs = (batch + 1) / 2;
+  p->direction = direction;
+  p->inner = inner;
+  const size_t bytes = (size_t)p->pairs * n * n * n * sizeof(float2);
+  if (cudaMalloc(&p->d_work, bytes) != cudaSuccess) {
+    cudaGetLastError();
+    fft3d_plan_destroy(inner);
+    delete p;
+    return FFT3D_ERR_ALLOC;
+  }
+  *out_plan = p;
+  return FFT3D_SUCCESS;
+}
+
+// The complex kernel of fft3d_real_plan_create_fixed: at 48^3, 80^3 and 96^3
+// the persistent kernel, from as many pairs as first chosen the thread-pair
+// kernel (another arithmetic order); elsewhere the pencil passes, which have
+// the order of the passes before them (pencil.cuh: split_a).
+int fixed_variant(int n, int pairs) {
+  const int from = n == 48 ? 32 : n == 80 ? 8 : n == 96 ? 4 : 0;
+  return !from ? kGeneralVariant : pairs >= from ? 13 : n == 80 && pairs >= 4 ? 4 : 0;
+}
+
+}  // namespace
+}  // namespace fft3d
+
 extern "C" {
 
 int fft3d_real_plan_create(int n, int batch, int precision, int direction, int norm,
@@ -381,32 +419,33 @@ int fft3d_real_plan_create(int n, int batch, int precision, int direction, int n
   if (precision == FFT3D_FP32 && !pairs_only) {
     const fft3d::KernelInfo k = fft3d::real_kernel_info(n, direction == FFT3D_FORWARD ? -1 : 1);
     if (k.launch) return fft3d::create_fused_real(n, batch, direction, norm, k, out_plan);
+    if (n > 2) return fft3d::create_pencil_real(n, batch, direction, norm, out_plan);
   }
-  if (precision == FFT3D_FP32 && !pairs_only && n > 2)
-    return fft3d::create_pencil_real(n, batch, direction, norm, out_plan);
+  fft3d_plan inner = nullptr;
+  const int rc = fft3d_plan_create(n, n, n, (batch + 1) / 2, precision, direction, norm, &inner);
+  return rc ? rc : fft3d::create_pair_real(n, batch, direction, inner, out_plan);
+}
+
+int fft3d_real_plan_create_fixed(int n, int batch, fft3d_real_plan* out_plan) {
+  if (!out_plan) return FFT3D_ERR_NULL_PTR;
+  *out_plan = nullptr;
+  if (batch < 1 || batch > (1 << 24)) return FFT3D_ERR_INVALID_ARG;
+  if (n < 2 || (n & 1) || !fft3d_size_supported(n)) return FFT3D_ERR_UNSUPPORTED_SIZE;
+  const char* path = std::getenv("FFT3D_REAL_PATH");
+  const bool pairs_only = path && std::strcmp(path, "pairs") == 0;
+  const fft3d::KernelInfo k = fft3d::real_kernel_info(n, -1);
+  if (k.launch && !pairs_only)
+    return fft3d::create_fused_real(n, batch, FFT3D_FORWARD, FFT3D_NORM_NONE, k, out_plan);
+  // (a variant set in the environment or a tuning cache holds here too)
   const int pairs = (batch + 1) / 2;
   fft3d_plan inner = nullptr;
-  int rc = fft3d_plan_create(n, n, n, pairs, precision, direction, norm, &inner);
-  if (rc) return rc;
-  auto* p = new (std::nothrow) fft3d_real_plan_s();
-  if (!p) {
-    fft3d_plan_destroy(inner);
-    return FFT3D_ERR_ALLOC;
-  }
-  p->n = n;
-  p->batch = batch;
-  p->pairs = pairs;
-  p->direction = direction;
-  p->inner = inner;
-  const size_t bytes = (size_t)pairs * n * n * n * sizeof(float2);
-  if (cudaMalloc(&p->d_work, bytes) != cudaSuccess) {
-    cudaGetLastError();
-    fft3d_plan_destroy(inner);
-    delete p;
-    return FFT3D_ERR_ALLOC;
-  }
-  *out_plan = p;
-  return FFT3D_SUCCESS;
+  int rc;
+  if (k.launch || std::getenv("FFT3D_VARIANT") || std::getenv("FFT3D_TUNE_CACHE"))
+    rc = fft3d_plan_create(n, n, n, pairs, FFT3D_FP32, FFT3D_FORWARD, FFT3D_NORM_NONE, &inner);
+  else
+    rc = fft3d_internal_create_variant(false, n, pairs, FFT3D_FP32, FFT3D_FORWARD, nullptr, 0,
+                                       fft3d::fixed_variant(n, pairs), &inner);
+  return rc ? rc : fft3d::create_pair_real(n, batch, FFT3D_FORWARD, inner, out_plan);
 }
 
 int fft3d_real_execute(fft3d_real_plan plan, const void* in, void* out, void* stream) {

@@ -236,6 +236,19 @@ class RealPlan:
                 "fft3d_real_plan_create")
         self._h = h
 
+    @classmethod
+    def fixed(cls, n: int, batch: int = 1) -> "RealPlan":
+        """A forward FP32 plan whose spectra keep their bits from one version
+        of the kernels to the next (``fft3d_real_plan_create_fixed``)."""
+        p = cls.__new__(cls)
+        p.n, p.batch = int(n), int(batch)
+        p.precision, p.inverse, p.norm = "fp32", False, "none"
+        h = ctypes.c_void_p()
+        L.check(L.lib().fft3d_real_plan_create_fixed(p.n, p.batch, ctypes.byref(h)),
+                "fft3d_real_plan_create_fixed")
+        p._h = h
+        return p
+
     def _check(self, t: torch.Tensor, name: str, dtype, points: int) -> None:
         if not isinstance(t, torch.Tensor) or not t.is_cuda:
             raise ValueError(f"{name} must be a CUDA tensor")
@@ -354,15 +367,16 @@ _REAL_CACHE_MAX = 4
 _real_cache: "collections.OrderedDict" = collections.OrderedDict()
 
 
-def _get_real_plan(n, batch, precision, inverse, norm, dev, stream=None) -> RealPlan:
-    key = (n, batch, precision, bool(inverse), norm, dev, _stream_handle(stream))
+def _get_real_plan(n, batch, precision, inverse, norm, dev, stream=None, fixed=False) -> RealPlan:
+    key = (n, batch, precision, bool(inverse), norm, dev, _stream_handle(stream), fixed)
     with _cache_lock:
         p = _real_cache.get(key)
         if p is not None:
             _real_cache.move_to_end(key)
             return p
         with torch.cuda.device(dev):
-            p = RealPlan(n, batch, precision, inverse, norm)
+            p = (RealPlan.fixed(n, batch) if fixed
+                 else RealPlan(n, batch, precision, inverse, norm))
         _real_cache[key] = p
         while len(_real_cache) > _REAL_CACHE_MAX:
             _real_cache.popitem(last=False)
@@ -373,6 +387,10 @@ def rfft3d(x: torch.Tensor, norm: str = "none", precision: str = "fp32",
            out: torch.Tensor | None = None) -> torch.Tensor:
     """Half spectrum (..., n, n, n // 2 + 1) of the forward transform (Eq. 1)
     of real float32 CUDA grids (..., n, n, n); leading dims are a batch."""
+    return _rfft3d(x, norm, precision, out, False)
+
+
+def _rfft3d(x, norm, precision, out, fixed):
     if not isinstance(x, torch.Tensor) or not x.is_cuda or x.dtype != torch.float32:
         raise TypeError("x must be a float32 CUDA tensor")
     if x.dim() < 3 or not (x.shape[-1] == x.shape[-2] == x.shape[-3]):
@@ -387,7 +405,7 @@ def rfft3d(x: torch.Tensor, norm: str = "none", precision: str = "fp32",
     dev = x.device.index
     with _on_device(dev):
         stream = _current_stream_handle(dev)
-        p = _get_real_plan(n, batch, precision, False, norm, dev, stream)
+        p = _get_real_plan(n, batch, precision, False, norm, dev, stream, fixed)
         return p.execute(x, out, stream)
 
 

@@ -19,7 +19,7 @@ from __future__ import annotations
 import torch
 
 from . import _lib as L
-from .fft import _stream_handle, fft3d, irfft3d, rfft3d
+from .fft import _rfft3d, _stream_handle, fft3d, irfft3d
 
 _ws_cache: dict = {}
 
@@ -120,7 +120,8 @@ class HartreeEnergy(torch.autograd.Function):
         ctx.cell = float(cell)
         ctx.half = rho.shape[-1] % 2 == 0
         if ctx.half:
-            rhohat = rfft3d(rho.contiguous())
+            # (the energy is FP64: from a spectrum whose bits stay)
+            rhohat = _rfft3d(rho.contiguous(), "none", "fp32", None, True)
             ctx.save_for_backward(rhohat)
             return energy_from_half_spectrum(rhohat, cell)
         rhohat = fft3d(real_to_complex(rho))

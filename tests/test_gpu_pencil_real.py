@@ -70,3 +70,21 @@ def test_real_two_chains(cuda):
         q1.execute(f[b], refb[b])
     assert torch.equal(f, ref) and torch.equal(back, refb)
     assert oracle.rel_l2(back.cpu().numpy(), r.cpu().numpy()) <= TOL
+
+
+@pytest.mark.parametrize("n,batch", [(18, 3), (48, 5), (80, 9), (90, 2), (96, 8), (100, 1)])
+def test_fixed_spectra_and_the_energy_taken_from_them(cuda, n, batch):
+    """RealPlan.fixed against the oracle (pairs of grids of equal size, so the
+    same bar holds), and hartree_energy's value is bit for bit the one of its
+    spectrum."""
+    from paper_2006_08435_gb300 import RealPlan, hartree_energy
+    from paper_2006_08435_gb300.hartree import energy_from_half_spectrum
+    r = np.ascontiguousarray(synth.uniform_grids(n, batch, seed=n).real.astype(np.float32))
+    rd = torch.from_numpy(r).cuda()
+    f = torch.empty((batch, n, n, n // 2 + 1), dtype=torch.complex64, device="cuda")
+    p = RealPlan.fixed(n, batch)
+    p.execute(rd, f)
+    assert p.device_status() == 0
+    for b in (0, batch - 1):
+        assert oracle.rel_l2(f[b].cpu().numpy(), oracle.rdft3d(r[b].astype(np.float64))) <= TOL
+    assert torch.equal(hartree_energy(rd, 10.0), energy_from_half_spectrum(f, 10.0))

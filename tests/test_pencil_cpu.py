@@ -1,5 +1,5 @@
-"""The pencil passes' building blocks without a GPU: the register codelets
-they add, and the two-codelet split of every plannable edge, compiled as host
+"""The pencil passes' building blocks without a GPU: the register transforms
+of their steps, and the two-step split of every plannable edge, compiled as host
 code from the kernels' own headers and compared with numpy.fft."""
 import os
 import subprocess
@@ -7,7 +7,7 @@ import subprocess
 import numpy as np
 import pytest
 
-RADICES = [18, 20, 25, 27]
+RADICES = [16, 18, 20, 24, 25, 27, 30, 32]
 
 SRC = r"""
 #include <cmath>
@@ -20,7 +20,7 @@ void one() {
   float2 v[R];
   for (int n = 0; n < R; ++n)
     v[n] = make_float2((float)std::cos(0.7 * n + 0.3), (float)std::sin(1.3 * n - 0.2));
-  DFT<R, DIR>::run(v);
+  pc::transform<R, DIR>(v);
   std::printf("dft %d %d", R, DIR);
   for (int n = 0; n < R; ++n) std::printf(" %.9e %.9e", v[n].x, v[n].y);
   std::printf("\n");
@@ -31,7 +31,7 @@ void both() {
   one<R, 1>();
 }
 int main() {
-  both<18>(); both<20>(); both<25>(); both<27>();
+  both<16>(); both<18>(); both<20>(); both<24>(); both<25>(); both<27>(); both<30>(); both<32>();
   for (int n = 0; n <= kAxisMaxLen + 1; ++n)
     if (pc::smooth(n))
       std::printf("split %d %d %d %d\n", n, pc::split_a(n, pc::kStrided), pc::split_a(n, pc::kContig),
@@ -62,7 +62,7 @@ def host_output(tmp_path_factory):
     return subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout
 
 
-def test_codelets_of_the_pencil_passes(host_output):
+def test_transforms_of_the_steps(host_output):
     seen = 0
     for line in host_output.splitlines():
         f = line.split()
@@ -80,7 +80,7 @@ def test_codelets_of_the_pencil_passes(host_output):
     assert seen == 2 * len(RADICES)
 
 
-def test_every_plannable_edge_splits_into_two_codelets(host_output):
+def test_every_plannable_edge_splits_into_two_steps(host_output):
     edges = []
     for line in host_output.splitlines():
         f = line.split()
