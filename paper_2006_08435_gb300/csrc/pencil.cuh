@@ -39,7 +39,14 @@
 // of the even and odd samples, X[k] = E[k] + W_n^k O[k], k = 0 .. L.  The
 // split needs Z[k] and Z[L-k], which are outputs of the phase-2 items k2 and
 // B - k2: one thread takes both and splits in registers.  The inverse undoes
-// the split as it loads, one thread taking the points of n1 and A - n1.
+// the split as it starts, one thread taking the points of n1 and A - n1.
+// These rows are staged: copied in with cp.async and out as whole runs, at an
+// odd pitch, and the lanes of a warp are rows -- no bank conflicts, one n1 or
+// k2 (one branch of the split, one twiddle) per half-warp, where lanes along
+// the row took 5 to 8 short runs per access and both branches (10 grids of
+// 96^3: L1 wavefronts of the forward x pass 5.0 -> 2.9 M, 21.5 -> 15.6 us;
+// 96^3 x 32 forward 107 -> 93, inverse 106 -> 101 us; 100^3 x 16 64 -> 55, 60 ->
+// 59).  Complex rows do better without (256^3 x 4 419 us, staged 489).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -75,7 +82,8 @@ constexpr bool codelet(int r) {
 // those of the stage-by-stage passes before: the Hartree energy is returned
 // in FP64 and keeps its value.
 // Fused edges and 512, whose Hartree spectra come from other kernels, and real
-// rows: the closest pair (64^3 x 4 12.2 us, with 16 * 4 16.8; 48^3 x 12 12.0,
+// rows: the closest pair, the larger factor in the phase that holds one
+// transform per thread (64^3 x 4 12.2 us, with 16 * 4 16.8; 48^3 x 12 12.0,
 // with 16 * 3 16.2; 512^3 1060, with 16 * 2 * 16 1255).
 // Pencils of a codelet's length stay in one thread (no exchange), rows only
 // below 16 points (real ones up to 6): the lanes of a warp share longer ones.
@@ -94,7 +102,7 @@ constexpr int split_a(int L, int kind) {
   int best = 0;
   for (a = 1; a * a <= L; ++a)
     if (L % a == 0 && codelet(a) && codelet(L / a)) best = a;
-  return best;
+  return kind == kC2R ? L / best : best;
 }
 // Threads of a block: the multiple of 32 up to 512 that leaves the fewest
 // lanes idle over the two phases (n1 items of work w1, then n2 of w2), at
@@ -124,17 +132,6 @@ constexpr int tile_pencils(int L, int A) {
   return w;
 }
 
-// Pitch of staged rows of R points written by lanes that walk `run`
-// consecutive points of a row, then the next row: odd rows are packed (one
-// run of memory), even ones padded (to an even pitch: 16-byte copies) so
-// that the next row's banks follow on.
-constexpr int stage_pitch(int R, int run) {
-  if (R % 2) return R;
-  int p = R;
-  while (p % 16 != (run + 1) / 2 * 2 % 16) p += 2;
-  return p;
-}
-
 // Registers a thread may use (complex kinds), so that the compiler aims at
 // 32 warps and more: 256^3 x 4 419 -> 395, 100^3 x 16 102 -> 94 us.
 constexpr int reg_budget(int B) { return B <= 8 ? 48 : B <= 12 ? 56 : B <= 16 ? 64 : 96; }
@@ -142,23 +139,22 @@ constexpr int reg_budget(int B) { return B <= 8 ? 48 : B <= 12 ? 56 : B <= 16 ? 
 template <int L, int KIND>
 struct Cfg {
   static constexpr int A = split_a(L, KIND), B = L / A;
+  static constexpr bool REAL = KIND == kR2C || KIND == kC2R;
   static constexpr int W = tile_pencils(L, A);
   // items of the two phases (real rows: mirrored pairs where the split is)
   static constexpr int N1 = W * (KIND == kC2R && A > 1 ? A / 2 + 1 : A);
   static constexpr int N2 = A == 1 ? 0 : W * (KIND == kR2C ? B / 2 + 1 : B);
   static constexpr int T = block_threads(N1, KIND == kC2R ? 2 * B : B, N2, KIND == kR2C ? 2 * A : A);
   static constexpr int I1 = (N1 + T - 1) / T, I2 = (N2 + T - 1) / T;
-  // contiguous kinds: exchange slot of (pencil, k2, n1); odd pitch of k2
-  static constexpr int AP = A | 1, RP = B * AP;
+  // rows: exchange slot of (pencil, k2, n1), odd pitch of k2 (and of real rows)
+  static constexpr int AP = A | 1, RP = REAL ? B * AP | 1 : B * AP;
   static constexpr int exchange = A == 1 ? 0 : KIND == kStrided ? W * L : W * RP;
-  // Half spectra leave through shared memory, as packed rows of L + 1 points,
-  // where the direct stores' runs of B / 2 + 1 points would split most
-  // sectors: forward 96^3 (B = 8) 135 -> 117 us, 160^3 (B = 10) 76 -> 69,
-  // but 256^3 (B = 16) 129 -> 143.
-  static constexpr bool staged = KIND == kR2C && B <= 10;
-  static constexpr int OP = stage_pitch(L + 1, A == 1 ? 1 : B / 2 + 1);
-  static constexpr size_t smem =
-      sizeof(float2) * (size_t)(exchange + (staged ? W * OP : 0));
+  // real rows: points of a staged row in and out, odd pitch; one buffer (two
+  // for one-step rows, whose threads read and write it in the same phase)
+  static constexpr int IR = KIND == kC2R ? L + 1 : L, OR = KIND == kR2C ? L + 1 : L;
+  static constexpr int SP = (L + 1) | 1;
+  static constexpr int out_at = A == 1 ? W * SP : 0;
+  static constexpr size_t smem = sizeof(float2) * (size_t)(exchange + (REAL ? out_at + W * SP : 0));
   static constexpr int blocks = KIND == kStrided || KIND == kContig ? 65536 / (T * reg_budget(A > B ? A : B)) : 1;
   static_assert(A >= 1, "no split into two codelets");
   static_assert(KIND == kStrided || KIND == kContig || L <= 256, "real rows hold 2 L points");
@@ -174,9 +170,9 @@ FFT3D_HD float2 twiddle(float2 a, float2 w) {
 }
 
 // The R-point transform of a step.  Above 16 points (but 32, which only fused
-// edges and 512 have), R = R1 * R2 with R1 = first_radix(R): the two decimation-in-frequency stages of the mixed-radix
-// plan in registers, R1 points R2 apart, the twiddles W_R^(j k) as the table
-// has them, then R2 points.
+// edges and 512 have) R = R1 * R2 with R1 = first_radix(R): the two decimation-
+// in-frequency stages of the mixed-radix plan in registers, R1 points R2
+// apart, the twiddles W_R^(j k) as the table has them, then R2 points.
 template <int R, int DIR>
 FFT3D_HD void transform(float2* v) {
   if constexpr (R <= 16 || R == 32) {
@@ -227,26 +223,19 @@ __device__ __forceinline__ void stg(float2* p, float2 v, uint64_t pol) {
                ::"l"(p), "f"(v.x), "f"(v.y), "l"(pol) : "memory");
 }
 
-// `rows` consecutive rows of R points from pitch P in shared memory, packed
-// at g.  Even R: every row starts on 16 bytes (the grids do).  Odd R: the
-// packed run may start on 8 bytes.
-__device__ __forceinline__ void stg16(float2* g, const float2* s, float sc, uint64_t pol) {
-  float4 v = *reinterpret_cast<const float4*>(s);
-  asm volatile("st.global.L2::cache_hint.v4.f32 [%0], {%1, %2, %3, %4}, %5;"
-               ::"l"(g), "f"(v.x * sc), "f"(v.y * sc), "f"(v.z * sc), "f"(v.w * sc), "l"(pol) : "memory");
+// `rows` consecutive rows of R points, packed at g, to pitch P at s, and back.
+template <int R, int P, int T>
+__device__ __forceinline__ void rows_in(float2* s, const float2* g, int rows, uint64_t pol) {
+  for (int u = threadIdx.x; u < rows * R; u += T)
+    asm volatile("cp.async.ca.shared.global.L2::cache_hint [%0], [%1], 8, %2;"
+                 ::"r"((uint32_t)__cvta_generic_to_shared(s + u / R * P + u % R)), "l"(g + u), "l"(pol)
+                 : "memory");
+  asm volatile("cp.async.wait_all;" ::: "memory");
 }
 template <int R, int P, int T>
 __device__ __forceinline__ void rows_out(float2* g, const float2* s, int rows, float sc, uint64_t pol) {
-  if constexpr (R % 2 == 0) {
-    for (int u = threadIdx.x; u < rows * (R / 2); u += T)
-      stg16(g + 2 * u, s + u / (R / 2) * P + 2 * (u % (R / 2)), sc, pol);
-  } else if ((reinterpret_cast<uintptr_t>(g) & 15) == 0) {
-    const int n = rows * R;
-    for (int u = threadIdx.x; u < n / 2; u += T) stg16(g + 2 * u, s + 2 * u, sc, pol);
-    if ((n & 1) && threadIdx.x == 0) stg(g + n - 1, cscale(s[n - 1], sc), pol);
-  } else {
-    for (int u = threadIdx.x; u < rows * R; u += T) stg(g + u, cscale(s[u], sc), pol);
-  }
+#pragma unroll 4
+  for (int u = threadIdx.x; u < rows * R; u += T) stg(g + u, cscale(s[u / R * P + u % R], sc), pol);
 }
 
 // Half spectrum of a real row of 2 L points from Z: X[k] = E + W_n^k O and
@@ -254,9 +243,9 @@ __device__ __forceinline__ void rows_out(float2* g, const float2* s, int rows, f
 // O = -i (Z[k] - conj Z[L-k]) / 2.  z[k1] = Z[k2 + B k1]; mz holds the
 // mirrors: mz[A-1-k1] = Z[L-k2-B k1], or, for k2 = 0, z itself with
 // Z[L - B k1] = z[(A - k1) % A].  A = 1 (L = B): z and mz are the row.
-template <int L, int A, bool STAGED>
-__device__ __forceinline__ void split_store(const PencilArgs& a, float2* dst, const float2* z,
-                                            const float2* mz, int k2, uint64_t pout) {
+template <int L, int A>
+__device__ __forceinline__ void split(const float2* twr, float2* dst, const float2* z,
+                                      const float2* mz, int k2) {
   constexpr int B = L / A, N = A == 1 ? L : A, S = A == 1 ? 1 : B;
 #pragma unroll
   for (int k1 = 0; k1 < N; ++k1) {
@@ -264,19 +253,9 @@ __device__ __forceinline__ void split_store(const PencilArgs& a, float2* dst, co
     const float2 u = z[k1], m = k2 == 0 ? z[(N - k1) % N] : mz[N - 1 - k1];
     const float2 E = make_float2(0.5f * (u.x + m.x), 0.5f * (u.y - m.y));
     const float2 O = make_float2(0.5f * (u.y + m.y), 0.5f * (m.x - u.x));
-    const float2 t = cmul_tw<-1>(O, __ldg(a.twr + k));
-    float2 lo = cadd(E, t), hi = make_float2(E.x - t.x, t.y - E.y);
-    if constexpr (STAGED) {
-      dst[k] = lo;
-      dst[L - k] = hi;
-    } else {
-      if (a.do_scale) {
-        lo = cscale(lo, a.scale);
-        hi = cscale(hi, a.scale);
-      }
-      stg(dst + k, lo, pout);
-      stg(dst + L - k, hi, pout);
-    }
+    const float2 t = cmul_tw<-1>(O, __ldg(twr + k));
+    dst[k] = cadd(E, t);
+    dst[L - k] = make_float2(E.x - t.x, t.y - E.y);
   }
 }
 
@@ -291,38 +270,43 @@ __global__ void __launch_bounds__(Cfg<L, KIND>::T, Cfg<L, KIND>::blocks) pencil_
   const uint64_t pin = l2_policy(a.pol_in), pout = l2_policy(a.pol_out);
   asm volatile("griddepcontrol.wait;" ::: "memory");
 
-  // first point of pencil p (in: input side, else output side)
-  auto base = [&](unsigned p, bool in) -> long long {
+  const int np = (int)min((unsigned)W, a.np - p0);  // pencils of this block
+  // first point of pencil c of the block
+  auto base = [&](int c) -> long long {
+    const unsigned p = p0 + (unsigned)c;
     if constexpr (KIND == kStrided) {
       const unsigned o = fdiv(p, a.divn);
       return (long long)o * a.so + (long long)(p - o * a.nx);
     } else {
-      const int pitch = KIND == kR2C && !in ? L + 1 : KIND == kC2R && in ? L + 1 : L;
-      return (long long)p * pitch;
+      return (long long)p * L;
     }
   };
+  float2* const st = sm + C::exchange;  // staged real rows in
+  float2* const so = st + C::out_at;    // and out
+  if constexpr (C::REAL) {
+    rows_in<C::IR, C::SP, T>(st, a.in + (size_t)p0 * C::IR, np, pin);
+    __syncthreads();
+  }
 
   // phase 1
 #pragma unroll 1
   for (int it = 0; it < C::I1; ++it) {
     const int e = threadIdx.x + it * T;
     if (e >= C::N1) break;
+    const int c = KIND == kContig ? e / A : e % W, n1 = KIND == kContig ? e % A : e / W;
+    if (c >= np) continue;
     if constexpr (KIND == kC2R) {
       // Z[k] = 2 E + i 2 O and Z[L-k] = conj(2 E) + i conj(2 O) with
       // 2 E = X[k] + conj X[L-k], 2 O = (X[k] - conj X[L-k]) W_n^-k: the item
       // of n1 makes the points n1 + A j and their mirrors, A - n1 + A j (its
       // own points for n1 = 0 and A / 2).  Of X[0] and X[L] only the real
       // parts count.
-      constexpr int H = A > 1 ? A / 2 + 1 : 1;
-      const int c = e / H, n1 = e % H;
-      const unsigned p = p0 + (unsigned)c;
-      if (p >= a.np) continue;
-      const float2* src = a.in + base(p, true);
+      const float2* row = st + c * C::SP;
       float2 u[B], m[B];
 #pragma unroll
       for (int j = 0; j < B; ++j) {
-        u[j] = ldg(src + n1 + A * j, pin);
-        m[j] = ldg(src + L - n1 - A * j, pin);
+        u[j] = row[n1 + A * j];
+        m[j] = row[L - n1 - A * j];
       }
       if (n1 == 0) u[0].y = m[0].y = 0.0f;
 #pragma unroll
@@ -335,9 +319,10 @@ __global__ void __launch_bounds__(Cfg<L, KIND>::T, Cfg<L, KIND>::blocks) pencil_
       }
       transform<B, DIR>(u);
       if constexpr (A > 1) {
+        float2* x = sm + c * C::RP;
 #pragma unroll
         for (int k = 0; k < B; ++k)
-          sm[c * C::RP + k * C::AP + n1] = k ? twiddle<DIR>(u[k], __ldg(a.tw + k * A + n1)) : u[k];
+          x[k * C::AP + n1] = k ? twiddle<DIR>(u[k], __ldg(a.tw + k * A + n1)) : u[k];
         if (n1 != 0 && 2 * n1 != A) {
           float2 v[B];
 #pragma unroll
@@ -346,24 +331,24 @@ __global__ void __launch_bounds__(Cfg<L, KIND>::T, Cfg<L, KIND>::blocks) pencil_
           const int n2 = A - n1;
 #pragma unroll
           for (int k = 0; k < B; ++k)
-            sm[c * C::RP + k * C::AP + n2] = k ? twiddle<DIR>(v[k], __ldg(a.tw + k * A + n2)) : v[k];
+            x[k * C::AP + n2] = k ? twiddle<DIR>(v[k], __ldg(a.tw + k * A + n2)) : v[k];
         }
       } else {
-        float2* dst = a.out + base(p, false);
 #pragma unroll
-        for (int k = 0; k < B; ++k) stg(dst + k, a.do_scale ? cscale(u[k], sc) : u[k], pout);
+        for (int k = 0; k < B; ++k) so[c * C::SP + k] = u[k];
       }
     } else {
-      const int c = KIND == kStrided ? e % W : e / A;
-      const int n1 = KIND == kStrided ? e / W : e % A;
-      const unsigned p = p0 + (unsigned)c;
-      if (p >= a.np) continue;
-      const float2* src = a.in + base(p, true);
-      const long long step = KIND == kStrided ? (long long)A * a.pi : A;
-      src += KIND == kStrided ? (long long)n1 * a.pi : n1;
       float2 v[B];
+      if constexpr (KIND == kR2C) {
+        const float2* row = st + c * C::SP + n1;
 #pragma unroll
-      for (int j = 0; j < B; ++j) v[j] = ldg(src + j * step, pin);
+        for (int j = 0; j < B; ++j) v[j] = row[A * j];
+      } else {
+        const long long pi = KIND == kStrided ? a.pi : 1, step = A * pi;
+        const float2* src = a.in + base(c) + n1 * pi;
+#pragma unroll
+        for (int j = 0; j < B; ++j) v[j] = ldg(src + j * step, pin);
+      }
       transform<B, DIR>(v);
       if constexpr (A > 1) {
 #pragma unroll
@@ -372,9 +357,9 @@ __global__ void __launch_bounds__(Cfg<L, KIND>::T, Cfg<L, KIND>::blocks) pencil_
           sm[KIND == kStrided ? (k * A + n1) * W + c : c * C::RP + k * C::AP + n1] = y;
         }
       } else if constexpr (KIND == kR2C) {
-        split_store<L, 1, true>(a, sm + c * C::OP, v, v, 0, pout);
+        split<L, 1>(a.twr, so + c * C::SP, v, v, 0);
       } else {
-        float2* dst = a.out + base(p, false);
+        float2* dst = a.out + base(c);
         const long long ostep = KIND == kStrided ? a.pi : 1;
 #pragma unroll
         for (int k = 0; k < B; ++k) stg(dst + k * ostep, a.do_scale ? cscale(v[k], sc) : v[k], pout);
@@ -389,47 +374,45 @@ __global__ void __launch_bounds__(Cfg<L, KIND>::T, Cfg<L, KIND>::blocks) pencil_
     for (int it = 0; it < C::I2; ++it) {
       const int e = threadIdx.x + it * T;
       if (e >= C::N2) break;
-      constexpr int H = KIND == kR2C ? B / 2 + 1 : B;  // items of a row
-      const int c = KIND == kStrided ? e % W : e / H;
-      const int k2 = KIND == kStrided ? e / W : e % H;
-      const unsigned p = p0 + (unsigned)c;
-      if (p >= a.np) continue;
+      const int c = KIND == kContig ? e / B : e % W, k2 = KIND == kContig ? e % B : e / W;
+      if (c >= np) continue;
       float2 v[A];
 #pragma unroll
       for (int j = 0; j < A; ++j)
         v[j] = sm[KIND == kStrided ? (k2 * A + j) * W + c : c * C::RP + k2 * C::AP + j];
       transform<A, DIR>(v);
       if constexpr (KIND == kR2C) {
-        float2* row = C::staged ? sm + C::exchange + c * C::OP : a.out + base(p, false);
+        float2* row = so + c * C::SP;
         // the mirrors of this item's outputs are those of B - k2
         if (k2 == 0 || 2 * k2 == B) {
-          split_store<L, A, C::staged>(a, row, v, v, k2, pout);
+          split<L, A>(a.twr, row, v, v, k2);
         } else {
           float2 w[A];
 #pragma unroll
           for (int j = 0; j < A; ++j) w[j] = sm[c * C::RP + (B - k2) * C::AP + j];
           transform<A, DIR>(w);
-          split_store<L, A, C::staged>(a, row, v, w, k2, pout);
+          split<L, A>(a.twr, row, v, w, k2);
         }
+      } else if constexpr (KIND == kC2R) {
+        float2* row = so + c * C::SP + k2;
+#pragma unroll
+        for (int k = 0; k < A; ++k) row[B * k] = v[k];
       } else {
-        float2* dst = a.out + base(p, false);
+        const long long pi = KIND == kStrided ? a.pi : 1, step = B * pi;
+        float2* dst = a.out + base(c) + k2 * pi;
         if (a.do_scale) {
 #pragma unroll
           for (int k = 0; k < A; ++k) v[k] = cscale(v[k], sc);
         }
-        const long long step = KIND == kStrided ? (long long)B * a.pi : B;
-        dst += KIND == kStrided ? (long long)k2 * a.pi : k2;
 #pragma unroll
         for (int k = 0; k < A; ++k) stg(dst + k * step, v[k], pout);
       }
     }
   }
 
-  if constexpr (C::staged) {
+  if constexpr (C::REAL) {
     __syncthreads();
-    const int rows = (int)min((unsigned)W, a.np - p0);
-    rows_out<L + 1, C::OP, T>(a.out + (size_t)p0 * (L + 1), sm + C::exchange, rows,
-                              a.do_scale ? sc : 1.0f, pout);
+    rows_out<C::OR, C::SP, T>(a.out + (size_t)p0 * C::OR, so, np, a.do_scale ? sc : 1.0f, pout);
   }
 }
 

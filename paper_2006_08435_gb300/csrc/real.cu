@@ -25,7 +25,7 @@
 // other edges above 2 as one pencil pass per axis (passes.cu): 24 bytes per
 // real point through L2 where the pair scheme moves about 60 and makes the
 // passes of a whole complex transform (96^3 x 32, forward + inverse 333 ->
-// 214 us, 100^3 x 16 286 -> 124, 20^3 x 500 373 -> 45).  The pair scheme
+// 194 us, 100^3 x 16 286 -> 114, 20^3 x 500 373 -> 45).  The pair scheme
 // remains for n = 2 and the tensor-core precisions; its kernels here move
 // data only (pack, separate, rebuild, split) and its transforms are the
 // library's complex plans.  Packing two grids into one makes each grid's
