@@ -290,7 +290,8 @@ int fft3d_selftest_wait_timeout(int64_t timeout_ns);
  * the general path (every plan that is not cubic with a fused edge;
  * selectable for those too): per chunk of grids that fits L2, the x pass
  * (in -> out) and the y and z passes in place on out, each a batched 1D
- * transform of the pencils of one axis, split into two register codelets;
+ * transform of the pencils of one axis, split into two register codelets
+ * (cubic edges 48, 60, 64, 72, 80, 90, 96, 100, 108 and 128: two passes);
  * the launches of a batch above 40 MB alternate between the caller's stream
  * and a side stream of the plan, forked and joined by events (in a captured
  * graph, parallel branches). Mixed plans:

@@ -83,6 +83,7 @@ struct KernelInfo {
 // axis at a time (axis.cu).
 constexpr int kAxisMaxLen = 512;
 constexpr int kGeneralVariant = 10;  // plan variant of the general path
+constexpr int kFixedVariant = 11;    // the same as three passes at every edge (internal)
 constexpr int kAxisMaxStages = 12;
 
 // n / d = (hi32(n * mul) + n) >> shift for every n < 2^32 (make_fastdiv).
@@ -122,8 +123,27 @@ struct PencilKernel {
 // same inverse (dir 1); launch is null for an edge that is not plannable.
 PencilKernel pencil_kernel_info(int L, int dir, int kind);
 
+// Two-pass transforms of cubic edges (twopass.cuh).  tx, ty, tz: W_L^(n1 k) at
+// [k * split + n1] for the splits AX, A and AZ.
+constexpr int kTwoPassMaxLen = 160;
+struct TwoPassArgs {
+  const float2* in;  // may equal out
+  float2* out;
+  const float2 *tx, *tzg;
+  float2 ty[kTwoPassMaxLen], tz[kTwoPassMaxLen];
+  float scale;
+  int do_scale;
+};
+struct TwoPassKernel {
+  cudaError_t (*launch)(const TwoPassArgs&, int grids, int which, cudaStream_t) = nullptr;
+  const void* func[3] = {};  // pass 1, pass 1 in place, pass 2
+  size_t smem[3] = {};
+  int A = 0, AX = 0, AZ = 0;
+};
+TwoPassKernel two_pass_kernel_info(int L, int dir);  // launch null: none
+
 // A 3D transform as three pencil passes (passes.cu): complex grids (x, y, z,
-// out of place or in place), real grids to half spectra (x, y, z) or back
+// out of place or in place; as two passes at some cubic edges unless `fixed`), real grids to half spectra (x, y, z) or back
 // (z into a workspace of work_points() complex points, y, x).
 constexpr int kMaxChains = 2;
 enum PassKind { kPassC2C = 0, kPassR2C = 1, kPassC2R = 2 };
@@ -133,6 +153,8 @@ struct AxisPasses {
   long long chunk = 0;  // grids per chunk
   long long sub = 0;    // planes per launch of the x and y passes
   PencilKernel k[3];
+  TwoPassKernel two;    // launch not null: two passes instead
+  TwoPassArgs two_args;
   int chains = 1;       // streams the chunks alternate between
   cudaStream_t side = nullptr;
   cudaEvent_t fork = nullptr, join = nullptr;
@@ -143,7 +165,7 @@ struct AxisPasses {
   float scale = 1.0f;
   int do_scale = 0;
   int create(PassKind kind, int nx, int ny, int nz, int batch, int dir, float scale, int do_scale,
-             int l2_bytes);
+             int l2_bytes, bool fixed = false);
   void destroy();
   long long work_points() const;
   cudaError_t execute(const void* in, void* out, float2* work, cudaStream_t s) const;

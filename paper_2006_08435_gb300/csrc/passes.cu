@@ -1,5 +1,5 @@
 // The general path's schedule: a 3D transform as one pencil pass per axis
-// (pencil.cuh), over chunks of grids -- or, for a grid beyond the chunk
+// (pencil.cuh), or two passes at some cubic edges (twopass.cuh), over chunks of grids -- or, for a grid beyond the chunk
 // budget, ranges of its planes for x and y -- whose intermediate stays in
 // L2 from one pass to the next.
 //
@@ -55,7 +55,7 @@ float2 root(long long m, int n) {
 }  // namespace
 
 int AxisPasses::create(PassKind kind_, int nx_, int ny_, int nz_, int batch_, int dir, float scale_,
-                       int do_scale_, int l2_bytes) {
+                       int do_scale_, int l2_bytes, bool fixed) {
   kind = kind_;
   nx = nx_;
   ny = ny_;
@@ -67,6 +67,16 @@ int AxisPasses::create(PassKind kind_, int nx_, int ny_, int nz_, int batch_, in
   hx = kind == kPassC2C ? nx : nx / 2 + 1;
   const int len[3] = {lx, ny, nz};
   const int kx = kind == kPassC2C ? 1 : kind == kPassR2C ? 2 : 3;
+  two = TwoPassKernel{};
+  if (kind == kPassC2C && nx == ny && ny == nz && !fixed) two = two_pass_kernel_info(nx, dir);
+  if (two.launch)
+    for (int i = 0; i < 3; ++i)
+      if (two.smem[i] > 48 * 1024 &&
+          cudaFuncSetAttribute(two.func[i], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)two.smem[i]) != cudaSuccess) {
+        cudaGetLastError();
+        return FFT3D_ERR_CUDA;
+      }
   std::vector<float2> tab;
   size_t off[3], off_r = 0;
   for (int a = 0; a < 3; ++a) {
@@ -79,7 +89,8 @@ int AxisPasses::create(PassKind kind_, int nx_, int ny_, int nz_, int batch_, in
       return FFT3D_ERR_CUDA;
     }
     off[a] = tab.size();
-    const int A = k[a].A, B = len[a] / A;
+    const int A = !two.launch ? k[a].A : a == 0 ? two.AX : a == 1 ? two.A : two.AZ;
+    const int B = len[a] / A;
     if (A > 1)
       for (int k2 = 0; k2 < B; ++k2)
         for (int n1 = 0; n1 < A; ++n1) tab.push_back(root((long long)n1 * k2, len[a]));
@@ -100,18 +111,29 @@ int AxisPasses::create(PassKind kind_, int nx_, int ny_, int nz_, int batch_, in
   }
   for (int a = 0; a < 3; ++a) tw[a] = d_tab + off[a];
   twr = d_tab + off_r;
+  if (two.launch) {
+    two_args.tx = tw[0];
+    two_args.tzg = tw[2];
+    for (int i = 0; i < nx; ++i) {
+      two_args.ty[i] = tab[off[1] + i];
+      two_args.tz[i] = tab[off[2] + i];
+    }
+    two_args.scale = scale;
+    two_args.do_scale = do_scale;
+  }
 
   // Chunk budget: the intermediates of the chunks in flight within 40% of L2
   // (complex grids: 96 x 128 x 64 x 64 261 us, 60%: 270), 60% for real
   // grids, whose other side is half as large (96^3 x 32 forward 111 -> 107,
-  // 160^3 x 4 65 -> 61 us).  One chain below 40 MB, where the fork and join
+  // 160^3 x 4 65 -> 61 us), and for two passes (128^3 x 32: 40% 338, 55% 297,
+  // 70% 297, 85% 312; 64^3 x 256: 297, 295, 298, 316).  One chain below 40 MB, where the fork and join
   // cost more than the overlap gives (64^3, one chain / two: 8 grids 18.9 /
   // 20.7 us, 16 grids 27.8 / 27.9, 24 grids 38.8 / 35.3).
   const long long pp = (long long)hx * ny;
   const double plane_bytes = 8.0 * (double)pp, grid_bytes = plane_bytes * nz;
   const double l2 = (double)l2_bytes;
   chains = batch >= 2 && grid_bytes * batch > 40.0 * 1048576.0 ? kMaxChains : 1;
-  const double budget = (kind == kPassC2C ? 0.4 : 0.6) * l2 / chains;
+  const double budget = (kind == kPassC2C && !two.launch ? 0.4 : 0.6) * l2 / chains;
   // a pass's pencils stay below 2^31
   const long long most = std::max({(long long)ny * nz, (long long)nz * hx, pp});
   const long long cap = std::max(1LL, (1LL << 30) / most);
@@ -155,6 +177,14 @@ long long AxisPasses::work_points() const { return chains * chunk * hx * ny * nz
 cudaError_t AxisPasses::chunk_passes(long long g, const void* in, void* out, float2* work,
                                      cudaStream_t s) const {
   const long long pp = (long long)hx * ny;  // complex points of a plane
+  if (two.launch) {
+    const long long m = std::min(chunk, batch - g);
+    TwoPassArgs a = two_args;
+    a.in = static_cast<const float2*>(in) + g * pp * nz;
+    a.out = static_cast<float2*>(out) + g * pp * nz;
+    const cudaError_t e = two.launch(a, (int)m, 1, s);
+    return e == cudaSuccess ? two.launch(a, (int)m, 2, s) : e;
+  }
   // contiguous rows of `planes` planes
   auto x_pass = [&](const float2* src, float2* dst, long long planes) {
     PencilArgs a{};

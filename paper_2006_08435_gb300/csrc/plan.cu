@@ -206,9 +206,8 @@ std::vector<int> variant_candidates(bool mixed, int n, int precision) {
 // (back-to-back executes):
 //   16^3: cluster-fused below 128 grids, whole grid per block from 128;
 //   32^3: cluster-fused below 48 grids, pencil passes below 300, thread pairs;
-//   48^3, 64^3, 80^3, 96^3, 128^3: pencil passes for few grids (below 36, 20,
-//     18, 8 and 3), then thread pairs (48, 80, 96), thread-per-pencil and from
-//     64 grids two-plane (64), split-y (128);
+//   48^3: two passes; 64^3, 80^3, 96^3, 128^3: two passes (below 80, 150, 36 and
+//     20 grids), then two-plane (64), thread pairs (80, 96), split-y (128);
 //   tensor-core precisions: the plain persistent kernel (mma.sync) for few
 //     grids, the tcgen05 kernels from 16 (64^3) and 2 (128^3) grids.
 int builtin_default_variant(bool mixed, int n, int batch, int precision) {
@@ -226,27 +225,28 @@ int builtin_default_variant(bool mixed, int n, int batch, int precision) {
     // the whole-grid kernel from 128 (x 256: 0.29 against 0.15; x 4096:
     // 0.53 against 0.17)
     case 16: return batch >= 128 ? 12 : 3;
-    // Pencil passes (three dependent launches) fill the GPU with small blocks
-    // where the ticket kernels' large items leave it idle; their 48 bytes
-    // per point through L2 lose to the two-phase kernels once those fill it.
-    // us, pencil passes / the kernels before:
-    // 32^3 x 16 8.9 / 10.5, x 32 13.1 / 12.2 (3), x 64 15.7 / 18.8, x 127 24.5 /
+    // The general path (dependent launches of small blocks: three pencil
+    // passes at 32^3, two passes at the others) fills the GPU where the ticket
+    // kernels' large items leave it idle, and pays 4 us per launch of a chunk
+    // where they pay once.  us, general path / the kernels before:
+    // 32^3 x 16 8.5 / 10.5, x 32 13.1 / 12.2 (3), x 64 15.7 / 18.8, x 127 24.5 /
     // 31.5, x 200 35.9 / 39.5 (13), x 400 67.6 / 66.5
     case 32: return batch >= 300 ? 13 : batch >= 48 ? kGeneralVariant : 3;
-    // 48^3 x 1 8.9 / 11.8 (0), x 4 8.6 / 14.1, x 24 19.7 / 25.3, x 32 24.6 / 25.3
-    // (13), x 48 33.3 / 30.2
-    case 48: return batch >= 36 ? 13 : kGeneralVariant;
-    // 64^3 x 1 8.8 / 11.7 (5), x 4 12.2 / 18.4 (1), x 16 25.2 / 29.0 (7), x 24
-    // 35.1 / 33.8, x 48 68.3 / 61.6, x 64 89.1 / 77.0 (8)
-    case 64: return batch >= 64 ? 8 : batch >= 20 ? 7 : kGeneralVariant;
-    // 80^3 x 1 8.6 / 14.9 (0), x 4 15.7 / 25.1 (4), x 8 26.0 / 32.4 (13), x 16
-    // 48.1 / 52.2
-    case 80: return batch >= 18 ? 13 : kGeneralVariant;
-    // 96^3 x 1 12.6 / 17.1 (0), x 4 24.1 / 33.9 (13), x 6 30.8 / 35.0, x 8 43.1 /
-    // 42.7
-    case 96: return batch >= 8 ? 13 : kGeneralVariant;
-    // 128^3 x 1 17.0 / 20.9 (5), x 2 27.7 / 32.6 (6), x 3 42.4 / 40.3
-    case 128: return batch >= 3 ? 6 : kGeneralVariant;
+    // 48^3 x 1 7.2 / 11.8 (0), x 16 12.6 / 23.1, x 40 19.8 / 27.9 (13), x 400 178 /
+    // 192
+    case 48: return kGeneralVariant;
+    // 64^3 x 1 7.1 / 11.7 (5), x 4 8.7 / 18.4 (1), x 32 38.3 / 51.0 (7), x 64
+    // 74.6 / 77.7 (8), x 100 113.8 / 110.1
+    case 64: return batch >= 80 ? 8 : kGeneralVariant;
+    // 80^3 x 1 9.5 / 14.9 (0), x 12 30.8 / 37.6 (13), x 80 182 / 189, x 200 450 /
+    // 442
+    case 80: return batch >= 150 ? 13 : kGeneralVariant;
+    // 96^3 x 1 10.5 / 17.1 (0), x 8 33.6 / 43.0 (13), x 24 97.8 / 101.9, x 48 188.9 /
+    // 182.9
+    case 96: return batch >= 36 ? 13 : kGeneralVariant;
+    // 128^3 x 1 17.3 / 20.9 (5), x 2 23.6 / 31.7 (6), x 8 78.7 / 86.4, x 16 152.6 /
+    // 155.2, x 24 225.4 / 222.8
+    case 128: return batch >= 20 ? 6 : kGeneralVariant;
     default: return 0;
   }
 }
@@ -622,7 +622,7 @@ int create_general(fft3d_plan p) {
   if (cudaDeviceGetAttribute(&l2_bytes, cudaDevAttrL2CacheSize, p->device) != cudaSuccess)
     return FFT3D_ERR_CUDA;
   return p->passes.create(kPassC2C, p->nx, p->ny, p->nz, p->batch, p->direction, p->scale,
-                          p->do_scale, l2_bytes);
+                          p->do_scale, l2_bytes, p->variant == kFixedVariant);
 }
 
 // Validated arguments -> plan (variant < 0: environment override, tuning
@@ -636,7 +636,7 @@ int create_uniform(int nx, int ny, int nz, int batch, int precision, int directi
     // the general path is the only one for these edges
     if (precision != FFT3D_FP32) return FFT3D_ERR_UNSUPPORTED_PRECISION;
     if (variant < 0) variant = kGeneralVariant;
-    if (variant != kGeneralVariant) return FFT3D_ERR_INVALID_ARG;
+    if (variant != kGeneralVariant && variant != kFixedVariant) return FFT3D_ERR_INVALID_ARG;
   } else {
     if (variant < 0) variant = pick_variant(false, nx, batch, precision, direction, nullptr, 0);
     const std::vector<int> cand = variant_candidates(false, nx, precision);
@@ -654,7 +654,7 @@ int create_uniform(int nx, int ny, int nz, int batch, int precision, int directi
   for (int g = 0; g < batch; ++g) p->offsets[g] = (long long)g * pts;
   p->total_points = pts * batch;
   set_scale(p, (double)pts);
-  if (variant == kGeneralVariant) {
+  if (variant == kGeneralVariant || variant == kFixedVariant) {
     p->general = true;
     if (cudaMalloc(&p->d_status, sizeof(unsigned)) != cudaSuccess ||
         cudaMemset(p->d_status, 0, sizeof(unsigned)) != cudaSuccess)

@@ -394,11 +394,11 @@ int create_pair_real(int n, int batch, int direction, fft3d_plan inner, fft3d_re
 
 // The complex kernel of fft3d_real_plan_create_fixed: at 48^3, 80^3 and 96^3
 // the persistent kernel, from as many pairs as first chosen the thread-pair
-// kernel (another arithmetic order); elsewhere the pencil passes, which have
-// the order of the passes before them (pencil.cuh: split_a).
+// kernel (another arithmetic order); elsewhere three pencil passes, which
+// have the order of the passes before them (pencil.cuh: split_a).
 int fixed_variant(int n, int pairs) {
   const int from = n == 48 ? 32 : n == 80 ? 8 : n == 96 ? 4 : 0;
-  return !from ? kGeneralVariant : pairs >= from ? 13 : n == 80 && pairs >= 4 ? 4 : 0;
+  return !from ? kFixedVariant : pairs >= from ? 13 : n == 80 && pairs >= 4 ? 4 : 0;
 }
 
 }  // namespace
