@@ -205,8 +205,9 @@ int fft3d_plan_grid_offset(fft3d_plan plan, int g, int64_t* offset);
  *   stream  : cudaStream_t or NULL.
  * Asynchronous, allocates nothing, never synchronises, and is capturable in
  * a CUDA graph (per launch unit a memset node for its work counters, when
- * its kernel uses them, and a kernel node; mixed variant 2 puts the units
- * on the plan's side streams between event fork and join nodes).
+ * its kernel uses them, and kernel nodes; mixed variant 2 and large batches on
+ * the general path put half of them on the plan's side stream, between event
+ * fork and join nodes).
  */
 int fft3d_execute(fft3d_plan plan, const void* in, void* out, void* stream);
 
@@ -295,16 +296,15 @@ int fft3d_selftest_wait_timeout(int64_t timeout_ns);
  * the launches of a batch above 40 MB alternate between the caller's stream
  * and a side stream of the plan, forked and joined by events (in a captured
  * graph, parallel branches). Mixed plans:
- * 0 one launch of the mixed-edge kernel, 1 one launch per distinct edge (the
- * tensor-TMA kernels of 128^3 and 32^3 .. 96^3 take one pair of
- * tensor maps per grid, up to 32 grids of an edge; an edge whose default is
- * a tensor-TMA kernel otherwise takes variant 0 at 32^3 .. 96^3
- * (4 at 80^3 from 4 grids) and 5 at 128^3, as do calls with pointer
- * arrays), 2 the
- * launches of 1 on two concurrent branches, the caller's stream and a side
- * stream of the plan: it waits on the caller's stream and the caller's
- * stream waits on it (in a captured graph, parallel branches between a fork
- * and a join).
+ * 0 one launch of the mixed-edge kernel, 1 the launches of each distinct edge
+ * in sequence (the two-pass kernels of 10 where they are the default of so
+ * many grids; else the edge's kernel, the tensor-TMA kernels of 128^3 and
+ * 32^3 .. 96^3 with one pair of tensor maps per grid, up to 32 grids of an edge;
+ * beyond that, and for calls with pointer arrays, variant 0 at 48^3 and 96^3, 4
+ * at 80^3, 3 at 32^3 and 5 at 128^3), 2 the launches of 1 on two concurrent
+ * branches, the caller's stream and a side stream of the plan: it waits on
+ * the caller's stream and the caller's stream waits on it (in a captured
+ * graph, parallel branches between a fork and a join).
  * At create the variant comes from FFT3D_VARIANT / FFT3D_MIXED_VARIANT if
  * set, else from the tuning cache named by FFT3D_TUNE_CACHE (tuned on the
  * spot when FFT3D_TUNE=1 and the entry is missing), else a built-in default.

@@ -133,14 +133,27 @@ struct TwoPassArgs {
   float2 ty[kTwoPassMaxLen], tz[kTwoPassMaxLen];
   float scale;
   int do_scale;
+  // grids that do not lie back to back (two_pass_apart_kernel_info): grid i is
+  // plan grid map[first + i] (map null: first + i), at element off[.] of in and
+  // out or at the pointers of the arrays
+  const long long* off;
+  const int* map;
+  const float2* const* in_ptrs;
+  float2* const* out_ptrs;
+  int first;
 };
 struct TwoPassKernel {
-  cudaError_t (*launch)(const TwoPassArgs&, int grids, int which, cudaStream_t) = nullptr;
+  // passes 1 and 2 of `grids` grids; in_place: some output may overlie its input
+  cudaError_t (*launch)(const TwoPassArgs&, int grids, bool in_place, cudaStream_t) = nullptr;
   const void* func[3] = {};  // pass 1, pass 1 in place, pass 2
   size_t smem[3] = {};
   int A = 0, AX = 0, AZ = 0;
 };
-TwoPassKernel two_pass_kernel_info(int L, int dir);  // launch null: none
+TwoPassKernel two_pass_kernel_info(int L, int dir);        // launch null: none
+TwoPassKernel two_pass_apart_kernel_info(int L, int dir);  // for mixed-edge plans
+// The kernel's twiddles: ty and tz into a, tx and tzg appended to tab (2 L
+// entries: a.tx and a.tzg are set once tab is on the device).
+int two_pass_prepare(const TwoPassKernel& k, int L, TwoPassArgs& a, std::vector<float2>& tab);
 
 // A 3D transform as three pencil passes (passes.cu): complex grids (x, y, z,
 // out of place or in place; as two passes at some cubic edges unless `fixed`), real grids to half spectra (x, y, z) or back

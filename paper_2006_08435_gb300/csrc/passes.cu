@@ -54,6 +54,24 @@ float2 root(long long m, int n) {
 
 }  // namespace
 
+int two_pass_prepare(const TwoPassKernel& k, int L, TwoPassArgs& a, std::vector<float2>& tab) {
+  for (int i = 0; i < 3; ++i)
+    if (k.smem[i] > 48 * 1024 &&
+        cudaFuncSetAttribute(k.func[i], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)k.smem[i]) != cudaSuccess) {
+      cudaGetLastError();
+      return FFT3D_ERR_CUDA;
+    }
+  a = TwoPassArgs{};
+  for (int i = 0; i < L; ++i) {
+    a.ty[i] = root((long long)(i / k.A) * (i % k.A), L);
+    a.tz[i] = root((long long)(i / k.AZ) * (i % k.AZ), L);
+  }
+  for (int i = 0; i < L; ++i) tab.push_back(root((long long)(i / k.AX) * (i % k.AX), L));
+  tab.insert(tab.end(), a.tz, a.tz + L);
+  return FFT3D_SUCCESS;
+}
+
 int AxisPasses::create(PassKind kind_, int nx_, int ny_, int nz_, int batch_, int dir, float scale_,
                        int do_scale_, int l2_bytes, bool fixed) {
   kind = kind_;
@@ -69,17 +87,15 @@ int AxisPasses::create(PassKind kind_, int nx_, int ny_, int nz_, int batch_, in
   const int kx = kind == kPassC2C ? 1 : kind == kPassR2C ? 2 : 3;
   two = TwoPassKernel{};
   if (kind == kPassC2C && nx == ny && ny == nz && !fixed) two = two_pass_kernel_info(nx, dir);
-  if (two.launch)
-    for (int i = 0; i < 3; ++i)
-      if (two.smem[i] > 48 * 1024 &&
-          cudaFuncSetAttribute(two.func[i], cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)two.smem[i]) != cudaSuccess) {
-        cudaGetLastError();
-        return FFT3D_ERR_CUDA;
-      }
   std::vector<float2> tab;
-  size_t off[3], off_r = 0;
-  for (int a = 0; a < 3; ++a) {
+  size_t off[3] = {}, off_r = 0;
+  if (two.launch) {
+    const int rc = two_pass_prepare(two, nx, two_args, tab);
+    if (rc) return rc;
+    two_args.scale = scale;
+    two_args.do_scale = do_scale;
+  }
+  for (int a = 0; a < 3 && !two.launch; ++a) {
     k[a] = pencil_kernel_info(len[a], dir, a == 0 ? kx : 0);
     if (!k[a].launch) return FFT3D_ERR_UNSUPPORTED_SIZE;
     if (k[a].smem > 48 * 1024 &&
@@ -89,8 +105,7 @@ int AxisPasses::create(PassKind kind_, int nx_, int ny_, int nz_, int batch_, in
       return FFT3D_ERR_CUDA;
     }
     off[a] = tab.size();
-    const int A = !two.launch ? k[a].A : a == 0 ? two.AX : a == 1 ? two.A : two.AZ;
-    const int B = len[a] / A;
+    const int A = k[a].A, B = len[a] / A;
     if (A > 1)
       for (int k2 = 0; k2 < B; ++k2)
         for (int n1 = 0; n1 < A; ++n1) tab.push_back(root((long long)n1 * k2, len[a]));
@@ -111,16 +126,8 @@ int AxisPasses::create(PassKind kind_, int nx_, int ny_, int nz_, int batch_, in
   }
   for (int a = 0; a < 3; ++a) tw[a] = d_tab + off[a];
   twr = d_tab + off_r;
-  if (two.launch) {
-    two_args.tx = tw[0];
-    two_args.tzg = tw[2];
-    for (int i = 0; i < nx; ++i) {
-      two_args.ty[i] = tab[off[1] + i];
-      two_args.tz[i] = tab[off[2] + i];
-    }
-    two_args.scale = scale;
-    two_args.do_scale = do_scale;
-  }
+  two_args.tx = d_tab;
+  two_args.tzg = d_tab + nx;
 
   // Chunk budget: the intermediates of the chunks in flight within 40% of L2
   // (complex grids: 96 x 128 x 64 x 64 261 us, 60%: 270), 60% for real
@@ -182,8 +189,7 @@ cudaError_t AxisPasses::chunk_passes(long long g, const void* in, void* out, flo
     TwoPassArgs a = two_args;
     a.in = static_cast<const float2*>(in) + g * pp * nz;
     a.out = static_cast<float2*>(out) + g * pp * nz;
-    const cudaError_t e = two.launch(a, (int)m, 1, s);
-    return e == cudaSuccess ? two.launch(a, (int)m, 2, s) : e;
+    return two.launch(a, (int)m, in == out, s);
   }
   // contiguous rows of `planes` planes
   auto x_pass = [&](const float2* src, float2* dst, long long planes) {

@@ -289,6 +289,16 @@ struct Unit {
   // (KernelInfo::launch_maps) over these element offsets of the unit's grids
   bool use_maps = false;
   std::vector<long long> host_off;
+  // mixed-edge plans: the two-pass kernels (twopass.cuh) instead of `kernel`
+  TwoPassKernel two;
+  TwoPassArgs two_args;
+  float2* d_two = nullptr;
+};
+
+// One launch of a mixed-edge plan: grids [first, first + count) of a unit, on
+// the caller's stream (branch 0) or the side stream (1).
+struct MixedStep {
+  int unit, first, count, branch;
 };
 
 struct HostIO;
@@ -314,6 +324,7 @@ struct fft3d_plan_s {
   // mixed variant 2: the units on two concurrent branches, the caller's
   // stream and a side stream forked from it (owned)
   bool branches = false;
+  std::vector<MixedStep> steps;
   cudaEvent_t fork = nullptr, join = nullptr;
   cudaStream_t side = nullptr;
   // device buffers shared by the units (owned)
@@ -336,6 +347,8 @@ void free_plan_buffers(fft3d_plan p) {
     cudaFree(u.d_blocks);
     cudaFree(u.d_work);
     cudaFree(u.d_map);
+    cudaFree(u.d_two);
+    u.d_two = nullptr;
     u.d_tw = nullptr;
     u.d_frag = nullptr;
     u.d_blocks = nullptr;
@@ -409,6 +422,19 @@ int upload(T** dst, const T* src, size_t count) {
 // grids by their own index (no map).  Local grids are scheduled largest
 // edge first.
 int finish_unit(fft3d_plan p, Unit& u, bool identity) {
+  if (u.two.launch) {
+    std::vector<float2> tab;
+    int rc = two_pass_prepare(u.two, p->dims[u.grids[0]], u.two_args, tab);
+    if (!rc) rc = upload(&u.d_two, tab.data(), tab.size());
+    if (!rc && !identity) rc = upload(&u.d_map, u.grids.data(), u.grids.size());
+    u.two_args.tx = u.d_two;
+    u.two_args.tzg = u.d_two + tab.size() / 2;
+    u.two_args.scale = p->scale;
+    u.two_args.do_scale = p->do_scale;
+    u.two_args.off = p->d_off;
+    u.two_args.map = u.d_map;
+    return rc;
+  }
   cudaError_t e = cudaFuncSetAttribute(u.kernel.func, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)u.kernel.smem);
   if (e == cudaSuccess && u.use_maps)
@@ -538,8 +564,23 @@ int launch_general(fft3d_plan p, const float2* in, float2* out, cudaStream_t str
   return FFT3D_SUCCESS;
 }
 
-int launch_unit(fft3d_plan p, const Unit& u, const float2* in, float2* out,
+// Grids [first, first + count) of a unit (a unit of a ticket kernel: all).
+int launch_unit(fft3d_plan p, const Unit& u, int first, int count, const float2* in, float2* out,
                 const float2* const* in_ptrs, float2* const* out_ptrs, cudaStream_t stream) {
+  if (u.two.launch) {
+    TwoPassArgs a = u.two_args;
+    a.in = in;
+    a.out = out;
+    a.in_ptrs = in_ptrs;
+    a.out_ptrs = out_ptrs;
+    a.first = first;
+    // (whether pointer arrays overlap is known on the device only)
+    if (u.two.launch(a, count, in_ptrs || in == out, stream) != cudaSuccess) {
+      cudaGetLastError();
+      return FFT3D_ERR_CUDA;
+    }
+    return FFT3D_SUCCESS;
+  }
   {
     // ticket kernels start from zeroed counters; cluster and whole-grid
     // kernels use none
@@ -581,30 +622,31 @@ int launch(fft3d_plan p, const float2* in, float2* out, const float2* const* in_
            float2* const* out_ptrs, cudaStream_t stream) {
   if (p->general) return launch_general(p, in, out, stream);
   const std::vector<Unit>& units = in_ptrs && !p->units_ptr.empty() ? p->units_ptr : p->units;
+  int rc = FFT3D_SUCCESS;
+  if (!p->mixed) return launch_unit(p, units[0], 0, p->batch, in, out, nullptr, nullptr, stream);
   if (!p->branches) {
-    for (const Unit& u : units) {
-      const int rc = launch_unit(p, u, in, out, in_ptrs, out_ptrs, stream);
-      if (rc) return rc;
-    }
+    for (const MixedStep& t : p->steps)
+      if ((rc = launch_unit(p, units[t.unit], t.first, t.count, in, out, in_ptrs, out_ptrs, stream)))
+        return rc;
     return FFT3D_SUCCESS;
   }
   // two concurrent branches, the caller's stream and a side stream forked
-  // from it: the units alternate between them, smallest first, so that one
-  // branch's launch drains while the other's runs; a captured graph records
-  // the fork and join as edges.  (A side stream per edge, six on the 64-grid
-  // workload, ran it in 540 us when its plans were the only ones and in 663
-  // with two more pairs of plans alive, whose streams share the device's
-  // queues; one branch 569, two 495, three 520, four 514 us, largest first
-  // 510.)
-  int rc = FFT3D_SUCCESS;
+  // from it, so that one branch's launch drains while the other's runs; a
+  // captured graph records the fork and join as edges.  (A side stream per
+  // edge, six on the 64-grid workload, ran its forward and inverse in 540 us
+  // when these plans were the only ones and in 663 with two more pairs alive,
+  // whose streams share the device's queues; one branch 569, two 495, three
+  // 520, four 514 us; two with the two-pass kernels 431.)
   if (cudaEventRecord(p->fork, stream) != cudaSuccess ||
       cudaStreamWaitEvent(p->side, p->fork, 0) != cudaSuccess) {
     cudaGetLastError();
     return FFT3D_ERR_CUDA;
   }
-  for (size_t i = 0; i < units.size() && !rc; ++i)
-    rc = launch_unit(p, units[units.size() - 1 - i], in, out, in_ptrs, out_ptrs,
-                     i & 1 ? p->side : stream);
+  for (size_t i = 0; i < p->steps.size() && !rc; ++i) {
+    const MixedStep& t = p->steps[i];
+    rc = launch_unit(p, units[t.unit], t.first, t.count, in, out, in_ptrs, out_ptrs,
+                     t.branch ? p->side : stream);
+  }
   // the side stream is joined even when a launch failed: the caller's stream
   // then still waits for what was launched there, and a capture does not end
   // with an unjoined stream
@@ -734,13 +776,21 @@ int create_mixed(int count, const int* dims, int direction, int norm, int varian
       Unit u;
       for (int g = 0; g < count; ++g)
         if (p->dims[g] == n) u.grids.push_back(g);
-      // the edge's kernel (unit_variant).  The tensor-map kernels read a packed
+      // the two-pass kernels where they are the default of so many grids, else
+      // the edge's kernel from unit_variant.  The tensor-map kernels read a packed
       // batch: at 128^3 the split-y kernel (6) takes one pair of tensor maps
       // per grid with the launch (up to kMixMaps grids) on packed buffers,
       // and calls with pointer arrays use the warp-owned kernel (5) in a
       // unit of their own; at 64^3 no tensor-map kernel is used,
       // the plain persistent ones are as fast at a mixed batch's grid counts
       const int ng = (int)u.grids.size();
+      if (builtin_default_variant(false, n, ng, FFT3D_FP32) == kGeneralVariant)
+        u.two = two_pass_apart_kernel_info(n, direction);
+      if (u.two.launch) {
+        p->units.push_back(u);
+        ptr_units.push_back(u);
+        continue;
+      }
       int v = unit_variant(n, ng);
       // the tensor-map kernels with per-grid maps: split-y (128^3) and the
       // thread-pair kernel (80^3, 96^3); for pointer arrays a kernel that
@@ -761,7 +811,30 @@ int create_mixed(int count, const int* dims, int direction, int norm, int varian
     }
     if (any_maps) p->units_ptr = ptr_units;
   }
-  if (variant == 2 && p->units.size() > 1) {
+  // the launches: two-pass units in runs of grids whose intermediates take 30%
+  // of L2, the others whole, largest edges first, each on the branch with
+  // fewer bytes so far
+  int l2_bytes = 0;
+  if (cudaDeviceGetAttribute(&l2_bytes, cudaDevAttrL2CacheSize, p->device) != cudaSuccess) {
+    cudaGetLastError();
+    delete p;
+    return FFT3D_ERR_CUDA;
+  }
+  double load[2] = {0.0, 0.0};
+  for (size_t i = 0; i < p->units.size(); ++i) {
+    const Unit& u = p->units[i];
+    const int ng = (int)u.grids.size();
+    double bytes = 0.0;
+    for (int g : u.grids) bytes += 8.0 * p->dims[g] * p->dims[g] * p->dims[g];
+    const int runs = u.two.launch ? std::min(ng, (int)std::ceil(bytes / (0.3 * l2_bytes))) : 1;
+    const int per = (ng + runs - 1) / runs;
+    for (int f = 0; f < ng; f += per) {
+      const int m = std::min(per, ng - f), b = variant == 2 && load[1] < load[0];
+      p->steps.push_back(MixedStep{(int)i, f, m, b});
+      load[b] += bytes * m / ng;
+    }
+  }
+  if (variant == 2 && p->steps.size() > 1) {
     p->branches = true;
     if (cudaEventCreateWithFlags(&p->fork, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&p->join, cudaEventDisableTiming) != cudaSuccess ||

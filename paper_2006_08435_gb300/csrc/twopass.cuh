@@ -119,18 +119,42 @@ struct Dims : Cfg<L> {
   static constexpr size_t smem2 = sizeof(float2) * (size_t)C::BZ * ZP;
 };
 
-template <int L, int DIR, bool INPLACE>
+// Where grid g of a launch lies (plan data first: it may be read before the
+// launch it depends on is done; the callers' pointer arrays may not).
+template <bool APART>
+struct GridAt {
+  size_t off;
+  int pg;
+  __device__ __forceinline__ GridAt(const TwoPassArgs& a, unsigned g, size_t points)
+      : off(g * points), pg(0) {
+    if constexpr (APART) {
+      pg = a.first + (int)g;
+      if (a.map) pg = a.map[pg];
+      off = (size_t)a.off[pg];
+    }
+  }
+  __device__ __forceinline__ const float2* in(const TwoPassArgs& a) const {
+    return APART && a.in_ptrs ? a.in_ptrs[pg] : a.in + off;
+  }
+  __device__ __forceinline__ float2* out(const TwoPassArgs& a) const {
+    return APART && a.out_ptrs ? a.out_ptrs[pg] : a.out + off;
+  }
+};
+
+template <int L, int DIR, bool INPLACE, bool APART>
 __global__ void __launch_bounds__(Dims<L>::T1) pass1_kernel(const __grid_constant__ TwoPassArgs a) {
   using D = Dims<L>;
   constexpr int A = D::A, B = D::B, AX = D::AX, BX = D::BX, T = D::T1;
   extern __shared__ __align__(16) float2 sm[];
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const unsigned zz = blockIdx.x / A;  // plane
+  const unsigned zz = blockIdx.x / A, g = zz / L;  // plane, grid
   const int n1 = (int)(blockIdx.x - zz * A);
   const uint64_t once = l2_policy(kEvictFirst), keep = l2_policy(kEvictLast);
-  const float2* src = a.in + (size_t)zz * L * L + (size_t)n1 * L;
-  float2* dst = a.out + (size_t)zz * L * L + (size_t)n1 * B * L;
+  const GridAt<APART> at(a, g, (size_t)L * L * L);
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  const size_t plane = (size_t)(zz - g * L) * L * L;
+  const float2* src = at.in(a) + plane + (size_t)n1 * L;
+  float2* dst = at.out(a) + plane + (size_t)n1 * B * L;
   // x, first step: item (row j, m) -> points m + AX i
   constexpr int N1 = B * AX;
 #pragma unroll 1
@@ -188,7 +212,7 @@ __global__ void __launch_bounds__(Dims<L>::T1) pass1_kernel(const __grid_constan
   }
 }
 
-template <int L, int DIR>
+template <int L, int DIR, bool APART>
 __global__ void __launch_bounds__(Dims<L>::T2) pass2_kernel(const __grid_constant__ TwoPassArgs a) {
   using D = Dims<L>;
   constexpr int A = D::A, B = D::B, AZ = D::AZ, BZ = D::BZ, W = D::W, T = D::T2;
@@ -198,8 +222,9 @@ __global__ void __launch_bounds__(Dims<L>::T2) pass2_kernel(const __grid_constan
   const unsigned xt = blockIdx.x % (L / W), r = blockIdx.x / (L / W);
   const unsigned k2 = r % B, g = r / B;
   const uint64_t once = l2_policy(kEvictFirst);
-  float2* base = a.out + (long long)g * LL * L + (long long)k2 * L + xt * W;
+  const GridAt<APART> at(a, g, (size_t)LL * L);
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  float2* base = at.out(a) + (long long)k2 * L + xt * W;
   // z, first step: item (m1, n1, q) -> planes m1 + AZ i
   constexpr int N1 = W * A * AZ;
 #pragma unroll 1
@@ -247,8 +272,8 @@ __global__ void __launch_bounds__(Dims<L>::T2) pass2_kernel(const __grid_constan
   }
 }
 
-template <int L, int DIR>
-cudaError_t launch(const TwoPassArgs& a, int grids, int which, cudaStream_t s) {
+template <int L, int DIR, bool APART>
+cudaError_t launch(const TwoPassArgs& a, int grids, bool in_place, cudaStream_t s) {
   using D = Dims<L>;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[2];
@@ -261,28 +286,28 @@ cudaError_t launch(const TwoPassArgs& a, int grids, int which, cudaStream_t s) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   cfg.stream = s;
-  if (which == 1) {
-    cfg.gridDim = dim3((unsigned)grids * L * D::A, 1, 1);
-    cfg.blockDim = dim3(D::T1, 1, 1);
-    cfg.dynamicSmemBytes = D::smem1;
-    if (a.in != a.out) return cudaLaunchKernelEx(&cfg, &pass1_kernel<L, DIR, false>, a);
-    cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, &pass1_kernel<L, DIR, true>, a);
-  }
+  cfg.gridDim = dim3((unsigned)grids * L * D::A, 1, 1);
+  cfg.blockDim = dim3(D::T1, 1, 1);
+  cfg.dynamicSmemBytes = D::smem1;
+  cfg.numAttrs = in_place ? 2 : 1;
+  const cudaError_t e = in_place ? cudaLaunchKernelEx(&cfg, &pass1_kernel<L, DIR, true, APART>, a)
+                                 : cudaLaunchKernelEx(&cfg, &pass1_kernel<L, DIR, false, APART>, a);
+  if (e != cudaSuccess) return e;
+  cfg.numAttrs = 1;
   cfg.gridDim = dim3((unsigned)grids * D::B * (L / D::W), 1, 1);
   cfg.blockDim = dim3(D::T2, 1, 1);
   cfg.dynamicSmemBytes = D::smem2;
-  return cudaLaunchKernelEx(&cfg, &pass2_kernel<L, DIR>, a);
+  return cudaLaunchKernelEx(&cfg, &pass2_kernel<L, DIR, APART>, a);
 }
 
-template <int L, int DIR>
+template <int L, int DIR, bool APART>
 TwoPassKernel entry() {
   using D = Dims<L>;
   TwoPassKernel k;
-  k.launch = &launch<L, DIR>;
-  k.func[0] = (const void*)&pass1_kernel<L, DIR, false>;
-  k.func[1] = (const void*)&pass1_kernel<L, DIR, true>;
-  k.func[2] = (const void*)&pass2_kernel<L, DIR>;
+  k.launch = &launch<L, DIR, APART>;
+  k.func[0] = (const void*)&pass1_kernel<L, DIR, false, APART>;
+  k.func[1] = (const void*)&pass1_kernel<L, DIR, true, APART>;
+  k.func[2] = (const void*)&pass2_kernel<L, DIR, APART>;
   k.smem[0] = k.smem[1] = D::smem1;
   k.smem[2] = D::smem2;
   k.A = D::A;
@@ -290,9 +315,9 @@ TwoPassKernel entry() {
   k.AZ = D::AZ;
   return k;
 }
-template <int L>
+template <int L, bool APART>
 TwoPassKernel entry_of(int dir) {
-  return dir < 0 ? entry<L, -1>() : entry<L, 1>();
+  return dir < 0 ? entry<L, -1, APART>() : entry<L, 1, APART>();
 }
 
 }  // namespace tp
