@@ -125,7 +125,7 @@ PencilKernel pencil_kernel_info(int L, int dir, int kind);
 
 // Two-pass transforms of cubic edges (twopass.cuh).  tx, ty, tz: W_L^(n1 k) at
 // [k * split + n1] for the splits AX, A and AZ.
-constexpr int kTwoPassMaxLen = 160;
+constexpr int kTwoPassMaxLen = 192;  // = 6 * 32: ny = A B of a box
 struct TwoPassArgs {
   const float2* in;  // may equal out
   float2* out;
@@ -155,6 +155,29 @@ TwoPassKernel two_pass_apart_kernel_info(int L, int dir);  // for mixed-edge pla
 // entries: a.tx and a.tzg are set once tab is on the device).
 int two_pass_prepare(const TwoPassKernel& k, int L, TwoPassArgs& a, std::vector<float2>& tab);
 
+// Two-pass transforms of boxes (twopass_box.cuh): ny = A B.
+struct BoxArgs {
+  const float2* in;
+  float2* out;
+  int in_place;  // out == in: pass 1 runs in clusters of A blocks
+  const float2 *tx, *tzg;
+  float2 ty[kTwoPassMaxLen], tz[kTwoPassMaxLen];
+  int A, B, nx, xtiles;
+  FastDiv divA, divB, divxt;
+  float scale;
+  int do_scale;
+};
+struct BoxKernel {
+  const void* func = nullptr;
+  int threads = 0;
+  size_t smem = 0;  // pass 1: per row
+  int split = 0;    // AX or AZ
+};
+BoxKernel box1_kernel_info(int nx, int dir);         // func null: none
+BoxKernel box2_kernel_info(int A, int nz, int dir);
+cudaError_t launch_box(const BoxKernel& k, unsigned grid, size_t smem, int cluster, const BoxArgs& a,
+                       cudaStream_t s);
+
 // A 3D transform as three pencil passes (passes.cu): complex grids (x, y, z,
 // out of place or in place; as two passes at some cubic edges unless `fixed`), real grids to half spectra (x, y, z) or back
 // (z into a workspace of work_points() complex points, y, x).
@@ -168,6 +191,8 @@ struct AxisPasses {
   PencilKernel k[3];
   TwoPassKernel two;    // launch not null: two passes instead
   TwoPassArgs two_args;
+  BoxKernel box[2];     // func not null: two passes of a box
+  BoxArgs box_args;
   int chains = 1;       // streams the chunks alternate between
   cudaStream_t side = nullptr;
   cudaEvent_t fork = nullptr, join = nullptr;

@@ -95,6 +95,51 @@ int AxisPasses::create(PassKind kind_, int nx_, int ny_, int nz_, int batch_, in
     two_args.scale = scale;
     two_args.do_scale = do_scale;
   }
+  // a box: ny = A B with B points per thread, A as small as it goes
+  box[0] = box[1] = BoxKernel{};
+  if (kind == kPassC2C && !two.launch && !fixed) {
+    int A = 0;
+    static_assert(6 * 32 <= kTwoPassMaxLen, "ny = A B");
+    const int radices[] = {32, 30, 27, 25, 24, 20, 18, 16, 15, 12, 10};
+    for (int B : radices)
+      if (!A && ny % B == 0 && ny / B >= 2 && ny / B <= 6) A = ny / B;
+    // enough blocks in one grid to fill the GPU, of enough points (45 x 75 x 50,
+    // 150 blocks: 2 grids 13.0 us, three passes 8.6, though 40 grids 40.5 and
+    // 46.0; 36^3, rows of 18 * 36 points: 68 us for 200 grids, three passes 54).
+    // The batch has no say: a grid's bits are the same alone and in a batch.
+    if (A && (nz * A < 220 || ny / A * nx < 800)) A = 0;
+    if (A) {
+      box[0] = box1_kernel_info(nx, dir);
+      box[1] = box2_kernel_info(A, nz, dir);
+    }
+    const size_t smem1 = A ? box[0].smem * (size_t)(ny / A) : 0;
+    if (!box[0].func || !box[1].func || smem1 > 72 * 1024) {
+      box[0] = box[1] = BoxKernel{};
+    } else {
+      for (int i = 0; i < 2; ++i)
+        if (cudaFuncSetAttribute(box[i].func, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(i ? box[1].smem : smem1)) != cudaSuccess) {
+          cudaGetLastError();
+          return FFT3D_ERR_CUDA;
+        }
+      BoxArgs& b = box_args;
+      b = BoxArgs{};
+      b.A = A;
+      b.B = ny / A;
+      b.nx = nx;
+      b.xtiles = (nx + 15) / 16;
+      b.divA = make_fastdiv((unsigned)b.A);
+      b.divB = make_fastdiv((unsigned)b.B);
+      b.divxt = make_fastdiv((unsigned)b.xtiles);
+      b.scale = scale;
+      b.do_scale = do_scale;
+      for (int i = 0; i < ny; ++i) b.ty[i] = root((long long)(i / A) * (i % A), ny);
+      const int ax = box[0].split, az = box[1].split;
+      for (int i = 0; i < nz; ++i) b.tz[i] = root((long long)(i / az) * (i % az), nz);
+      for (int i = 0; i < nx; ++i) tab.push_back(root((long long)(i / ax) * (i % ax), nx));
+      tab.insert(tab.end(), b.tz, b.tz + nz);
+    }
+  }
   for (int a = 0; a < 3 && !two.launch; ++a) {
     k[a] = pencil_kernel_info(len[a], dir, a == 0 ? kx : 0);
     if (!k[a].launch) return FFT3D_ERR_UNSUPPORTED_SIZE;
@@ -128,6 +173,8 @@ int AxisPasses::create(PassKind kind_, int nx_, int ny_, int nz_, int batch_, in
   twr = d_tab + off_r;
   two_args.tx = d_tab;
   two_args.tzg = d_tab + nx;
+  box_args.tx = d_tab;
+  box_args.tzg = d_tab + nx;
 
   // Chunk budget: the intermediates of the chunks in flight within 40% of L2
   // (complex grids: 96 x 128 x 64 x 64 261 us, 60%: 270), 60% for real
@@ -140,7 +187,7 @@ int AxisPasses::create(PassKind kind_, int nx_, int ny_, int nz_, int batch_, in
   const double plane_bytes = 8.0 * (double)pp, grid_bytes = plane_bytes * nz;
   const double l2 = (double)l2_bytes;
   chains = batch >= 2 && grid_bytes * batch > 40.0 * 1048576.0 ? kMaxChains : 1;
-  const double budget = (kind == kPassC2C && !two.launch ? 0.4 : 0.6) * l2 / chains;
+  const double budget = (kind == kPassC2C && !two.launch && !box[0].func ? 0.4 : 0.6) * l2 / chains;
   // a pass's pencils stay below 2^31
   const long long most = std::max({(long long)ny * nz, (long long)nz * hx, pp});
   const long long cap = std::max(1LL, (1LL << 30) / most);
@@ -237,6 +284,18 @@ cudaError_t AxisPasses::chunk_passes(long long g, const void* in, void* out, flo
     a.pol_out = kind == kPassC2R ? kEvictLast : kEvictFirst;
     return k[2].launch(a, s);
   };
+  if (box[0].func) {
+    const long long m = std::min(chunk, batch - g);
+    BoxArgs a = box_args;
+    a.in = static_cast<const float2*>(in) + g * pp * nz;
+    a.out = static_cast<float2*>(out) + g * pp * nz;
+    a.in_place = in == out;
+    const cudaError_t e = launch_box(box[0], (unsigned)(m * nz * a.A), box[0].smem * a.B,
+                                     a.in_place ? a.A : 1, a, s);
+    return e != cudaSuccess
+               ? e
+               : launch_box(box[1], (unsigned)(m * a.B * a.xtiles), box[1].smem, 1, a, s);
+  }
   // complex points of one grid on the x pass's two sides
   const long long real_pts = (long long)nx / 2 * ny * nz, spec_pts = pp * nz;
   const long long m = std::min(chunk, batch - g);

@@ -52,3 +52,24 @@ def test_two_chains_equal_one_grid_at_a_time(cuda, monkeypatch, n, batch):
         y.copy_(x)
         p.execute(y, y)
         assert torch.equal(y, ref)
+
+
+@pytest.mark.parametrize("shape,batch", [((64, 128, 96), 4), ((50, 75, 45), 6), ((45, 100, 32), 5),
+                                         ((80, 96, 128), 3), ((90, 120, 135), 2), ((40, 36, 160), 9),
+                                         ((75, 75, 75), 3), ((60, 162, 54), 5), ((128, 64, 50), 4)])
+@pytest.mark.parametrize("inverse", [False, True])
+def test_boxes_against_oracle(cuda, shape, batch, inverse):
+    """Boxes on the two-pass kernels: run-time y steps, x tiles cut off at the
+    edge, and the in-place form."""
+    from paper_2006_08435_gb300 import Plan
+    nz, ny, nx = shape
+    x = torch.from_numpy(synth.uniform_grids(shape, batch, seed=sum(shape))).cuda()
+    p = Plan(nx, ny, nz, batch, inverse=inverse, norm="ortho")
+    y = torch.empty_like(x)
+    p.execute(x, y)
+    for b in (0, batch - 1):
+        ref = oracle.dft3d(x[b].cpu().numpy().astype(np.complex128), 1 if inverse else -1)
+        assert oracle.rel_l2(y[b].cpu().numpy(), ref / np.sqrt(nx * ny * nz)) <= TOL
+    z = x.clone()
+    p.execute(z, z)
+    assert torch.equal(z, y)
