@@ -493,6 +493,19 @@ int fft3d_real_plan_create_fixed(int n, int batch, fft3d_real_plan* out_plan);
  */
 int fft3d_real_execute(fft3d_real_plan plan, const void* in, void* out, void* stream);
 
+/*
+ * The gradient of the Hartree energies in one step: what fft3d_hartree_seed_half
+ * (rhohat_half, n, batch, L, grad_energy, seed) and fft3d_real_execute(plan,
+ * seed, out) give together, without the seed's own pass and buffer: the inverse
+ * transform weights the half spectra as it reads them.  plan: an inverse plan
+ * of norm FFT3D_NORM_NONE; grad_energy: DEVICE array of `batch` doubles.
+ * Pointers, streams and capture as fft3d_real_execute.  Errors:
+ * FFT3D_ERR_INVALID_ARG (another plan, L not positive and finite),
+ * FFT3D_ERR_UNSUPPORTED_PRECISION (a plan of the pair scheme: take the two steps).
+ */
+int fft3d_real_execute_hartree(fft3d_real_plan plan, const void* rhohat_half, double L,
+                               const double* grad_energy, void* out, void* stream);
+
 /* As fft3d_get_device_status, for the plan's complex transform. */
 int fft3d_real_get_device_status(fft3d_real_plan plan, void* stream);
 

@@ -67,6 +67,7 @@ _SIGS = {
                                    ctypes.POINTER(_I), ctypes.POINTER(_I)]),
     "fft3d_real_plan_create": (_I, [_I, _I, _I, _I, _I, ctypes.POINTER(_VP)]),
     "fft3d_real_plan_create_fixed": (_I, [_I, _I, ctypes.POINTER(_VP)]),
+    "fft3d_real_execute_hartree": (_I, [_VP, _VP, ctypes.c_double, _VP, _VP, _VP]),
     "fft3d_real_execute": (_I, [_VP, _VP, _VP, _VP]),
     "fft3d_real_get_device_status": (_I, [_VP, _VP]),
     "fft3d_real_plan_destroy": (_I, [_VP]),

@@ -23,6 +23,7 @@
 #include <cstdint>
 
 #include "fft3d.h"
+#include "hartree.cuh"
 #include "internal.h"
 
 namespace fft3d {
@@ -33,17 +34,6 @@ constexpr int kRedThreads = 256;
 __host__ __device__ inline int energy_blocks(long long npts) {
   long long b = (npts + kRedThreads * 8 - 1) / (kRedThreads * 8);
   return (int)(b < 1 ? 1 : (b > 512 ? 512 : b));
-}
-
-__device__ __forceinline__ int signed_index(int k, int n) { return k < (n + 1) / 2 ? k : k - n; }
-
-// 1 / x by the hardware's approximate reciprocal (within 1 ulp by the PTX
-// ISA's bound; the callers' x = |m|^2 is a positive integer below 2^24,
-// exact in FP32).
-__device__ __forceinline__ float rcp_approx(float x) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
 }
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -216,7 +206,9 @@ int grid_for(long long count, int threads) {
   return (int)(b < 1 ? 1 : (b > 152 * 16 ? 152 * 16 : b));
 }
 
-bool valid_grid(int n, int batch, double L) {
+}  // namespace
+
+bool hartree_valid(int n, int batch, double L) {
   return n >= 2 && n <= 1024 && batch >= 1 && batch <= 65535 && L > 0.0 && std::isfinite(L);
 }
 
@@ -226,7 +218,6 @@ double hartree_s(int n, double L) {
   return L * L * L * 4.0 * 3.14159265358979323846 / (n3 * n3 * g * g);
 }
 
-}  // namespace
 }  // namespace fft3d
 
 using namespace fft3d;
@@ -248,7 +239,7 @@ template <bool HALF>
 int energy_impl(const void* rhohat, int n, int batch, double L, double* energy, void* workspace,
                 size_t workspace_bytes, void* stream) {
   if (!rhohat || !energy || !workspace) return FFT3D_ERR_NULL_PTR;
-  if (!valid_grid(n, batch, L) || (HALF && (n & 1))) return FFT3D_ERR_INVALID_ARG;
+  if (!hartree_valid(n, batch, L) || (HALF && (n & 1))) return FFT3D_ERR_INVALID_ARG;
   if (workspace_bytes < fft3d_hartree_workspace_bytes(n, batch)) return FFT3D_ERR_INVALID_ARG;
   if (reinterpret_cast<uintptr_t>(rhohat) & 7u || reinterpret_cast<uintptr_t>(workspace) & 7u)
     return FFT3D_ERR_MISALIGNED;
@@ -279,7 +270,7 @@ template <bool HALF>
 int seed_impl(const void* rhohat, int n, int batch, double L, const double* grad_energy,
               void* seed, void* stream) {
   if (!rhohat || !grad_energy || !seed) return FFT3D_ERR_NULL_PTR;
-  if (!valid_grid(n, batch, L) || (HALF && (n & 1))) return FFT3D_ERR_INVALID_ARG;
+  if (!hartree_valid(n, batch, L) || (HALF && (n & 1))) return FFT3D_ERR_INVALID_ARG;
   if (reinterpret_cast<uintptr_t>(rhohat) & 7u || reinterpret_cast<uintptr_t>(seed) & 7u)
     return FFT3D_ERR_MISALIGNED;
   const long long npts = (long long)n * n * (HALF ? n / 2 + 1 : n);

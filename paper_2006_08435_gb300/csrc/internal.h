@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "fft3d.h"
+#include "hartree.cuh"
 
 namespace fft3d {
 
@@ -48,6 +49,7 @@ struct FusedArgs {
   long long timeout_ns;
   const uint32_t* mma_frag;     // tensor-core B fragments (split precisions), or null
   int ngrids;                   // grids of the launch unit
+  HartreeWeight weight;         // real inverse kernels launched by launch_weighted
   float2* aux;                  // a kernel's own workspace (real grids: Nyquist columns), or null
 };
 
@@ -76,6 +78,8 @@ struct KernelInfo {
   int uses_work = 1;            // 0: no ticket counters (nothing to clear before a launch)
   LaunchMapsFn launch_maps = nullptr;  // mixed-edge units on packed buffers (tensor-map kernels)
   const void* func_maps = nullptr;     // its kernel
+  LaunchFn launch_weighted = nullptr;  // real inverse kernels: the input times FusedArgs::weight
+  const void* func_weighted = nullptr;
 };
 
 // ---------------------------------------------------------------- general path
@@ -112,6 +116,10 @@ struct PencilArgs {
   float scale;
   int do_scale;
   int pol_in, pol_out;  // L2 policies of the loads and the stores
+  // weighted kind: spectra of n^3 grids, rows of hx points, times weight / |m|^2
+  HartreeWeight weight;
+  FastDiv divh;  // by hx
+  int n, hx;
 };
 struct PencilKernel {
   cudaError_t (*launch)(const PencilArgs&, cudaStream_t) = nullptr;
@@ -120,7 +128,7 @@ struct PencilKernel {
   size_t smem = 0;
 };
 // kind: 0 strided, 1 rows, 2 real rows of 2 L points forward (dir -1), 3 the
-// same inverse (dir 1); launch is null for an edge that is not plannable.
+// same inverse (dir 1), 4 strided with weights (dir 1, even L); launch is null for an edge that is not plannable.
 PencilKernel pencil_kernel_info(int L, int dir, int kind);
 
 // Two-pass transforms of cubic edges (twopass.cuh).  tx, ty, tz: W_L^(n1 k) at
@@ -189,6 +197,7 @@ struct AxisPasses {
   long long chunk = 0;  // grids per chunk
   long long sub = 0;    // planes per launch of the x and y passes
   PencilKernel k[3];
+  PencilKernel kw;      // kPassC2R: the z pass with weights
   TwoPassKernel two;    // launch not null: two passes instead
   TwoPassArgs two_args;
   BoxKernel box[2];     // func not null: two passes of a box
@@ -206,9 +215,11 @@ struct AxisPasses {
              int l2_bytes, bool fixed = false);
   void destroy();
   long long work_points() const;
-  cudaError_t execute(const void* in, void* out, float2* work, cudaStream_t s) const;
-  cudaError_t chunk_passes(long long g, const void* in, void* out, float2* work,
-                           cudaStream_t s) const;
+  // weight (kPassC2R): the input times it, or null
+  cudaError_t execute(const void* in, void* out, float2* work, cudaStream_t s,
+                      const HartreeWeight* weight = nullptr) const;
+  cudaError_t chunk_passes(long long g, const void* in, void* out, float2* work, cudaStream_t s,
+                           const HartreeWeight* weight) const;
 };
 
 // Defined in the inst_*.cu translation units.

@@ -155,6 +155,16 @@ int AxisPasses::create(PassKind kind_, int nx_, int ny_, int nz_, int batch_, in
       for (int k2 = 0; k2 < B; ++k2)
         for (int n1 = 0; n1 < A; ++n1) tab.push_back(root((long long)n1 * k2, len[a]));
   }
+  kw = PencilKernel{};
+  if (kind == kPassC2R) {
+    kw = pencil_kernel_info(nz, dir, 4);
+    if (kw.launch && kw.smem > 48 * 1024 &&
+        cudaFuncSetAttribute(kw.func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kw.smem) !=
+            cudaSuccess) {
+      cudaGetLastError();
+      return FFT3D_ERR_CUDA;
+    }
+  }
   off_r = tab.size();
   if (kind != kPassC2C)
     for (int m = 0; m <= lx; ++m) tab.push_back(root(m, nx));
@@ -229,7 +239,7 @@ long long AxisPasses::work_points() const { return chains * chunk * hx * ny * nz
 
 // The passes of grids g .. g + chunk - 1 (work: one chunk of spectra, kPassC2R).
 cudaError_t AxisPasses::chunk_passes(long long g, const void* in, void* out, float2* work,
-                                     cudaStream_t s) const {
+                                     cudaStream_t s, const HartreeWeight* weight) const {
   const long long pp = (long long)hx * ny;  // complex points of a plane
   if (two.launch) {
     const long long m = std::min(chunk, batch - g);
@@ -282,6 +292,14 @@ cudaError_t AxisPasses::chunk_passes(long long g, const void* in, void* out, flo
     a.do_scale = kind != kPassC2R && do_scale;
     a.pol_in = kEvictFirst;
     a.pol_out = kind == kPassC2R ? kEvictLast : kEvictFirst;
+    if (weight) {
+      a.weight = *weight;
+      a.weight.grad += g;
+      a.n = nz;
+      a.hx = hx;
+      a.divh = make_fastdiv((unsigned)hx);
+      return kw.launch(a, s);
+    }
     return k[2].launch(a, s);
   };
   if (box[0].func) {
@@ -325,11 +343,12 @@ cudaError_t AxisPasses::chunk_passes(long long g, const void* in, void* out, flo
   return cudaSuccess;
 }
 
-cudaError_t AxisPasses::execute(const void* in, void* out, float2* work, cudaStream_t s) const {
+cudaError_t AxisPasses::execute(const void* in, void* out, float2* work, cudaStream_t s,
+                                const HartreeWeight* weight) const {
   cudaError_t e = cudaSuccess;
   if (chains == 1) {
     for (long long g = 0; g < batch && e == cudaSuccess; g += chunk)
-      e = chunk_passes(g, in, out, work, s);
+      e = chunk_passes(g, in, out, work, s, weight);
     return e;
   }
   // the events are recorded and waited for under a lock: executes of one
@@ -339,7 +358,7 @@ cudaError_t AxisPasses::execute(const void* in, void* out, float2* work, cudaStr
   if ((e = cudaStreamWaitEvent(side, fork, 0)) != cudaSuccess) return e;
   int c = 0;
   for (long long g = 0; g < batch && e == cudaSuccess; g += chunk, c ^= 1)
-    e = chunk_passes(g, in, out, work && c ? work + chunk * hx * ny * nz : work, c ? side : s);
+    e = chunk_passes(g, in, out, work && c ? work + chunk * hx * ny * nz : work, c ? side : s, weight);
   // the side stream is joined even when a launch failed
   cudaError_t j = cudaEventRecord(join, side);
   if (j == cudaSuccess) j = cudaStreamWaitEvent(s, join, 0);

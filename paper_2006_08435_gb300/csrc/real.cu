@@ -228,7 +228,10 @@ int create_fused_real(int n, int batch, int direction, int norm, const KernelInf
   }
   if (major != 10 || minor != 3) return FFT3D_ERR_NO_DEVICE;
   if (cudaFuncSetAttribute(k.func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem) !=
-      cudaSuccess) {
+          cudaSuccess ||
+      (k.func_weighted &&
+       cudaFuncSetAttribute(k.func_weighted, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                            (int)k.smem) != cudaSuccess)) {
     cudaGetLastError();
     return FFT3D_ERR_CUDA;
   }
@@ -338,7 +341,8 @@ int create_pencil_real(int n, int batch, int direction, int norm, fft3d_real_pla
   return FFT3D_SUCCESS;
 }
 
-int execute_fused_real(fft3d_real_plan p, const void* in, void* out, cudaStream_t s) {
+int execute_fused_real(fft3d_real_plan p, const void* in, void* out, cudaStream_t s,
+                       const HartreeWeight* weight = nullptr) {
   if (p->kern.uses_work &&
       cudaMemsetAsync(p->d_count, 0, sizeof(unsigned) * (size_t)(p->batch + 1), s) != cudaSuccess) {
     cudaGetLastError();
@@ -357,7 +361,8 @@ int execute_fused_real(fft3d_real_plan p, const void* in, void* out, cudaStream_
   a.timeout_ns = kDefaultWaitNs;
   a.ngrids = p->batch;
   a.aux = p->d_aux;
-  if (p->kern.launch(a, p->grid, s) != cudaSuccess) {
+  if (weight) a.weight = *weight;
+  if ((weight ? p->kern.launch_weighted : p->kern.launch)(a, p->grid, s) != cudaSuccess) {
     cudaGetLastError();
     return FFT3D_ERR_CUDA;
   }
@@ -436,15 +441,23 @@ int fft3d_real_plan_create_fixed(int n, int batch, fft3d_real_plan* out_plan) {
   const fft3d::KernelInfo k = fft3d::real_kernel_info(n, -1);
   if (k.launch && !pairs_only)
     return fft3d::create_fused_real(n, batch, FFT3D_FORWARD, FFT3D_NORM_NONE, k, out_plan);
-  // (a variant set in the environment or a tuning cache holds here too)
   const int pairs = (batch + 1) / 2;
   fft3d_plan inner = nullptr;
   int rc;
-  if (k.launch || std::getenv("FFT3D_VARIANT") || std::getenv("FFT3D_TUNE_CACHE"))
+  if (k.launch) {
     rc = fft3d_plan_create(n, n, n, pairs, FFT3D_FP32, FFT3D_FORWARD, FFT3D_NORM_NONE, &inner);
-  else
-    rc = fft3d_internal_create_variant(false, n, pairs, FFT3D_FP32, FFT3D_FORWARD, nullptr, 0,
-                                       fft3d::fixed_variant(n, pairs), &inner);
+  } else {
+    int v = fft3d::fixed_variant(n, pairs);
+    // a variant set in the environment or a tuning cache holds here too, but
+    // for the default's two passes, whose order is another
+    if (v != fft3d::kFixedVariant) {
+      const int picked =
+          fft3d::pick_variant(false, n, pairs, FFT3D_FP32, FFT3D_FORWARD, nullptr, 0);
+      if (picked != fft3d::kGeneralVariant) v = picked;
+    }
+    rc = fft3d_internal_create_variant(false, n, pairs, FFT3D_FP32, FFT3D_FORWARD, nullptr, 0, v,
+                                       &inner);
+  }
   return rc ? rc : fft3d::create_pair_real(n, batch, FFT3D_FORWARD, inner, out_plan);
 }
 
@@ -482,6 +495,27 @@ int fft3d_real_execute(fft3d_real_plan plan, const void* in, void* out, void* st
         pairs);
   }
   return cudaGetLastError() == cudaSuccess ? FFT3D_SUCCESS : FFT3D_ERR_CUDA;
+}
+
+int fft3d_real_execute_hartree(fft3d_real_plan plan, const void* rhohat_half, double L,
+                               const double* grad_energy, void* out, void* stream) {
+  using namespace fft3d;
+  if (!plan || !rhohat_half || !grad_energy || !out) return FFT3D_ERR_NULL_PTR;
+  if (plan->direction != FFT3D_INVERSE || plan->do_scale || !hartree_valid(plan->n, plan->batch, L))
+    return FFT3D_ERR_INVALID_ARG;
+  if (plan->inner) return FFT3D_ERR_UNSUPPORTED_PRECISION;  // the pair scheme
+  if (!aligned16(rhohat_half) || !aligned16(out)) return FFT3D_ERR_MISALIGNED;
+  HartreeWeight w;
+  w.grad = grad_energy;
+  w.s = hartree_s(plan->n, L);
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  if (plan->fused) return execute_fused_real(plan, rhohat_half, out, s, &w);
+  if (!plan->passes.kw.launch) return FFT3D_ERR_UNSUPPORTED_SIZE;
+  if (plan->passes.execute(rhohat_half, out, plan->d_work, s, &w) != cudaSuccess) {
+    cudaGetLastError();
+    return FFT3D_ERR_CUDA;
+  }
+  return FFT3D_SUCCESS;
 }
 
 int fft3d_real_get_device_status(fft3d_real_plan plan, void* stream) {

@@ -243,6 +243,35 @@ __device__ __forceinline__ void load_dif_rows(const unsigned char* t, int col, i
   else load_dif<N, DIR, 1>(at, v);
 }
 
+// The same with the points kz = r times scale / |m|^2, m = (., ., kz) with
+// mx^2 + my^2 = xy, or as they are (packed: column 0 holds two weighted columns).
+// r and H - r go together: their four points r, r + H, H - r, N - r have two
+// weights (kz and -kz have one), which halves the reciprocals.
+template <int N, int DIR, int HALF, class At>
+__device__ __forceinline__ void load_dif_weighted(At&& at, float xy, float scale, bool packed,
+                                                  float2* v) {
+  constexpr int H = N / 2;
+  auto weight = [&](int mz) {  // (xy >= 1 where not packed)
+    const float w = scale * rcp_approx(xy + (float)(mz * mz));
+    return packed ? 1.0f : w;
+  };
+  auto put = [&](auto R, float wa, float wb) {
+    constexpr int r = decltype(R)::value;
+    const float2 p = *at(r), q = *at(r + H);
+    const float2 a = make_float2(__fmul_rn(p.x, wa), __fmul_rn(p.y, wa));
+    const float2 b = make_float2(__fmul_rn(q.x, wb), __fmul_rn(q.y, wb));
+    if constexpr (HALF == 0) v[r] = cadd(a, b);
+    else v[r] = twc<r, N, DIR>(csub(a, b));
+  };
+  put(std::integral_constant<int, 0>{}, weight(0), weight(H));
+  static_for<1, H / 2 + 1>([&](auto R) {
+    constexpr int r = decltype(R)::value;
+    const float w = weight(r), wm = weight(H - r);
+    put(R, w, wm);
+    if constexpr (2 * r != H) put(std::integral_constant<int, H - r>{}, wm, w);
+  });
+}
+
 // --------------------------------------------------------------- producer
 // Lane 0 takes tickets (two ahead, so the atomic's round trip overlaps the
 // item before) and resolves them (schedule block by binary search over the
@@ -427,7 +456,12 @@ __device__ __forceinline__ void publisher(const FusedArgs& a, unsigned long long
 // floats x 1 x n), m1 = the real grids `in` (box 32 floats x n x 1,
 // swizzled); inverse m0 = the half spectra `in` as row pairs (box n + 4 x 1
 // x n), m1 = the same view with boxes of 4 floats (mirror columns).
-template <int N, int DIR>
+// WEIGHT (inverse): the half spectra times a.weight / |m|^2 as the z items read
+// them, which takes the seed's own pass over them (read and write, 85 us at
+// 128^3 x 32) away for the arithmetic of the weights in the z items (us, with
+// weights / without: 128^3 x 32 204.6 / 173.1, 64^3 x 128 91.0 / 88.8; Hartree
+// energies and gradients at 128^3 x 32 531.7 -> 482.0).
+template <int N, int DIR, bool WEIGHT>
 __global__ void __launch_bounds__(Cfg<N>::T, 1)
     rgrid_fft3d_kernel(const FusedArgs a, const __grid_constant__ CUtensorMap m0,
                        const __grid_constant__ CUtensorMap m1) {
@@ -506,6 +540,14 @@ __global__ void __launch_bounds__(Cfg<N>::T, 1)
     // the forward Nyquist item uses the threads of row 0 only
     const bool idle = DIR < 0 && pass == 3 && r != 0;
     bool fail = false;
+    float wscale = 0.0f, wxy = 0.0f;  // WEIGHT: of column c of row i0 + r
+    if constexpr (WEIGHT) {
+      if (pass == 0) {
+        const int my = signed_index(i0 + r, N);
+        wscale = (float)(a.weight.s * a.weight.grad[d.grid]);
+        wxy = (float)(c * c + my * my);
+      }
+    }
     if constexpr (DIR > 0) {
       if (pass == 0) {
         // rows (kz, ky = i0 + rs) of the input: columns 0 and H -> their
@@ -513,13 +555,20 @@ __global__ void __launch_bounds__(Cfg<N>::T, 1)
         const int kz = gt % N, rs = gt / N;
         const int offs = P == 1 ? off : 8 * HC * rs;
         unsigned char* rk = t + kz * K::PITCH + offs;
-        const float2 T0 = *reinterpret_cast<const float2*>(rk);
-        const float2 Th = *reinterpret_cast<const float2*>(rk + 8 * H);
+        float2 T0 = *reinterpret_cast<const float2*>(rk);
+        float2 Th = *reinterpret_cast<const float2*>(rk + 8 * H);
         // mirror row (-kz, -ky): its columns 0 and h from the mirror boxes
         const int mz = (N - kz) % N, mo = 16 * mz + 8 * (((N - i0 - rs) % N) & 1);
-        const float2 M0 = *reinterpret_cast<const float2*>(t + K::MAIN + 2 * rs * N * 16 + mo);
-        const float2 Mh =
-            *reinterpret_cast<const float2*>(t + K::MAIN + (2 * rs + 1) * N * 16 + mo);
+        float2 M0 = *reinterpret_cast<const float2*>(t + K::MAIN + 2 * rs * N * 16 + mo);
+        float2 Mh = *reinterpret_cast<const float2*>(t + K::MAIN + (2 * rs + 1) * N * 16 + mo);
+        if constexpr (WEIGHT) {  // (a bin and its mirror have one |m|)
+          const int my = signed_index(i0 + rs, N), mzz = signed_index(kz, N);
+          const float yz = (float)(my * my + mzz * mzz);
+          T0 = weighted(T0, wscale, yz);
+          M0 = weighted(M0, wscale, yz);
+          Th = weighted(Th, wscale, yz + (float)(H * H));
+          Mh = weighted(Mh, wscale, yz + (float)(H * H));
+        }
         const float2 A = make_float2(0.5f * (T0.x + M0.x), 0.5f * (T0.y - M0.y));
         const float2 B = make_float2(0.5f * (Th.x + Mh.x), 0.5f * (Th.y - Mh.y));
         *reinterpret_cast<float2*>(rk) = make_float2(A.x - B.y, A.y + B.x);  // A + i B
@@ -559,7 +608,15 @@ __global__ void __launch_bounds__(Cfg<N>::T, 1)
       } else {
         if (pass == 0) {
           // z: column c of the rows (kz, ky = i0 + r)
-          load_dif_rows<N, DIR, K::PITCH>(t, off + 8 * c, h, v);
+          if constexpr (WEIGHT) {
+            auto at = [&](int z) {
+              return reinterpret_cast<const float2*>(t + z * K::PITCH + off + 8 * c);
+            };
+            if (h == 0) load_dif_weighted<N, DIR, 0>(at, wxy, wscale, c == 0, v);
+            else load_dif_weighted<N, DIR, 1>(at, wxy, wscale, c == 0, v);
+          } else {
+            load_dif_rows<N, DIR, K::PITCH>(t, off + 8 * c, h, v);
+          }
           release(s);
         } else if (pass == 1) {
           // y: column c of plane i0 + r (dense rows of H complex)
@@ -739,7 +796,7 @@ inline bool encode_pairs(CUtensorMap* m, const void* base, int n, int grids, uns
   return encode(m, base, dims, strides, box, false);
 }
 
-template <int N, int DIR>
+template <int N, int DIR, bool WEIGHT>
 cudaError_t launch(const FusedArgs& a, int grid, cudaStream_t stream) {
   if (a.in_ptrs || a.grid_map || a.grid_off) return cudaErrorInvalidValue;
   CUtensorMap m0, m1;
@@ -758,15 +815,19 @@ cudaError_t launch(const FusedArgs& a, int grid, cudaStream_t stream) {
     if (!encode_pairs(&m0, a.in, N, a.ngrids, zx, zy) || !encode_pairs(&m1, a.in, N, a.ngrids, 4))
       return cudaErrorInvalidValue;
   }
-  rgrid_fft3d_kernel<N, DIR><<<grid, Cfg<N>::T, Cfg<N>::smem, stream>>>(a, m0, m1);
+  rgrid_fft3d_kernel<N, DIR, WEIGHT><<<grid, Cfg<N>::T, Cfg<N>::smem, stream>>>(a, m0, m1);
   return cudaGetLastError();
 }
 
 template <int N, int DIR>
 KernelInfo info() {
   KernelInfo k;
-  k.launch = &launch<N, DIR>;
-  k.func = (const void*)&rgrid_fft3d_kernel<N, DIR>;
+  k.launch = &launch<N, DIR, false>;
+  k.func = (const void*)&rgrid_fft3d_kernel<N, DIR, false>;
+  if constexpr (DIR > 0) {
+    k.launch_weighted = &launch<N, DIR, true>;
+    k.func_weighted = (const void*)&rgrid_fft3d_kernel<N, DIR, true>;
+  }
   k.threads = Cfg<N>::T;
   k.smem = Cfg<N>::smem;
   k.sizes[0] = N;

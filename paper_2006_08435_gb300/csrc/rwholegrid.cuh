@@ -150,8 +150,11 @@ __global__ void __launch_bounds__(Cfg<N>::T, Cfg<N>::MINB_F) rwholegrid_fwd_kern
   }
 }
 
-// Inverse kernel: a.in holds half spectra, a.out real grids.
-template <int N>
+// Inverse kernel: a.in holds half spectra, a.out real grids.  WEIGHT: the
+// spectrum times a.weight / |m|^2 as it is read (us, with / without: 32^3 x 512
+// 55.6 / 49.9, 16^3 x 4096 38.1 / 35.2; a seed pass of its own reads and writes
+// the spectra once more).
+template <int N, bool WEIGHT>
 __global__ void __launch_bounds__(Cfg<N>::T, Cfg<N>::MINB_I) rwholegrid_inv_kernel(const FusedArgs a) {
   using K = Cfg<N>;
   constexpr int H = K::H, HC = K::HC;
@@ -174,11 +177,26 @@ __global__ void __launch_bounds__(Cfg<N>::T, Cfg<N>::MINB_I) rwholegrid_inv_kern
       const int ky = t / HC, kx = t % HC;
 #pragma unroll
       for (int z = 0; z < N; ++z) v[z] = __ldg(gin + z * K::COLS + t);
+      float scale = 0.0f, xy = 0.0f;
+      if constexpr (WEIGHT) {
+        const int my = signed_index(ky, N);
+        scale = (float)(a.weight.s * a.weight.grad[grid]);
+        xy = (float)(kx * kx + my * my);
+#pragma unroll
+        for (int z = 0; z < N; ++z) {
+          const float mz = (float)signed_index(z, N);
+          v[z] = weighted(v[z], scale, xy + mz * mz);
+        }
+      }
       if (kx == 0 || kx == H) {
         const float2* mir = gin + ((N - ky) % N) * HC + kx;
 #pragma unroll
         for (int z = 0; z < N; ++z) {
-          const float2 c = __ldg(mir + ((N - z) % N) * K::COLS);
+          float2 c = __ldg(mir + ((N - z) % N) * K::COLS);
+          if constexpr (WEIGHT) {
+            const float mz = (float)signed_index(z, N);
+            c = weighted(c, scale, xy + mz * mz);
+          }
           v[z] = make_float2(0.5f * (v[z].x + c.x), 0.5f * (v[z].y - c.y));
         }
       }
@@ -240,21 +258,26 @@ __global__ void __launch_bounds__(Cfg<N>::T, Cfg<N>::MINB_I) rwholegrid_inv_kern
   }
 }
 
-template <int N, int DIR>
+template <int N, int DIR, bool WEIGHT>
 cudaError_t launch(const FusedArgs& a, int grid, cudaStream_t stream) {
   grid = grid < a.ngrids ? grid : a.ngrids;  // one block per grid at most
   if (DIR < 0)
     rwholegrid_fwd_kernel<N><<<grid, Cfg<N>::T, Cfg<N>::smem, stream>>>(a);
   else
-    rwholegrid_inv_kernel<N><<<grid, Cfg<N>::T, Cfg<N>::smem, stream>>>(a);
+    rwholegrid_inv_kernel<N, WEIGHT><<<grid, Cfg<N>::T, Cfg<N>::smem, stream>>>(a);
   return cudaGetLastError();
 }
 
 template <int N, int DIR>
 KernelInfo info() {
   KernelInfo k;
-  k.launch = &launch<N, DIR>;
-  k.func = DIR < 0 ? (const void*)&rwholegrid_fwd_kernel<N> : (const void*)&rwholegrid_inv_kernel<N>;
+  k.launch = &launch<N, DIR, false>;
+  k.func = DIR < 0 ? (const void*)&rwholegrid_fwd_kernel<N>
+                   : (const void*)&rwholegrid_inv_kernel<N, false>;
+  if (DIR > 0) {
+    k.launch_weighted = &launch<N, DIR, true>;
+    k.func_weighted = (const void*)&rwholegrid_inv_kernel<N, true>;
+  }
   k.threads = Cfg<N>::T;
   k.smem = Cfg<N>::smem;
   k.sizes[0] = N;

@@ -19,7 +19,7 @@ from __future__ import annotations
 import torch
 
 from . import _lib as L
-from .fft import _rfft3d, _stream_handle, fft3d, irfft3d
+from .fft import _get_real_plan, _on_device, _rfft3d, _stream_handle, fft3d, irfft3d
 
 _ws_cache: dict = {}
 
@@ -97,6 +97,30 @@ def seed_from_half_spectrum(rhohat_half: torch.Tensor, cell: float,
     return seed
 
 
+def gradient_from_half_spectrum(rhohat_half: torch.Tensor, cell: float,
+                                grad_e: torch.Tensor) -> torch.Tensor:
+    """irfft3d(seed_from_half_spectrum(rhohat_half, cell, grad_e)) in one
+    transform that weights the spectrum as it reads it."""
+    n = rhohat_half.shape[-2]
+    batch = rhohat_half.numel() // (n * n * (n // 2 + 1))
+    g = grad_e.to(torch.float64).contiguous().reshape(-1)
+    if g.numel() != batch:
+        raise ValueError("one gradient per grid")
+    rhohat_half = rhohat_half.contiguous()
+    dev = rhohat_half.get_device()
+    out = torch.empty(rhohat_half.shape[:-1] + (n,), dtype=torch.float32, device=rhohat_half.device)
+    with _on_device(dev):
+        stream = _stream_handle(None)
+        plan = _get_real_plan(n, batch, "fp32", True, "none", dev, stream)
+        code = L.lib().fft3d_real_execute_hartree(plan._h, rhohat_half.data_ptr(), float(cell),
+                                                  g.data_ptr(), out.data_ptr(), stream)
+    if code in (L.FFT3D_ERR_UNSUPPORTED_PRECISION, L.FFT3D_ERR_MISALIGNED):
+        # a plan of the pair scheme, a spectrum on an 8-byte boundary only
+        return irfft3d(seed_from_half_spectrum(rhohat_half, cell, grad_e))
+    L.check(code, "fft3d_real_execute_hartree")
+    return out
+
+
 def seed_from_spectrum(rhohat: torch.Tensor, cell: float, grad_e: torch.Tensor) -> torch.Tensor:
     n = rhohat.shape[-1]
     batch = rhohat.numel() // n ** 3
@@ -132,8 +156,7 @@ class HartreeEnergy(torch.autograd.Function):
     def backward(ctx, grad_e):
         (rhohat,) = ctx.saved_tensors
         if ctx.half:
-            seed = seed_from_half_spectrum(rhohat, ctx.cell, grad_e)
-            return irfft3d(seed), None
+            return gradient_from_half_spectrum(rhohat, ctx.cell, grad_e), None
         seed = seed_from_spectrum(rhohat, ctx.cell, grad_e)
         return complex_to_real(fft3d(seed, inverse=True)), None
 
