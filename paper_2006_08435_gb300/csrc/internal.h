@@ -159,9 +159,26 @@ struct TwoPassKernel {
 };
 TwoPassKernel two_pass_kernel_info(int L, int dir);        // launch null: none
 TwoPassKernel two_pass_apart_kernel_info(int L, int dir);  // for mixed-edge plans
-// The kernel's twiddles: ty and tz into a, tx and tzg appended to tab (2 L
-// entries: a.tx and a.tzg are set once tab is on the device).
+// The twiddles of splits A, AX, AZ of axes of L (x: lx) points: ty and tz into a,
+// tx and tzg appended to tab (lx + L entries: a.tx and a.tzg are set once tab is
+// on the device).
+void two_pass_twiddles(int A, int AX, int AZ, int lx, int L, TwoPassArgs& a,
+                       std::vector<float2>& tab);
 int two_pass_prepare(const TwoPassKernel& k, int L, TwoPassArgs& a, std::vector<float2>& tab);
+
+// Two-pass real transforms (twopass_real.cuh).
+struct RealPassArgs : TwoPassArgs {
+  const float2* twr;     // W_N^k, k <= N / 2
+  float2* work;          // inverse: the grids' spectra between the passes
+  HartreeWeight weight;  // inverse: grad null: none
+};
+struct RealPassKernel {
+  cudaError_t (*launch)(const RealPassArgs&, int grids, cudaStream_t) = nullptr;
+  const void* func[3] = {};
+  size_t smem[3] = {};
+  int A = 0, AX = 0, AZ = 0;
+};
+RealPassKernel real_pass_kernel_info(int n, int dir);  // launch null: none
 
 // Two-pass transforms of boxes (twopass_box.cuh): ny = A B.
 struct BoxArgs {
@@ -202,6 +219,8 @@ struct AxisPasses {
   TwoPassArgs two_args;
   BoxKernel box[2];     // func not null: two passes of a box
   BoxArgs box_args;
+  RealPassKernel real;  // launch not null: two passes of real grids
+  RealPassArgs real_args;
   int chains = 1;       // streams the chunks alternate between
   cudaStream_t side = nullptr;
   cudaEvent_t fork = nullptr, join = nullptr;

@@ -54,6 +54,16 @@ float2 root(long long m, int n) {
 
 }  // namespace
 
+void two_pass_twiddles(int A, int AX, int AZ, int lx, int L, TwoPassArgs& a,
+                       std::vector<float2>& tab) {
+  for (int i = 0; i < L; ++i) {
+    a.ty[i] = root((long long)(i / A) * (i % A), L);
+    a.tz[i] = root((long long)(i / AZ) * (i % AZ), L);
+  }
+  for (int i = 0; i < lx; ++i) tab.push_back(root((long long)(i / AX) * (i % AX), lx));
+  tab.insert(tab.end(), a.tz, a.tz + L);
+}
+
 int two_pass_prepare(const TwoPassKernel& k, int L, TwoPassArgs& a, std::vector<float2>& tab) {
   for (int i = 0; i < 3; ++i)
     if (k.smem[i] > 48 * 1024 &&
@@ -63,12 +73,7 @@ int two_pass_prepare(const TwoPassKernel& k, int L, TwoPassArgs& a, std::vector<
       return FFT3D_ERR_CUDA;
     }
   a = TwoPassArgs{};
-  for (int i = 0; i < L; ++i) {
-    a.ty[i] = root((long long)(i / k.A) * (i % k.A), L);
-    a.tz[i] = root((long long)(i / k.AZ) * (i % k.AZ), L);
-  }
-  for (int i = 0; i < L; ++i) tab.push_back(root((long long)(i / k.AX) * (i % k.AX), L));
-  tab.insert(tab.end(), a.tz, a.tz + L);
+  two_pass_twiddles(k.A, k.AX, k.AZ, L, L, a, tab);
   return FFT3D_SUCCESS;
 }
 
@@ -94,6 +99,21 @@ int AxisPasses::create(PassKind kind_, int nx_, int ny_, int nz_, int batch_, in
     if (rc) return rc;
     two_args.scale = scale;
     two_args.do_scale = do_scale;
+  }
+  real = RealPassKernel{};
+  if (kind != kPassC2C && nx == ny && ny == nz) real = real_pass_kernel_info(nx, dir);
+  if (real.launch) {
+    for (int i = 0; i < 3; ++i)
+      if (real.func[i] && real.smem[i] > 48 * 1024 &&
+          cudaFuncSetAttribute(real.func[i], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)real.smem[i]) != cudaSuccess) {
+        cudaGetLastError();
+        return FFT3D_ERR_CUDA;
+      }
+    real_args = RealPassArgs{};
+    two_pass_twiddles(real.A, real.AX, real.AZ, lx, nx, real_args, tab);
+    real_args.scale = scale;
+    real_args.do_scale = do_scale;
   }
   // a box: ny = A B with B points per thread, A as small as it goes
   box[0] = box[1] = BoxKernel{};
@@ -140,7 +160,7 @@ int AxisPasses::create(PassKind kind_, int nx_, int ny_, int nz_, int batch_, in
       tab.insert(tab.end(), b.tz, b.tz + nz);
     }
   }
-  for (int a = 0; a < 3 && !two.launch; ++a) {
+  for (int a = 0; a < 3 && !two.launch && !real.launch; ++a) {
     k[a] = pencil_kernel_info(len[a], dir, a == 0 ? kx : 0);
     if (!k[a].launch) return FFT3D_ERR_UNSUPPORTED_SIZE;
     if (k[a].smem > 48 * 1024 &&
@@ -156,7 +176,7 @@ int AxisPasses::create(PassKind kind_, int nx_, int ny_, int nz_, int batch_, in
         for (int n1 = 0; n1 < A; ++n1) tab.push_back(root((long long)n1 * k2, len[a]));
   }
   kw = PencilKernel{};
-  if (kind == kPassC2R) {
+  if (kind == kPassC2R && !real.launch) {
     kw = pencil_kernel_info(nz, dir, 4);
     if (kw.launch && kw.smem > 48 * 1024 &&
         cudaFuncSetAttribute(kw.func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kw.smem) !=
@@ -185,6 +205,9 @@ int AxisPasses::create(PassKind kind_, int nx_, int ny_, int nz_, int batch_, in
   two_args.tzg = d_tab + nx;
   box_args.tx = d_tab;
   box_args.tzg = d_tab + nx;
+  real_args.tx = d_tab;
+  real_args.tzg = d_tab + lx;
+  real_args.twr = twr;
 
   // Chunk budget: the intermediates of the chunks in flight within 40% of L2
   // (complex grids: 96 x 128 x 64 x 64 261 us, 60%: 270), 60% for real
@@ -247,6 +270,19 @@ cudaError_t AxisPasses::chunk_passes(long long g, const void* in, void* out, flo
     a.in = static_cast<const float2*>(in) + g * pp * nz;
     a.out = static_cast<float2*>(out) + g * pp * nz;
     return two.launch(a, (int)m, in == out, s);
+  }
+  if (real.launch) {
+    const long long m = std::min(chunk, batch - g);
+    const long long real_pts = (long long)nx / 2 * ny * nz, spec_pts = pp * nz;
+    RealPassArgs a = real_args;
+    a.in = static_cast<const float2*>(in) + g * (kind == kPassR2C ? real_pts : spec_pts);
+    a.out = static_cast<float2*>(out) + g * (kind == kPassR2C ? spec_pts : real_pts);
+    a.work = work;
+    if (weight) {
+      a.weight = *weight;
+      a.weight.grad += g;
+    }
+    return real.launch(a, (int)m, s);
   }
   // contiguous rows of `planes` planes
   auto x_pass = [&](const float2* src, float2* dst, long long planes) {

@@ -350,7 +350,6 @@ __global__ void __launch_bounds__(Cfg<L, KIND>::T, Cfg<L, KIND>::blocks) pencil_
 #pragma unroll
         for (int j = 0; j < B; ++j) v[j] = ldg(src + j * step, pin);
         if constexpr (KIND == kWeighted) {
-          // (96^3 x 32: 101.4 us for the transform, 100.6 without the weights)
           // pencil -> (grid, ky, kx); its points are kz = n1 + A j
           const unsigned p = p0 + (unsigned)c, o = fdiv(p, a.divn), r = p - o * a.nx;
           const int ky = (int)fdiv(r, a.divh), kx = (int)r - ky * a.hx;

@@ -397,6 +397,17 @@ int create_pair_real(int n, int batch, int direction, fft3d_plan inner, fft3d_re
   return FFT3D_SUCCESS;
 }
 
+// Edges with a persistent kernel and a two-pass one (twopass_real.cuh): where
+// the two passes are faster.  us, persistent / two passes: forward 64^3 x 1 17.2 /
+// 6.6, x 64 50.8 / 43.9, x 1024 764 / 662, 128^3 x 1 30.9 / 15.5, x 32 193.7 /
+// 165.4, x 128 757 / 629; inverse 64^3 x 1 15.8 / 6.5, x 96 68.0 / 67.5, x 128
+// 88.0 / 88.9, x 1024 618 / 680, 128^3 x 1 24.0 / 12.1, x 16 92.8 / 87.1, x 48 252.2 /
+// 252.3, x 128 641 / 664 (with the Hartree weights x 32 204.1 / 174.0).
+bool two_pass_real(int n, int batch, int direction) {
+  if (n != 64 && n != 128) return false;
+  return direction == FFT3D_FORWARD || batch < (n == 64 ? 100 : 48);
+}
+
 // The complex kernel of fft3d_real_plan_create_fixed: at 48^3, 80^3 and 96^3
 // the persistent kernel, from as many pairs as first chosen the thread-pair
 // kernel (another arithmetic order); elsewhere three pencil passes, which
@@ -423,7 +434,8 @@ int fft3d_real_plan_create(int n, int batch, int precision, int direction, int n
   const bool pairs_only = path && std::strcmp(path, "pairs") == 0;
   if (precision == FFT3D_FP32 && !pairs_only) {
     const fft3d::KernelInfo k = fft3d::real_kernel_info(n, direction == FFT3D_FORWARD ? -1 : 1);
-    if (k.launch) return fft3d::create_fused_real(n, batch, direction, norm, k, out_plan);
+    if (k.launch && !fft3d::two_pass_real(n, batch, direction))
+      return fft3d::create_fused_real(n, batch, direction, norm, k, out_plan);
     if (n > 2) return fft3d::create_pencil_real(n, batch, direction, norm, out_plan);
   }
   fft3d_plan inner = nullptr;
@@ -510,7 +522,7 @@ int fft3d_real_execute_hartree(fft3d_real_plan plan, const void* rhohat_half, do
   w.s = hartree_s(plan->n, L);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (plan->fused) return execute_fused_real(plan, rhohat_half, out, s, &w);
-  if (!plan->passes.kw.launch) return FFT3D_ERR_UNSUPPORTED_SIZE;
+  if (!plan->passes.kw.launch && !plan->passes.real.launch) return FFT3D_ERR_UNSUPPORTED_SIZE;
   if (plan->passes.execute(rhohat_half, out, plan->d_work, s, &w) != cudaSuccess) {
     cudaGetLastError();
     return FFT3D_ERR_CUDA;
