@@ -187,8 +187,8 @@ struct BoxArgs {
   int in_place;  // out == in: pass 1 runs in clusters of A blocks
   const float2 *tx, *tzg;
   float2 ty[kTwoPassMaxLen], tz[kTwoPassMaxLen];
-  int A, B, nx, xtiles;
-  FastDiv divA, divB, divxt;
+  int A, B, nx, tiles;  // tiles: pass-2 blocks of a grid, 16 of its B nx columns each
+  FastDiv divA, divB, divt;
   float scale;
   int do_scale;
 };

@@ -147,10 +147,10 @@ int AxisPasses::create(PassKind kind_, int nx_, int ny_, int nz_, int batch_, in
       b.A = A;
       b.B = ny / A;
       b.nx = nx;
-      b.xtiles = (nx + 15) / 16;
+      b.tiles = (b.B * nx + 15) / 16;
       b.divA = make_fastdiv((unsigned)b.A);
       b.divB = make_fastdiv((unsigned)b.B);
-      b.divxt = make_fastdiv((unsigned)b.xtiles);
+      b.divt = make_fastdiv((unsigned)b.tiles);
       b.scale = scale;
       b.do_scale = do_scale;
       for (int i = 0; i < ny; ++i) b.ty[i] = root((long long)(i / A) * (i % A), ny);
@@ -346,9 +346,8 @@ cudaError_t AxisPasses::chunk_passes(long long g, const void* in, void* out, flo
     a.in_place = in == out;
     const cudaError_t e = launch_box(box[0], (unsigned)(m * nz * a.A), box[0].smem * a.B,
                                      a.in_place ? a.A : 1, a, s);
-    return e != cudaSuccess
-               ? e
-               : launch_box(box[1], (unsigned)(m * a.B * a.xtiles), box[1].smem, 1, a, s);
+    return e != cudaSuccess ? e
+                            : launch_box(box[1], (unsigned)(m * a.tiles), box[1].smem, 1, a, s);
   }
   // complex points of one grid on the x pass's two sides
   const long long real_pts = (long long)nx / 2 * ny * nz, spec_pts = pp * nz;

@@ -228,25 +228,27 @@ int builtin_default_variant(bool mixed, int n, int batch, int precision) {
     // The general path (dependent launches of small blocks: three pencil
     // passes at 32^3, two passes at the others) fills the GPU where the ticket
     // kernels' large items leave it idle, and pays 4 us per launch of a chunk
-    // where they pay once.  us, general path / the kernels before:
+    // where they pay once.  In place it is up to 15% slower at 80^3, 96^3 and
+    // 128^3, so the lines there lie where that still costs under 4%.
+    // us, general path / the kernels before:
     // 32^3 x 16 8.5 / 10.5, x 32 13.1 / 12.2 (3), x 64 15.7 / 18.8, x 127 24.5 /
     // 31.5, x 200 35.9 / 39.5 (13), x 400 67.6 / 66.5
     case 32: return batch >= 300 ? 13 : batch >= 48 ? kGeneralVariant : 3;
-    // 48^3 x 1 7.2 / 11.8 (0), x 16 12.6 / 23.1, x 40 19.8 / 27.9 (13), x 400 178 /
-    // 192
+    // 48^3 x 1 7.2 / 11.8 (0), x 48 24.5 / 29.4 (13), x 300 128 / 152, x 2000 825 /
+    // 941 (in place 860 / 940)
     case 48: return kGeneralVariant;
-    // 64^3 x 1 7.1 / 11.7 (5), x 4 8.7 / 18.4 (1), x 32 38.3 / 51.0 (7), x 64
-    // 74.6 / 77.7 (8), x 100 113.8 / 110.1
-    case 64: return batch >= 80 ? 8 : kGeneralVariant;
-    // 80^3 x 1 9.5 / 14.9 (0), x 12 30.8 / 37.6 (13), x 80 182 / 189, x 200 450 /
-    // 442
-    case 80: return batch >= 150 ? 13 : kGeneralVariant;
-    // 96^3 x 1 10.5 / 17.1 (0), x 8 33.6 / 43.0 (13), x 24 97.8 / 101.9, x 48 188.9 /
-    // 182.9
-    case 96: return batch >= 36 ? 13 : kGeneralVariant;
-    // 128^3 x 1 17.3 / 20.9 (5), x 2 23.6 / 31.7 (6), x 8 78.7 / 86.4, x 16 152.6 /
-    // 155.2, x 24 225.4 / 222.8
-    case 128: return batch >= 20 ? 6 : kGeneralVariant;
+    // 64^3 x 1 7.1 / 11.7 (5), x 4 8.7 / 18.4 (1), x 32 37.5 / 50.1 (7), x 80 90.6 /
+    // 95.5 (8), x 96 107.8 / 105.4, x 1024 1100 / 957
+    case 64: return batch >= 88 ? 8 : kGeneralVariant;
+    // 80^3 x 1 7.8 / 14.9 (0), x 20 47.7 / 59.3 (13), x 54 118.6 / 131.5 (in place
+    // 134.2 / 130.6), x 80 170 / 188 (196 / 188), x 400 825 / 859 (948 / 858)
+    case 80: return batch >= 64 ? 13 : kGeneralVariant;
+    // 96^3 x 1 10.8 / 17.1 (0), x 8 34.5 / 43.3 (13), x 24 98.1 / 102.5 (in place
+    // 101.1 / 101.3), x 28 113.9 / 116.9 (121.5 / 115.9), x 48 190 / 185
+    case 96: return batch >= 28 ? 13 : kGeneralVariant;
+    // 128^3 x 1 16.4 / 20.9 (5), x 2 24.3 / 32.0 (6), x 8 80.7 / 87.8, x 12 117.9 /
+    // 123.2 (in place 121.8 / 121.3), x 16 155.0 / 157.2 (163 / 155), x 32 301 / 295
+    case 128: return batch >= 16 ? 6 : kGeneralVariant;
     default: return 0;
   }
 }

@@ -6,27 +6,34 @@
 //     register steps with one exchange in shared memory), then per column the
 //     B-point DFT over j in one thread, times W_L^(n1 k2), stored to row
 //     k2 + B n1 of plane z;
-//   pass 2, block (grid, k2, W columns): the rows k2 + B n1 of every z: first
-//     step of the z transform from global memory to shared memory, then one
-//     thread per (column, kz2) holds its points of all A rows, finishes the z
-//     transforms and the A-point DFT over n1, and stores rows k2 + B k1, the
-//     same rows it read.
+//   pass 2, block (grid, W of the B L columns (k2, x)): the rows k2 + B n1 of
+//     every z: first step of the z transform from global memory to shared memory,
+//     then one thread per (column, kz2) holds its points of all A rows, finishes
+//     the z transforms and the A-point DFT over n1, and stores rows k2 + B k1, the
+//     same points it read.
 // A grid crosses L2 twice (32 bytes per point; the separate passes of
 // pencil.cuh 48), which with HBM's own fills and write-backs is what bounds
 // both: 48 and 64 bytes per point at the 13.8 TB/s that a copy from and to HBM
-// reaches there (64^3 x 256: 233 us; measured 283).  The rest is L1: wavefronts
-// of short runs and of bank conflicts.  Hence at least 16 lanes along x in the
-// first step of pass 1 (AX; 128^3 x 32 with 8 columns and 8 lanes 434 us, with 16
-// and 16 338), W >= 16 columns in pass 2, pitches searched at compile time for
-// the three access patterns of pass 1, and twiddles that are the same for a
-// whole warp read from the kernel's parameters (constant bank).  Splits per
-// edge from a sweep; the next best lies 1-5% behind.  Measured, us, two passes /
-// three: 64^3 x 12 16.8 / 21.5, x 64 74.6 / 90.3; 96^3 x 8 33.6 / 44.2; 128^3 x 2
-// 23.6 / 27.5, x 8 78.7 / 92.7; 100^3 x 16 86 / 94; 60^3 x 80 89 / 98.  At 120, 144
-// and 160 no split gains more than the tiles' size costs.
+// reaches there (64^3 x 106: 97 us; measured 119).  The rest is L1 and latency:
+// short runs, bank conflicts, loads in flight.  Hence runs of 64 bytes and more
+// in the first step of pass 1, shared rows whose strided accesses do not conflict
+// (row_layout), columns taken 16 at a time across the rows k2 (whatever L is, full
+// and aligned to 128 bytes where B L is a multiple of 16), and
+// twiddles that are the same for a whole warp read from the kernel's parameters
+// (constant bank; of x they stay in the first step: in the second, where lanes
+// run along the rows, 96 x 128 x 64 x 64 took 257 us for 231).
+// Splits per edge from a sweep; the next best lies 1-5% behind.  us, three passes /
+// two passes with padded rows of their own splits / now: 60^3 x 129 - / 140 / 123;
+// 72^3 x 75 - / 135 / 120; 80^3 x 54 - / 129 / 118; 90^3 x 38 - / 174 / 137; 108^3 x 22
+// - / 155 / 129; 100^3 x 16 94 / 86 / 79; 48^3 x 400 - / 191 / 169; 64^3 x 64 90.3 / 74.6 /
+// 72.4; 96^3 x 8 44.2 / 33.6 / 34.5; 128^3 x 8 92.7 / 78.7 / 80.5.
 //
-// In place, the A blocks of a plane read rows that the others write: they run
-// as a cluster and store after a cluster barrier behind everybody's loads.
+// In place, the A groups of a plane read rows that the others write.  Where their
+// rows take at most 56 KB they are one block (four fit a multiprocessor);
+// above, they run as a cluster of blocks and store after a cluster barrier behind
+// everybody's loads.  us in place, cluster / one block: 48^3 x 253 158 / 116, 60^3 x
+// 129 178 / 135, 64^3 x 106 156 / 120, 80^3 x 54 140 / 134, 96^3 x 31 139 / 144, 128^3 x
+// 32 317 / 379.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -45,73 +52,79 @@ using pc::transform;
 using pc::twiddle;
 
 // Splits of an edge: y into A groups of B; x and z into two register steps,
-// BX (BZ) points first, AX (AZ) apart, then AX (AZ); W columns in pass 2.
+// BX (BZ) points first, AX (AZ) apart, then AX (AZ).
 template <int L>
 struct Cfg;
-#define FFT3D_TP(L_, A_, AX_, AZ_, W_)                                  \
+#define FFT3D_TP(L_, A_, AX_, AZ_)                                      \
   template <>                                                           \
   struct Cfg<L_> {                                                      \
     static constexpr int L = L_, A = A_, B = L_ / A_;                   \
     static constexpr int AX = AX_, BX = L_ / AX_, AZ = AZ_, BZ = L_ / AZ_; \
-    static constexpr int W = W_;                                        \
+    static constexpr int W = 16; /* columns of a pass-2 block */        \
   };
-FFT3D_TP(48, 3, 16, 4, 16)
-FFT3D_TP(60, 3, 20, 6, 20)
-FFT3D_TP(64, 4, 16, 4, 16)
-FFT3D_TP(72, 3, 24, 6, 24)
-FFT3D_TP(80, 4, 16, 8, 16)
-FFT3D_TP(90, 3, 18, 9, 18)
-FFT3D_TP(96, 4, 16, 8, 16)
-FFT3D_TP(100, 4, 20, 5, 20)
-FFT3D_TP(108, 6, 18, 6, 18)
-FFT3D_TP(128, 4, 16, 8, 16)
+FFT3D_TP(48, 3, 8, 4)
+FFT3D_TP(60, 4, 12, 4)
+FFT3D_TP(64, 4, 16, 4)
+FFT3D_TP(72, 3, 12, 6)
+FFT3D_TP(80, 4, 16, 4)
+FFT3D_TP(90, 5, 15, 6)
+FFT3D_TP(96, 4, 16, 8)
+FFT3D_TP(100, 5, 10, 5)
+FFT3D_TP(108, 4, 12, 9)
+FFT3D_TP(128, 4, 16, 8)
 #undef FFT3D_TP
 
-// Bank conflicts (extra wavefronts per half-warp of 8-byte accesses) of the
-// three access patterns of pass 1 for slots (row j, k2, m) at j RP + k2 AP + m.
-constexpr int conflicts(int AX, int BX, int L, int AP, int RP) {
-  int total = 0;
-  for (int pat = 0; pat < 3; ++pat)
-    for (int h = 0; h < 4; ++h) {
-      int n[16] = {}, worst = 0;
-      for (int l = 0; l < 16; ++l) {
-        const int e = h * 16 + l;
-        const int at = pat == 0 ? e / AX * RP + e % AX
-                     : pat == 1 ? e / BX * RP + e % BX * AP
-                                : e % L % BX * AP + e % L / BX;
-        const int c = ++n[at % 16];
-        worst = c > worst ? c : worst;
-      }
-      total += worst - 1;
-    }
-  return total;
-}
-struct Pitch {
-  int AP, RP;
+// Rows in shared memory for an x transform in two register steps, P lanes of Q
+// points first, then Q of P: row j at j RP, its points in natural order (k + Q m
+// the output k of lane m), with one slot left free after every PD where PD is not
+// 0.  Each step's items read and write one set of slots, and columns lie side by
+// side.  The layout is the one of least extra wavefronts per half-warp of 8-byte
+// accesses in the two strided patterns: items (j, m) at j RP + m Q, and items
+// (k, j) with lanes along j at j RP + k (whose twiddles are the same for a row's
+// worth of lanes).
+struct Layout {
+  int PD, RP;
 };
-constexpr Pitch best_pitch(int AX, int BX, int L) {
-  Pitch best{AX, AX * BX};
+FFT3D_HD constexpr int slot(int PD, int p) { return PD ? p + p / PD : p; }
+constexpr Layout row_layout(int B, int P, int Q, int points) {
+  Layout best{0, 0};
   int least = 1 << 20;
-  for (int ap = AX; ap < AX + 4; ++ap)
-    for (int rp = ap * BX; rp < ap * BX + 16; ++rp) {
-      const int c = 64 * conflicts(AX, BX, L, ap, rp) + rp - AX * BX;
-      if (c < least) {
-        least = c;
-        best = Pitch{ap, rp};
+  int lcm = 16;
+  while (lcm % Q) lcm += 16;
+  for (int o = 0; o < (Q % 2 ? 1 : 2); ++o) {
+    const int PD = o ? lcm : 0;
+    for (int rp = slot(PD, points - 1) + 1, i = 0; i < 16; ++i, ++rp) {
+      int total = 0;
+      for (int pat = 0; pat < 2; ++pat)
+        for (int h = 0; h < 8; ++h) {
+          int n[16] = {}, worst = 0;
+          for (int l = 0; l < 16; ++l) {
+            const int e = h * 16 + l;
+            const int at = pat == 0 ? e / P * rp + slot(PD, e % P * Q) : e % B * rp + e / B;
+            const int c = ++n[at % 16];
+            worst = c > worst ? c : worst;
+          }
+          total += worst - 1;
+        }
+      if (total * 64 + i < least) {
+        least = total * 64 + i;
+        best = Layout{PD, rp};
       }
     }
+  }
   return best;
 }
 
 template <int L>
 struct Dims : Cfg<L> {
   using C = Cfg<L>;
-  // pass 1: row j at j * RP, point (k2, n1) of it at k2 * AP + n1
-  static constexpr Pitch pitch = best_pitch(C::AX, C::BX, L);
-  static constexpr int AP = pitch.AP, RP = pitch.RP;
+  static constexpr Layout rows = row_layout(C::B, C::AX, C::BX, L);
+  static constexpr int PD = rows.PD, RP = rows.RP;
   static constexpr int T1 = (L + 31) / 32 * 32;
   static constexpr size_t smem1 = sizeof(float2) * (size_t)C::B * RP;
+  static constexpr bool MERGED = C::A * smem1 <= 56 * 1024;  // in place: see above
   // pass 2: point (kz2, m1, n1) of column q at kz2 * ZP + (m1 * A + n1) * W + q
+  static constexpr int NC = C::B * L, TILES = (NC + C::W - 1) / C::W;  // columns (k2, x)
   static constexpr bool uniform = C::W * C::A % 32 == 0;  // m1 the same for a warp
   static constexpr int ZR = C::AZ * C::A * C::W;
   static constexpr int ZP = ZR % 16 == 0 ? ZR + 8 : ZR;
@@ -142,13 +155,18 @@ struct GridAt {
 };
 
 template <int L, int DIR, bool INPLACE, bool APART>
-__global__ void __launch_bounds__(Dims<L>::T1) pass1_kernel(const __grid_constant__ TwoPassArgs a) {
+__global__ void __launch_bounds__(Dims<L>::T1 * (INPLACE && Dims<L>::MERGED ? Dims<L>::A : 1))
+    pass1_kernel(const __grid_constant__ TwoPassArgs a) {
   using D = Dims<L>;
   constexpr int A = D::A, B = D::B, AX = D::AX, BX = D::BX, T = D::T1;
-  extern __shared__ __align__(16) float2 sm[];
+  extern __shared__ __align__(16) float2 rows[];
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const unsigned zz = blockIdx.x / A, g = zz / L;  // plane, grid
-  const int n1 = (int)(blockIdx.x - zz * A);
+  constexpr bool M = INPLACE && D::MERGED;
+  // plane, grid; group n1 of y and this thread of it
+  const unsigned zz = M ? blockIdx.x : blockIdx.x / A, g = zz / L;
+  const int n1 = M ? (int)threadIdx.x / T : (int)(blockIdx.x - zz * A);
+  const int tid = M ? (int)threadIdx.x % T : (int)threadIdx.x;
+  float2* const sm = rows + (M ? n1 * (B * D::RP) : 0);
   const uint64_t once = l2_policy(kEvictFirst), keep = l2_policy(kEvictLast);
   const GridAt<APART> at(a, g, (size_t)L * L * L);
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -159,7 +177,7 @@ __global__ void __launch_bounds__(Dims<L>::T1) pass1_kernel(const __grid_constan
   constexpr int N1 = B * AX;
 #pragma unroll 1
   for (int it = 0; it < (N1 + T - 1) / T; ++it) {
-    const int e = threadIdx.x + it * T;
+    const int e = tid + it * T;
     if (N1 % T && e >= N1) break;
     const int j = e / AX, m = e % AX;
     const float2* s = src + j * (A * L) + m;
@@ -167,40 +185,40 @@ __global__ void __launch_bounds__(Dims<L>::T1) pass1_kernel(const __grid_constan
 #pragma unroll
     for (int i = 0; i < BX; ++i) v[i] = ldg(s + AX * i, once);
     transform<BX, DIR>(v);
-    float2* x = sm + j * D::RP + m;
+    float2* x = sm + j * D::RP;
 #pragma unroll
-    for (int k = 0; k < BX; ++k)
-      x[k * D::AP] = k ? twiddle<DIR>(v[k], __ldg(a.tx + k * AX + m)) : v[k];
+    for (int k = 0; k < BX; ++k) x[slot(D::PD, BX * m + k)] = k ? twiddle<DIR>(v[k], __ldg(a.tx + k * AX + m)) : v[k];
   }
-  if constexpr (INPLACE) {
+  if constexpr (INPLACE && !M) {
     // the cluster's A blocks read and write the same plane
     __syncwarp();
     asm volatile("barrier.cluster.arrive.aligned;" ::: "memory");
   }
   __syncthreads();
-  // x, second step, in place: item (row j, k2)
+  // x, second step, in place: item (k2, row j)
   constexpr int N2 = B * BX;
 #pragma unroll 1
   for (int it = 0; it < (N2 + T - 1) / T; ++it) {
-    const int e = threadIdx.x + it * T;
+    const int e = tid + it * T;
     if (N2 % T && e >= N2) break;
-    float2* x = sm + e / BX * D::RP + e % BX * D::AP;
+    const int k = e / B;
+    float2* x = sm + e % B * D::RP;
     float2 v[AX];
 #pragma unroll
-    for (int i = 0; i < AX; ++i) v[i] = x[i];
+    for (int i = 0; i < AX; ++i) v[i] = x[slot(D::PD, BX * i + k)];
     transform<AX, DIR>(v);
 #pragma unroll
-    for (int i = 0; i < AX; ++i) x[i] = v[i];
+    for (int i = 0; i < AX; ++i) x[slot(D::PD, BX * i + k)] = v[i];
   }
-  if constexpr (INPLACE) {
+  if constexpr (INPLACE && !M) {
     __syncwarp();
     asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
   }
   __syncthreads();
   // y: column kx = k2 + BX k1, its B points of this group
-  if (threadIdx.x < L) {
-    const int kx = threadIdx.x;
-    const float2* x = sm + kx % BX * D::AP + kx / BX;
+  if (tid < L) {
+    const int kx = tid;
+    const float2* x = sm + slot(D::PD, kx);
     float2 v[B];
 #pragma unroll
     for (int j = 0; j < B; ++j) v[j] = x[j * D::RP];
@@ -215,16 +233,18 @@ __global__ void __launch_bounds__(Dims<L>::T1) pass1_kernel(const __grid_constan
 template <int L, int DIR, bool APART>
 __global__ void __launch_bounds__(Dims<L>::T2) pass2_kernel(const __grid_constant__ TwoPassArgs a) {
   using D = Dims<L>;
-  constexpr int A = D::A, B = D::B, AZ = D::AZ, BZ = D::BZ, W = D::W, T = D::T2;
+  constexpr int A = D::A, AZ = D::AZ, BZ = D::BZ, W = D::W, T = D::T2;
   constexpr long long LL = (long long)L * L;
   extern __shared__ __align__(16) float2 sm[];
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const unsigned xt = blockIdx.x % (L / W), r = blockIdx.x / (L / W);
-  const unsigned k2 = r % B, g = r / B;
+  constexpr int NC = D::NC;
+  const unsigned g = blockIdx.x / D::TILES;
+  const int c0 = (int)(blockIdx.x - g * D::TILES) * W;  // first column (k2, x)
+  const int cols = min(W, NC - c0);
   const uint64_t once = l2_policy(kEvictFirst);
   const GridAt<APART> at(a, g, (size_t)LL * L);
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  float2* base = at.out(a) + (long long)k2 * L + xt * W;
+  float2* base = at.out(a) + c0;
   // z, first step: item (m1, n1, q) -> planes m1 + AZ i
   constexpr int N1 = W * A * AZ;
 #pragma unroll 1
@@ -233,7 +253,8 @@ __global__ void __launch_bounds__(Dims<L>::T2) pass2_kernel(const __grid_constan
     if (N1 % T && e >= N1) break;
     const int q = e % W, n1 = e / W % A;
     const int m1 = D::uniform ? __shfl_sync(0xffffffffu, e / (W * A), 0) : e / (W * A);
-    const float2* s = base + m1 * LL + n1 * (B * L) + q;
+    if (NC % W && q >= cols) continue;
+    const float2* s = base + m1 * LL + n1 * NC + q;
     float2 v[BZ];
 #pragma unroll
     for (int i = 0; i < BZ; ++i) v[i] = ldg(s + (long long)(AZ * i) * LL, once);
@@ -249,6 +270,7 @@ __global__ void __launch_bounds__(Dims<L>::T2) pass2_kernel(const __grid_constan
   const int e = threadIdx.x;
   if (N2 % T == 0 || e < N2) {
     const int q = e % W, kz2 = e / W;
+    if (NC % W && q >= cols) return;
     const float2* x = sm + kz2 * D::ZP + q;
     float2 v[A][AZ];
 #pragma unroll
@@ -266,7 +288,7 @@ __global__ void __launch_bounds__(Dims<L>::T2) pass2_kernel(const __grid_constan
       transform<A, DIR>(u);
 #pragma unroll
       for (int k1 = 0; k1 < A; ++k1)
-        stg(o + (long long)(BZ * k) * LL + k1 * (B * L), a.do_scale ? cscale(u[k1], a.scale) : u[k1],
+        stg(o + (long long)(BZ * k) * LL + k1 * NC, a.do_scale ? cscale(u[k1], a.scale) : u[k1],
             once);
     }
   }
@@ -283,18 +305,18 @@ cudaError_t launch(const TwoPassArgs& a, int grids, bool in_place, cudaStream_t 
   attr[1].val.clusterDim.x = D::A;
   attr[1].val.clusterDim.y = 1;
   attr[1].val.clusterDim.z = 1;
+  const bool merged = in_place && D::MERGED;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = in_place && !merged ? 2 : 1;
   cfg.stream = s;
-  cfg.gridDim = dim3((unsigned)grids * L * D::A, 1, 1);
-  cfg.blockDim = dim3(D::T1, 1, 1);
-  cfg.dynamicSmemBytes = D::smem1;
-  cfg.numAttrs = in_place ? 2 : 1;
+  cfg.gridDim = dim3((unsigned)grids * L * (merged ? 1 : D::A), 1, 1);
+  cfg.blockDim = dim3(D::T1 * (merged ? D::A : 1), 1, 1);
+  cfg.dynamicSmemBytes = D::smem1 * (merged ? D::A : 1);
   const cudaError_t e = in_place ? cudaLaunchKernelEx(&cfg, &pass1_kernel<L, DIR, true, APART>, a)
                                  : cudaLaunchKernelEx(&cfg, &pass1_kernel<L, DIR, false, APART>, a);
   if (e != cudaSuccess) return e;
   cfg.numAttrs = 1;
-  cfg.gridDim = dim3((unsigned)grids * D::B * (L / D::W), 1, 1);
+  cfg.gridDim = dim3((unsigned)grids * D::TILES, 1, 1);
   cfg.blockDim = dim3(D::T2, 1, 1);
   cfg.dynamicSmemBytes = D::smem2;
   return cudaLaunchKernelEx(&cfg, &pass2_kernel<L, DIR, APART>, a);
@@ -308,7 +330,8 @@ TwoPassKernel entry() {
   k.func[0] = (const void*)&pass1_kernel<L, DIR, false, APART>;
   k.func[1] = (const void*)&pass1_kernel<L, DIR, true, APART>;
   k.func[2] = (const void*)&pass2_kernel<L, DIR, APART>;
-  k.smem[0] = k.smem[1] = D::smem1;
+  k.smem[0] = D::smem1;
+  k.smem[1] = D::smem1 * (D::MERGED ? D::A : 1);
   k.smem[2] = D::smem2;
   k.A = D::A;
   k.AX = D::AX;

@@ -2,8 +2,9 @@
 // per nx, with the points B per thread of its y step chosen at run time, pass 2
 // per (A, nz), ny = A B.  Packed batches; in place with clusters of A blocks.
 // What bounds it and why the steps are split as they are: see twopass.cuh.
-// GB300, us, two passes / three: 96 x 128 x 64, 64 grids 232 / 264; 128 x 96 x
-// 80 x 16 78 / 88; 75^3 x 20 49 / 59; 135 x 128 x 90 x 4 37 / 42.
+// GB300, us, two passes / three: 96 x 128 x 64, 64 grids 231 / 264; 128 x 96 x
+// 80 x 16 78 / 88; 75^3 x 20 46 / 59; 135 x 128 x 90 x 4 33.5 / 42; 120^3 x 16 143 /
+// 190 (two passes with tiles of 16 columns of one row k2).
 #pragma once
 
 #include "twopass.cuh"
@@ -11,10 +12,11 @@
 namespace fft3d {
 namespace tp {
 
-// x: AX points apart in the first step, the codelet nearest 16 whose partner
-// is one too (AX lanes of a warp read one run).
+// x: AX points apart in the first step (AX lanes of a warp read one run), the
+// first of the order whose partner is a codelet too; 10 .. 16 before more, which
+// leaves the first step too few points (90 x 90 x 90 x 38 by 18 / 15: 174 / 150 us).
 constexpr int box_ax(int L) {
-  const int order[] = {16, 20, 18, 15, 24, 25, 12, 27, 30, 32, 10, 9, 8};
+  const int order[] = {16, 15, 12, 10, 20, 18, 24, 25, 27, 30, 32, 9, 8};
   for (int a : order)
     if (L % a == 0 && L / a >= 2 && L / a <= 16 && pc::codelet(L / a)) return a;
   return 0;
@@ -31,8 +33,8 @@ constexpr int box_az(int A, int L) {
 template <int LX>
 struct BoxX {
   static constexpr int AX = box_ax(LX), BX = LX / AX;
-  static constexpr Pitch pitch = best_pitch(AX, BX, LX);
-  static constexpr int AP = pitch.AP, RP = pitch.RP;
+  static constexpr Layout rows = row_layout(32, AX, BX, LX);  // (any number of rows)
+  static constexpr int PD = rows.PD, RP = rows.RP;
   static constexpr int T = LX <= 64 ? 64 : (LX + 31) / 32 * 32;
 };
 constexpr int kBoxW = 16;  // columns of a pass-2 block
@@ -79,10 +81,9 @@ __global__ void __launch_bounds__(BoxX<LX>::T) box1_kernel(const __grid_constant
 #pragma unroll
     for (int i = 0; i < BX; ++i) v[i] = ldg(s + AX * i, once);
     transform<BX, DIR>(v);
-    float2* x = sm + j * D::RP + m;
+    float2* x = sm + j * D::RP;
 #pragma unroll
-    for (int k = 0; k < BX; ++k)
-      x[k * D::AP] = k ? twiddle<DIR>(v[k], __ldg(a.tx + k * AX + m)) : v[k];
+    for (int k = 0; k < BX; ++k) x[slot(D::PD, BX * m + k)] = k ? twiddle<DIR>(v[k], __ldg(a.tx + k * AX + m)) : v[k];
   }
   if (a.in_place) {  // the cluster's A blocks read and write the same plane
     __syncwarp();
@@ -91,13 +92,14 @@ __global__ void __launch_bounds__(BoxX<LX>::T) box1_kernel(const __grid_constant
   __syncthreads();
 #pragma unroll 1
   for (int e = threadIdx.x; e < B * BX; e += T) {
-    float2* x = sm + e / BX * D::RP + e % BX * D::AP;
+    const int k = (int)pc::fdiv((unsigned)e, a.divB);
+    float2* x = sm + (e - k * B) * D::RP;
     float2 v[AX];
 #pragma unroll
-    for (int i = 0; i < AX; ++i) v[i] = x[i];
+    for (int i = 0; i < AX; ++i) v[i] = x[slot(D::PD, BX * i + k)];
     transform<AX, DIR>(v);
 #pragma unroll
-    for (int i = 0; i < AX; ++i) x[i] = v[i];
+    for (int i = 0; i < AX; ++i) x[slot(D::PD, BX * i + k)] = v[i];
   }
   if (a.in_place) {
     __syncwarp();
@@ -106,7 +108,7 @@ __global__ void __launch_bounds__(BoxX<LX>::T) box1_kernel(const __grid_constant
   __syncthreads();
   const int kx = threadIdx.x;
   if (kx < LX) {
-    const float2* x = sm + kx % BX * D::AP + kx / BX;
+    const float2* x = sm + slot(D::PD, kx);
     float2* o = dst + kx;
     switch (B) {
       case 10: box_y<10, DIR>(x, D::RP, o, LX, a.ty, A, n1, keep); break;
@@ -131,13 +133,12 @@ __global__ void __launch_bounds__(BoxZ<A, LZ>::T) box2_kernel(const __grid_const
   constexpr int AZ = D::AZ, BZ = D::BZ, W = D::W, T = D::T;
   extern __shared__ __align__(16) float2 sm[];
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int B = a.B, nx = a.nx;
-  const unsigned r = pc::fdiv(blockIdx.x, a.divxt), xt = blockIdx.x - r * a.xtiles;
-  const unsigned g = pc::fdiv(r, a.divB), k2 = r - g * B;
+  const int nc = a.B * a.nx;  // columns (k2, x) of a group
+  const unsigned g = pc::fdiv(blockIdx.x, a.divt);
+  const int c0 = (int)(blockIdx.x - g * a.tiles) * W, cols = min(W, nc - c0);
   const uint64_t once = l2_policy(kEvictFirst);
-  const long long pl = (long long)A * B * nx;
-  float2* base = a.out + (long long)g * pl * LZ + (long long)k2 * nx + xt * W;
-  const int cols = min(W, nx - (int)xt * W);
+  const long long pl = (long long)A * nc;
+  float2* base = a.out + (long long)g * pl * LZ + c0;
   asm volatile("griddepcontrol.wait;" ::: "memory");
   constexpr int N1 = W * A * AZ;
 #pragma unroll 1
@@ -148,7 +149,7 @@ __global__ void __launch_bounds__(BoxZ<A, LZ>::T) box2_kernel(const __grid_const
     int m1 = e / (W * A);
     if constexpr (D::uniform) m1 = __shfl_sync(0xffffffffu, m1, 0);
     if (q >= cols) continue;
-    const float2* s = base + m1 * pl + n1 * (B * nx) + q;
+    const float2* s = base + m1 * pl + n1 * nc + q;
     float2 v[BZ];
 #pragma unroll
     for (int i = 0; i < BZ; ++i) v[i] = ldg(s + (long long)(AZ * i) * pl, once);
@@ -180,7 +181,7 @@ __global__ void __launch_bounds__(BoxZ<A, LZ>::T) box2_kernel(const __grid_const
       transform<A, DIR>(u);
 #pragma unroll
       for (int k1 = 0; k1 < A; ++k1)
-        stg(o + (long long)(BZ * k) * pl + k1 * (B * nx), a.do_scale ? cscale(u[k1], a.scale) : u[k1],
+        stg(o + (long long)(BZ * k) * pl + k1 * nc, a.do_scale ? cscale(u[k1], a.scale) : u[k1],
             once);
     }
   }

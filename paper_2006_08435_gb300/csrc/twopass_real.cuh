@@ -15,7 +15,7 @@
 // and write-backs 48 and 64 bytes per complex point (96^3 x 32, one direction: 50
 // and 67 us at the 13.8 TB/s that copies reach there; HBM alone 34).  What bounds
 // the row kernels is L1, in wavefronts of shared memory and of twiddles: hence
-// the layout below, which no access of the four steps conflicts in, and lanes
+// the row layout of twopass.cuh, which hardly an access conflicts in, and lanes
 // along the rows in the steps whose twiddles are then one address for a warp
 // (96^3 x 32, with padded runs and lanes along the columns: forward 77.5, inverse
 // 98.1 us; now 66.3 and 79.2).  The B HX columns of a group lie side by side, so a
@@ -39,6 +39,7 @@ using pc::ldg;
 using pc::stg;
 using pc::transform;
 using pc::twiddle;
+using tp::slot;
 
 // A groups of the y axis; x as P lanes of Q points, z as AZ BZ (first step BZ).
 template <int N>
@@ -61,46 +62,14 @@ FFT3D_TPR(120, 5, 12, 6, 96)
 FFT3D_TPR(128, 4, 16, 8, 96)
 #undef FFT3D_TPR
 
-// Row j lies at j RP, its points and bins in natural order (one pad in 16 where
-// Q is a power of two), so that each step's items read and write one set of slots
-// and the bins of a column step lie side by side.  RP: the least extra wavefronts
-// of the two other patterns, lanes along m (j RP + m Q) and lanes along j.
-template <bool PAD>
-FFT3D_HD constexpr int slot(int p) {
-  return PAD ? p + p / 16 : p;
-}
-template <bool PAD>
-constexpr int row_pitch(int B, int P, int Q, int points) {
-  int best = 0, least = 1 << 20;
-  for (int rp = slot<PAD>(points - 1) + 1, i = 0; i < 16; ++i, ++rp) {
-    int total = 0;
-    for (int pat = 0; pat < 2; ++pat)
-      for (int h = 0; h < 8; ++h) {
-        int n[16] = {}, worst = 0;
-        for (int l = 0; l < 16; ++l) {
-          const int e = h * 16 + l;
-          const int at = pat == 0 ? e / P * rp + slot<PAD>(e % P * Q) : e % B * rp + e / B;
-          const int c = ++n[at % 16];
-          worst = c > worst ? c : worst;
-        }
-        total += worst - 1;
-      }
-    if (total * 64 + i < least) {
-      least = total * 64 + i;
-      best = rp;
-    }
-  }
-  return best;
-}
-
 template <int N>
 struct Dims {
   static constexpr int L = N / 2, HX = L + 1;
   static constexpr int A = Split<N>::A, B = N / A;
   static constexpr int P = Split<N>::P, Q = L / P, AZ = Split<N>::AZ, BZ = N / AZ;
   static_assert(A * B == N && P * Q == L && AZ * BZ == N, "splits");
-  static constexpr bool PAD = (Q & (Q - 1)) == 0;
-  static constexpr int RP = row_pitch<PAD>(B, P, Q, HX);
+  static constexpr tp::Layout rows = tp::row_layout(B, P, Q, HX);
+  static constexpr int PD = rows.PD, RP = rows.RP;
   static constexpr int T1 = Split<N>::T;
   static constexpr size_t smem1 = sizeof(float2) * (size_t)B * RP;
   // columns: point (kz2, m1, n1) of column q at kz2 ZP + (m1 A + n1) W + q
@@ -116,7 +85,7 @@ template <int N>
 __global__ void __launch_bounds__(Dims<N>::T1) rows_fwd_kernel(const __grid_constant__ RealPassArgs a) {
   using D = Dims<N>;
   constexpr int A = D::A, B = D::B, L = D::L, P = D::P, Q = D::Q, T = D::T1;
-  constexpr bool PAD = D::PAD;
+  constexpr int PD = D::PD;
   extern __shared__ __align__(16) float2 sm[];
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const unsigned zz = blockIdx.x / A;  // plane
@@ -136,8 +105,7 @@ __global__ void __launch_bounds__(Dims<N>::T1) rows_fwd_kernel(const __grid_cons
     transform<Q, -1>(v);
     float2* x = sm + j * D::RP;
 #pragma unroll
-    for (int k = 0; k < Q; ++k)
-      x[slot<PAD>(m * Q + k)] = k ? twiddle<-1>(v[k], __ldg(a.tx + k * P + m)) : v[k];
+    for (int k = 0; k < Q; ++k) x[slot(PD, m * Q + k)] = k ? twiddle<-1>(v[k], __ldg(a.tx + k * P + m)) : v[k];
   }
   __syncthreads();
   // second step, in place: item (k, j), lanes along j
@@ -147,17 +115,17 @@ __global__ void __launch_bounds__(Dims<N>::T1) rows_fwd_kernel(const __grid_cons
     float2* x = sm + e % B * D::RP;
     float2 v[P];
 #pragma unroll
-    for (int i = 0; i < P; ++i) v[i] = x[slot<PAD>(Q * i + k)];
+    for (int i = 0; i < P; ++i) v[i] = x[slot(PD, Q * i + k)];
     transform<P, -1>(v);
 #pragma unroll
-    for (int i = 0; i < P; ++i) x[slot<PAD>(Q * i + k)] = v[i];
+    for (int i = 0; i < P; ++i) x[slot(PD, Q * i + k)] = v[i];
   }
   __syncthreads();
 #pragma unroll 1
   for (int kx = threadIdx.x; kx < D::HX; kx += T) {
     // X[k] = (Z[k] + conj Z[L-k]) / 2 - i W_N^k (Z[k] - conj Z[L-k]) / 2, Z[L] = Z[0]
     const int k = kx == L ? 0 : kx, mk = k == 0 ? 0 : L - k;
-    const float2 *xu = sm + slot<PAD>(k), *xm = sm + slot<PAD>(mk);
+    const float2 *xu = sm + slot(PD, k), *xm = sm + slot(PD, mk);
     const float2 w = __ldg(a.twr + kx);
     float2 v[B];
 #pragma unroll
@@ -179,7 +147,7 @@ template <int N>
 __global__ void __launch_bounds__(Dims<N>::T1) rows_inv_kernel(const __grid_constant__ RealPassArgs a) {
   using D = Dims<N>;
   constexpr int A = D::A, B = D::B, L = D::L, P = D::P, Q = D::Q, T = D::T1;
-  constexpr bool PAD = D::PAD;
+  constexpr int PD = D::PD;
   extern __shared__ __align__(16) float2 sm[];
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const unsigned zz = blockIdx.x / A;
@@ -196,7 +164,7 @@ __global__ void __launch_bounds__(Dims<N>::T1) rows_inv_kernel(const __grid_cons
 #pragma unroll
     for (int i = 1; i < B; ++i) v[i] = twiddle<1>(v[i], a.ty[i * A + n1]);
     transform<B, 1>(v);
-    float2* x = sm + slot<PAD>(kx);
+    float2* x = sm + slot(PD, kx);
 #pragma unroll
     for (int j = 0; j < B; ++j) x[j * D::RP] = v[j];
   }
@@ -212,8 +180,8 @@ __global__ void __launch_bounds__(Dims<N>::T1) rows_inv_kernel(const __grid_cons
     float2 u[P], m[P];
 #pragma unroll
     for (int i = 0; i < P; ++i) {
-      u[i] = x[slot<PAD>(n + Q * i)];
-      m[i] = x[slot<PAD>(L - n - Q * i)];
+      u[i] = x[slot(PD, n + Q * i)];
+      m[i] = x[slot(PD, L - n - Q * i)];
     }
     if (n == 0) u[0].y = m[0].y = 0.0f;
 #pragma unroll
@@ -227,7 +195,7 @@ __global__ void __launch_bounds__(Dims<N>::T1) rows_inv_kernel(const __grid_cons
     transform<P, 1>(u);
 #pragma unroll
     for (int k = 0; k < P; ++k)
-      x[slot<PAD>(n + Q * k)] = k ? twiddle<1>(u[k], __ldg(a.tx + n * P + k)) : u[k];
+      x[slot(PD, n + Q * k)] = k ? twiddle<1>(u[k], __ldg(a.tx + n * P + k)) : u[k];
     if (n != 0 && 2 * n != Q) {
       float2 v[P];
 #pragma unroll
@@ -235,7 +203,7 @@ __global__ void __launch_bounds__(Dims<N>::T1) rows_inv_kernel(const __grid_cons
       transform<P, 1>(v);
 #pragma unroll
       for (int k = 0; k < P; ++k)
-        x[slot<PAD>(Q - n + Q * k)] = k ? twiddle<1>(v[k], __ldg(a.tx + (Q - n) * P + k)) : v[k];
+        x[slot(PD, Q - n + Q * k)] = k ? twiddle<1>(v[k], __ldg(a.tx + (Q - n) * P + k)) : v[k];
     }
   }
   __syncthreads();
@@ -247,7 +215,7 @@ __global__ void __launch_bounds__(Dims<N>::T1) rows_inv_kernel(const __grid_cons
     const float2* x = sm + j * D::RP;
     float2 v[Q];
 #pragma unroll
-    for (int i = 0; i < Q; ++i) v[i] = x[slot<PAD>(Q * k + i)];
+    for (int i = 0; i < Q; ++i) v[i] = x[slot(PD, Q * k + i)];
     transform<Q, 1>(v);
     float2* o = dst + j * (A * L) + k;
 #pragma unroll
