@@ -49,8 +49,15 @@ struct FusedArgs {
   long long timeout_ns;
   const uint32_t* mma_frag;     // tensor-core B fragments (split precisions), or null
   int ngrids;                   // grids of the launch unit
-  HartreeWeight weight;         // real inverse kernels launched by launch_weighted
   float2* aux;                  // a kernel's own workspace (real grids: Nyquist columns), or null
+};
+static_assert(sizeof(FusedArgs) == 128, "tensor maps behind it keep their 128-byte lines");
+
+// Arguments of the weighted real inverse kernels.  (A type of their own: two more
+// words in FusedArgs moved the tensor maps behind it off their 128-byte lines in the
+// parameters: split precision 128^3 x 32 355 -> 375 us.)
+struct alignas(128) WeightedArgs : FusedArgs {
+  HartreeWeight weight;
 };
 
 using LaunchFn = cudaError_t (*)(const FusedArgs&, int grid, cudaStream_t);
@@ -78,7 +85,8 @@ struct KernelInfo {
   int uses_work = 1;            // 0: no ticket counters (nothing to clear before a launch)
   LaunchMapsFn launch_maps = nullptr;  // mixed-edge units on packed buffers (tensor-map kernels)
   const void* func_maps = nullptr;     // its kernel
-  LaunchFn launch_weighted = nullptr;  // real inverse kernels: the input times FusedArgs::weight
+  // real inverse kernels: the input times the weight
+  cudaError_t (*launch_weighted)(const WeightedArgs&, int grid, cudaStream_t) = nullptr;
   const void* func_weighted = nullptr;
 };
 

@@ -348,7 +348,7 @@ int execute_fused_real(fft3d_real_plan p, const void* in, void* out, cudaStream_
     cudaGetLastError();
     return FFT3D_ERR_CUDA;
   }
-  FusedArgs a{};
+  WeightedArgs a{};
   a.in = static_cast<const float2*>(in);
   a.out = static_cast<float2*>(out);
   a.blocks = p->d_blocks;
@@ -362,7 +362,8 @@ int execute_fused_real(fft3d_real_plan p, const void* in, void* out, cudaStream_
   a.ngrids = p->batch;
   a.aux = p->d_aux;
   if (weight) a.weight = *weight;
-  if ((weight ? p->kern.launch_weighted : p->kern.launch)(a, p->grid, s) != cudaSuccess) {
+  if ((weight ? p->kern.launch_weighted(a, p->grid, s) : p->kern.launch(a, p->grid, s)) !=
+      cudaSuccess) {
     cudaGetLastError();
     return FFT3D_ERR_CUDA;
   }

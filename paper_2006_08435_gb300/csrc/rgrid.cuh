@@ -71,6 +71,8 @@
 // Waits are bounded in time and report through the status word.
 #pragma once
 
+#include <type_traits>
+
 #include "rowfft.cuh"
 
 namespace fft3d {
@@ -83,6 +85,9 @@ using mb::mbar_wait_bounded;
 using mb::saddr;
 using mb::warp_wait;
 using rowk::spin_geq;
+
+template <bool WEIGHT>
+using Args = std::conditional_t<WEIGHT, WeightedArgs, FusedArgs>;
 
 template <int N>
 struct Cfg {
@@ -463,7 +468,7 @@ __device__ __forceinline__ void publisher(const FusedArgs& a, unsigned long long
 // energies and gradients at 128^3 x 32 531.7 -> 482.0).
 template <int N, int DIR, bool WEIGHT>
 __global__ void __launch_bounds__(Cfg<N>::T, 1)
-    rgrid_fft3d_kernel(const FusedArgs a, const __grid_constant__ CUtensorMap m0,
+    rgrid_fft3d_kernel(const Args<WEIGHT> a, const __grid_constant__ CUtensorMap m0,
                        const __grid_constant__ CUtensorMap m1) {
   using K = Cfg<N>;
   constexpr int NT = K::NTILE, G = K::GROUPS, H = K::H, HC = K::HC, P = K::P, IPP = K::IPP;
@@ -797,7 +802,7 @@ inline bool encode_pairs(CUtensorMap* m, const void* base, int n, int grids, uns
 }
 
 template <int N, int DIR, bool WEIGHT>
-cudaError_t launch(const FusedArgs& a, int grid, cudaStream_t stream) {
+cudaError_t launch(const Args<WEIGHT>& a, int grid, cudaStream_t stream) {
   if (a.in_ptrs || a.grid_map || a.grid_off) return cudaErrorInvalidValue;
   CUtensorMap m0, m1;
   using K = Cfg<N>;

@@ -39,10 +39,15 @@
 // that the next grid's reads meet L2 rather than HBM.
 #pragma once
 
+#include <type_traits>
+
 #include "persistent.cuh"
 
 namespace fft3d {
 namespace rwg {
+
+template <bool WEIGHT>
+using Args = std::conditional_t<WEIGHT, WeightedArgs, FusedArgs>;
 
 template <int N>
 struct Cfg {
@@ -155,7 +160,7 @@ __global__ void __launch_bounds__(Cfg<N>::T, Cfg<N>::MINB_F) rwholegrid_fwd_kern
 // 55.6 / 49.9, 16^3 x 4096 38.1 / 35.2; a seed pass of its own reads and writes
 // the spectra once more).
 template <int N, bool WEIGHT>
-__global__ void __launch_bounds__(Cfg<N>::T, Cfg<N>::MINB_I) rwholegrid_inv_kernel(const FusedArgs a) {
+__global__ void __launch_bounds__(Cfg<N>::T, Cfg<N>::MINB_I) rwholegrid_inv_kernel(const Args<WEIGHT> a) {
   using K = Cfg<N>;
   constexpr int H = K::H, HC = K::HC;
   extern __shared__ __align__(16) float2 S[];
@@ -259,7 +264,7 @@ __global__ void __launch_bounds__(Cfg<N>::T, Cfg<N>::MINB_I) rwholegrid_inv_kern
 }
 
 template <int N, int DIR, bool WEIGHT>
-cudaError_t launch(const FusedArgs& a, int grid, cudaStream_t stream) {
+cudaError_t launch(const Args<WEIGHT>& a, int grid, cudaStream_t stream) {
   grid = grid < a.ngrids ? grid : a.ngrids;  // one block per grid at most
   if (DIR < 0)
     rwholegrid_fwd_kernel<N><<<grid, Cfg<N>::T, Cfg<N>::smem, stream>>>(a);
