@@ -19,7 +19,7 @@ split FP16), tensor_core_kinds (split BF16, FP16, block floating point
 FP16, split FP8, FP8 on the same batch), real_r2c_fp32 / real_c2r_fp32 (real grids),
 real_16cubed_fp32 (16^3 x 16384 real grids), w64x256 (64^3 x 256 in FP32 and
 split FP16), mixed_c2 (64 mixed-edge grids, forward + inverse in one CUDA
-graph), general_path (256^3 and a non-cubic batch on the per-axis passes), hartree
+graph), general_path (256^3 in three passes and a non-cubic batch in two), hartree
 (energy + gradient of real densities, the differentiation workload; one
 density also replayed from a captured CUDA graph)
 and batch1 (one grid per launch, L2 flushed, the paper's setting).
@@ -46,13 +46,13 @@ sys.path.insert(0, ROOT)
 WORKLOADS = {
     "128x32": (128, 32),
     "64x256": (64, 256),
-    # smaller cases of the same kernels for ncu captures (inputs still > L2)
+    # smaller cases for ncu captures (inputs still > L2), of the same kernels but
+    # 64x64 (two passes)
     "128x16": (128, 16),
     "64x64": (64, 64),
     "64x128": (64, 128),
-    # the general path (edges without a fused kernel), for profiler captures
+    # the general path, for profiler captures: three passes, two passes
     "256x2": (256, 2),
-    # the thread-pair kernel (96^3), for profiler captures
     "96x16": (96, 16),
 }
 METRIC = "batched 3D FFT transforms/s and % of HBM roofline at 64^3/128^3 (FP32 vs split-FP16)"
@@ -66,8 +66,15 @@ _COMMON_SOURCES = ["paper_2006_08435_gb300/csrc/persistent.cuh",
 KERNEL_SOURCES = {128: ["paper_2006_08435_gb300/csrc/splity.cuh"] + _COMMON_SOURCES,
                   64: ["paper_2006_08435_gb300/csrc/rowfft2.cuh"] + _COMMON_SOURCES}
 KERNEL_NAMES = {128: "splity_fft3d_kernel<128,-1>", 64: "rowfft2_fft3d_kernel<64,-1>",
-                256: "axis_pass_kernel<-1,2> (general path, three passes)",
                 96: "pairfft_fft3d_kernel<96,-1>"}
+
+
+def kernel_name(n: int, variant: int) -> str:
+    """The kernels of a uniform FP32 plan (variant 10: the general path)."""
+    if variant == 10:
+        return ("pencil_kernel (three passes)" if n == 256
+                else f"pass1_kernel<{n},-1>, pass2_kernel<{n},-1>")
+    return KERNEL_NAMES.get(n, "fused_fft3d_kernel")
 
 
 def dist_env():
@@ -655,7 +662,7 @@ def run_ours(args, ws, rank, local):
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic,
                      "peak_source": f"{peak_kind} hbm_gbs",
-                     "kernel": KERNEL_NAMES.get(n, "fused_fft3d_kernel"),
+                     "kernel": kernel_name(n, plan.variant),
                      "bytes_per_launch": bytes_per_launch,
                      "avg_launch_ms": avg_launch_ms,
                      "median_launch_ms": statistics.median(launch_ms),

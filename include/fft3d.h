@@ -92,7 +92,7 @@ enum {
  * Cubic grids of edge 16, 32, 48, 64, 80, 96 or 128 have fused single-launch
  * kernels (and the tensor-core precisions at 64 and 128); every other grid,
  * cubic or not (nx, ny, nz each supported), runs on the general path: one
- * pencil pass per axis (FP32).
+ * pencil pass per axis, or two passes where the lengths split (FP32).
  */
 int fft3d_size_supported(int n);
 
@@ -292,7 +292,8 @@ int fft3d_selftest_wait_timeout(int64_t timeout_ns);
  * selectable for those too): per chunk of grids that fits L2, the x pass
  * (in -> out) and the y and z passes in place on out, each a batched 1D
  * transform of the pencils of one axis, split into two register codelets
- * (cubic edges 48, 60, 64, 72, 80, 90, 96, 100, 108 and 128: two passes);
+ * (cubic edges 48, 60, 64, 72, 80, 90, 96, 100, 108 and 128, and boxes whose
+ * y axis splits into few groups of 10 to 32: two passes);
  * the launches of a batch above 40 MB alternate between the caller's stream
  * and a side stream of the plan, forked and joined by events (in a captured
  * graph, parallel branches). Mixed plans:
@@ -460,10 +461,10 @@ typedef struct fft3d_real_plan_s* fft3d_real_plan;
  *               (half spectrum -> real).
  *   norm      : fft3d_norm (1/n^3 or 1/sqrt(n^3) on the output).
  * Validates its arguments before touching the GPU.  Owns its device memory,
- * allocated here and freed by fft3d_real_plan_destroy: at n = 64 and 128
- * in FP32 a schedule, counters and (forward) batch * n * n/2 complex64
- * points of workspace, at n = 16 and 32 a status word only; at the other
- * edges above 2 in FP32 twiddle tables and (inverse) the half spectra of the
+ * allocated here and freed by fft3d_real_plan_destroy: for inverses of 100
+ * grids and more at n = 64, of 48 and more at 128, in FP32 a schedule and
+ * counters, at n = 16 and 32 a status word only; at the other edges and
+ * batches above 2 in FP32 twiddle tables and (inverse) the half spectra of the
  * grids in flight (about 75 MB, or two grids if those are larger); elsewhere
  * a complex plan of ceil(batch/2) grids and a workspace of ceil(batch/2) *
  * n^3 complex64 points.  The environment variable
@@ -475,9 +476,10 @@ int fft3d_real_plan_create(int n, int batch, int precision, int direction, int n
 /*
  * As fft3d_real_plan_create with FFT3D_FORWARD and FFT3D_NORM_NONE in FP32,
  * for spectra whose bits must not depend on the library's choice of kernel:
- * the dedicated kernels at n = 16, 32, 64 and 128, elsewhere the pair scheme
- * over complex transforms of one fixed arithmetic order.  The Hartree energy,
- * which is returned in FP64, is taken from these.
+ * the dedicated kernels at n = 16, 32, 64 and 128 (at 64 and 128 with a
+ * schedule, counters and batch * n * n/2 complex64 points of workspace),
+ * elsewhere the pair scheme over complex transforms of one fixed arithmetic
+ * order.  The Hartree energy, which is returned in FP64, is taken from these.
  */
 int fft3d_real_plan_create_fixed(int n, int batch, fft3d_real_plan* out_plan);
 
@@ -486,8 +488,9 @@ int fft3d_real_plan_create_fixed(int n, int batch, fft3d_real_plan* out_plan);
  * 16-byte aligned, not overlapping (forward: in = real grids, out = half
  * spectra; inverse: the other way round).  Asynchronous on `stream`,
  * allocates nothing, capturable in a CUDA graph (one kernel at n = 16 and
- * 32, a counter reset and one kernel at n = 64 and 128 in FP32, one kernel
- * per pass and chunk at the other edges; in the pair scheme a packing or
+ * 32, a counter reset and one kernel in large inverses at n = 64 and 128 in
+ * FP32, else one kernel per pass and chunk, those of a batch above 40 MB on two
+ * branches; in the pair scheme a packing or
  * rebuilding kernel, the complex plan's launch, a separating or splitting
  * kernel).  A plan may run on one stream at a time.
  */

@@ -91,8 +91,7 @@ struct KernelInfo {
 };
 
 // ---------------------------------------------------------------- general path
-// Pencil passes for any edge 2..kAxisMaxLen with prime factors 2, 3, 5, one
-// axis at a time (axis.cu).
+// Passes for any edge 2..kAxisMaxLen with prime factors 2, 3, 5 (passes.cu).
 constexpr int kAxisMaxLen = 512;
 constexpr int kGeneralVariant = 10;  // plan variant of the general path
 constexpr int kFixedVariant = 11;    // the same as three passes at every edge (internal)
@@ -211,9 +210,10 @@ BoxKernel box2_kernel_info(int A, int nz, int dir);
 cudaError_t launch_box(const BoxKernel& k, unsigned grid, size_t smem, int cluster, const BoxArgs& a,
                        cudaStream_t s);
 
-// A 3D transform as three pencil passes (passes.cu): complex grids (x, y, z,
-// out of place or in place; as two passes at some cubic edges unless `fixed`), real grids to half spectra (x, y, z) or back
-// (z into a workspace of work_points() complex points, y, x).
+// A 3D transform as three pencil passes or two (passes.cu): complex grids (x, y,
+// z, out of place or in place; always three if `fixed`), real grids to half
+// spectra (x, y, z) or back (z into a workspace of work_points() complex points,
+// y, x).
 constexpr int kMaxChains = 2;
 enum PassKind { kPassC2C = 0, kPassR2C = 1, kPassC2R = 2 };
 struct AxisPasses {

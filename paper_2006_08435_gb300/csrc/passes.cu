@@ -1,7 +1,8 @@
 // The general path's schedule: a 3D transform as one pencil pass per axis
-// (pencil.cuh), or two passes at some cubic edges (twopass.cuh), over chunks of grids -- or, for a grid beyond the chunk
-// budget, ranges of its planes for x and y -- whose intermediate stays in
-// L2 from one pass to the next.
+// (pencil.cuh), or in two passes where there are kernels for the lengths (cubic
+// edges twopass.cuh, boxes twopass_box.cuh, real grids twopass_real.cuh), over
+// chunks of grids -- or, for a grid beyond the chunk budget, ranges of its planes
+// for x and y -- whose intermediate stays in L2 from one pass to the next.
 //
 // Three passes move 48 bytes per point through L2 (in-place copies of
 // 37 .. 75 MB run at 12.5 TB/s there once started), but a launch of a few

@@ -44,9 +44,9 @@
 // odd pitch, and the lanes of a warp are rows -- no bank conflicts, one n1 or
 // k2 (one branch of the split, one twiddle) per half-warp, where lanes along
 // the row took 5 to 8 short runs per access and both branches (10 grids of
-// 96^3: L1 wavefronts of the forward x pass 5.0 -> 2.9 M, 21.5 -> 15.6 us;
-// 96^3 x 32 forward 107 -> 93, inverse 106 -> 101 us; 100^3 x 16 64 -> 55, 60 ->
-// 59).  Complex rows do better without (256^3 x 4 419 us, staged 489).
+// 96^3: L1 wavefronts of the forward x pass 5.0 -> 2.9 M, 21.5 -> 15.6 us; the
+// three passes of 96^3 x 32 forward 107 -> 93, inverse 106 -> 101 us; 100^3 x 16 64 ->
+// 55, 60 -> 59).  Complex rows do better without (256^3 x 4 419 us, staged 489).
 #pragma once
 
 #include <cuda_runtime.h>

@@ -182,8 +182,8 @@ static bool fused_size(int n) { return fused_slot(n) >= 0; }
 // two-plane items).  Tensor-core precisions: 0 the plain persistent kernel,
 // 9 the tensor-TMA items with tcgen05 products (64^3 two-plane, 128^3
 // split-y).
-// Variant 10 (kGeneralVariant): the general path, one pencil pass per axis
-// (passes.cu), the only one for non-cubic grids and edges without a fused
+// Variant 10 (kGeneralVariant): the general path, one pencil pass per axis or
+// two passes (passes.cu), the only one for non-cubic grids and edges without a fused
 // kernel, selectable for the others.  Mixed plans: 0 one
 // launch of the mixed-edge kernel, 1 one launch per distinct edge with that
 // edge's default kernel, 2 the launches of 1 on two concurrent branches.
@@ -206,8 +206,8 @@ std::vector<int> variant_candidates(bool mixed, int n, int precision) {
 // (back-to-back executes):
 //   16^3: cluster-fused below 128 grids, whole grid per block from 128;
 //   32^3: cluster-fused below 48 grids, pencil passes below 300, thread pairs;
-//   48^3: two passes; 64^3, 80^3, 96^3, 128^3: two passes (below 80, 150, 36 and
-//     20 grids), then two-plane (64), thread pairs (80, 96), split-y (128);
+//   48^3: two passes; 64^3, 80^3, 96^3, 128^3: two passes (below 88, 64, 28 and
+//     16 grids), then two-plane (64), thread pairs (80, 96), split-y (128);
 //   tensor-core precisions: the plain persistent kernel (mma.sync) for few
 //     grids, the tcgen05 kernels from 16 (64^3) and 2 (128^3) grids.
 int builtin_default_variant(bool mixed, int n, int batch, int precision) {

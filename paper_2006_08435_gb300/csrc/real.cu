@@ -17,15 +17,18 @@
 // spectra A, B are rebuilt as one full spectrum H(A) + i H(B), transformed
 // once, and the real and imaginary parts of the result are the two grids.
 //
-// At 16^3 .. 128^3 in FP32 the transforms run instead as dedicated kernels
-// with half-length row transforms: at 16^3 and 32^3 a whole grid per block
-// (rwholegrid.cuh), at 64^3 and 128^3 two phases (rgrid.cuh: one pass over
-// the real grid and one over the half spectrum, a workspace of n^2/2
-// complex per grid for the Nyquist column of the forward transform), at the
-// other edges above 2 as one pencil pass per axis (passes.cu): 24 bytes per
-// real point through L2 where the pair scheme moves about 60 and makes the
-// passes of a whole complex transform (96^3 x 32, forward + inverse 333 ->
-// 194 us, 100^3 x 16 286 -> 114, 20^3 x 500 373 -> 45).  The pair scheme
+// In FP32 the transforms run instead as kernels with half-length row
+// transforms: at 16^3 and 32^3 a whole grid per block
+// (rwholegrid.cuh), at eleven edges from 48 to 128 in two passes
+// (twopass_real.cuh), at the other edges above 2 as one pencil pass per axis
+// (passes.cu): 24 bytes per real point through L2 (two passes 16) where the pair
+// scheme moves about 60 and makes the passes of a whole complex transform
+// (96^3 x 32, forward + inverse 333 -> 190 us on pencils, 141 in two passes;
+// 20^3 x 500 373 -> 45 on pencils).  Large inverses at 64^3 and 128^3, and
+// spectra whose bits are to stay, run on persistent kernels of two phases
+// (rgrid.cuh: one pass over the real grid and one over the half spectrum, a
+// workspace of n^2/2 complex per grid for the Nyquist column of the forward
+// transform).  The pair scheme
 // remains for n = 2 and the tensor-core precisions; its kernels here move
 // data only (pack, separate, rebuild, split) and its transforms are the
 // library's complex plans.  Packing two grids into one makes each grid's
@@ -48,7 +51,7 @@ struct fft3d_real_plan_s {
   // pair scheme
   fft3d_plan inner = nullptr;  // complex plan of `pairs` n^3 grids
   float2* d_work = nullptr;    // pairs * n^3 complex points
-  // pencil passes (passes.cu); the inverse keeps a chunk of spectra in d_work
+  // pencil or two passes (passes.cu); the inverse keeps a chunk of spectra in d_work
   bool pencils = false;
   fft3d::AxisPasses passes;
   // dedicated kernels (rgrid.cuh)
@@ -305,7 +308,8 @@ int create_fused_real(int n, int batch, int direction, int norm, const KernelInf
   return FFT3D_SUCCESS;
 }
 
-// Plan of the pencil passes: every even edge above 2 without a dedicated kernel.
+// Plan of the pencil or two passes: every even edge above 2 without a dedicated kernel,
+// and 64^3 and 128^3 where they are faster than it.
 int create_pencil_real(int n, int batch, int direction, int norm, fft3d_real_plan* out_plan) {
   int dev = -1, l2 = 0, major = 0, minor = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||

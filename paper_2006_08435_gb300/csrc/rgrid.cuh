@@ -1,4 +1,5 @@
-// Persistent transforms of REAL n^3 grids (n = 64, 128): forward (R2C, sign -1, real
+// Persistent transforms of REAL n^3 grids (n = 64, 128; the default of large
+// inverses and of the Hartree energy's spectra, two_pass_real in real.cu): forward (R2C, sign -1, real
 // grid -> half spectrum kx = 0 .. n/2) and inverse (C2R, sign +1), each in
 // two phases of work items with the ticket schedule and L2-resident
 // intermediate of the complex kernels.  Every 1D transform of n points is

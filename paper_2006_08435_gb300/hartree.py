@@ -6,8 +6,9 @@ gradient dE_H/drho = (Omega/n^3) V_H is the adjoint (inverse, unnormalised)
 transform of the seed s F(rho) / |m|^2.  Every step runs in the library's
 kernels.  For even n (the usual grids) the density being real, the path
 works on half spectra: real-grid forward transform, FP64 energy reduction
-over the half spectrum (mirrored points counted twice); seed on the half
-spectrum, real-grid inverse transform.  For odd n: real->complex, complex
+over the half spectrum (mirrored points counted twice); for the gradient one
+real-grid inverse transform that multiplies by s / |m|^2 as it reads the half
+spectrum.  For odd n: real->complex, complex
 forward transform, full-spectrum reduction; seed, complex inverse,
 complex->real.  To capture a step in a CUDA graph, run it once eagerly
 first with the same shapes and stream: that call allocates the reduction
