@@ -422,7 +422,8 @@ def run_ours(args, ws, rank, local):
             msr = max_over_ranks(r0.elapsed_time(r1) / kr, ws, dev)
             assert rplan.device_status() == 0
             real[name] = {"value": whole_job_rate(ws, batch, 1, msr), "unit": "transforms/s",
-                          "steps": kr, "ms_per_step": msr, "launches_per_step": 1,
+                          "steps": kr, "ms_per_step": msr,
+                          "launches_per_step": "2 per chunk of grids (64^3, 128^3: two passes)",
                           "bytes_per_transform": 4 * n ** 3 + 8 * n * n * (n // 2 + 1)}
             del rplan
         del xr, yr, br
@@ -609,7 +610,8 @@ def run_ours(args, ws, rank, local):
                 "value": whole_job_rate(ws, bg, 1, msg), "unit": "transforms/s", "steps": kg,
                 "ms_per_step": msg, "variant": pg.variant,
                 "roofline_frac": 16.0 * pts_g / (msg / 1e3) / 1e9 / peak,
-                "frac_of_pass_traffic": 48.0 * pts_g / (msg / 1e3) / 1e9 / peak}
+                # 16 bytes per point and pass: 256^3 three passes, the box two
+                "frac_of_pass_traffic": (48.0 if nx_ == 256 else 32.0) * pts_g / (msg / 1e3) / 1e9 / peak}
             del xg, yg, pg
 
     # the paper's setting: one grid per transform (Table 1), latency of

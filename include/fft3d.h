@@ -267,7 +267,8 @@ int fft3d_selftest_wait_timeout(int64_t timeout_ns);
 
 /*
  * The kernel variant a plan uses (written to *variant).  Single-edge FP32
- * plans (each variant the fastest for some edge and batch on the GB300):
+ * plans (each variant the fastest for some edge and batch on the GB300, or in
+ * a mixed plan):
  * 0 plain persistent kernel, 1 the same with twice the threads per block
  * (16^3 .. 96^3), 3 the cluster-fused single-pass kernel (16^3, 32^3), 12
  * a whole 16^3 grid per block (three passes of thread-per-pencil 16-point

@@ -174,7 +174,7 @@ static void umma_b_table(int prec, uint16_t* out /* 8192 */) {
 static bool fused_size(int n) { return fused_slot(n) >= 0; }
 
 // Kernel variants of a single-size FP32 plan (each the fastest for some
-// edge and batch on the GB300): 0 plain persistent kernel, 1 the same with
+// edge and batch on the GB300, or in a mixed plan): 0 plain persistent kernel, 1 the same with
 // twice the threads (16^3 to 96^3), 3 the cluster-fused single-pass kernel
 // (16^3, 32^3), 12 a whole 16^3 grid per block, 4 the double-buffered persistent kernel (32^3, 48^3, 80^3,
 // 96^3), 5 the warp-owned two-phase kernel (64^3, 128^3), 6 to 8 the
