@@ -53,9 +53,12 @@ __device__ __forceinline__ unsigned udiv(unsigned x, FastDiv d) {
 // threads sum the grid's partials together (one thread reading them one
 // after another took 38 us for the 512 partials of one 128^3 grid).
 // The spectrum is read as a flat array, U points per thread per step at a
-// grid stride (every warp load 256 consecutive bytes); a point's (kz, ky,
-// kx) come from its index by multiply-shift divisions by the row length
-// and by n.  (Rows of n/2 + 1 points taken one warp at a time left a
+// grid stride (every warp load 256 consecutive bytes); a thread's first (kz,
+// ky, kx) come from its index by multiply-shift divisions by the row length
+// and by n, the next from the stride's by additions with carry, as floats,
+// which hold them and |m|^2 < 2^24 exactly (32 grids of 128^3: 64.5 us, of which
+// the read alone takes 40; 73.7 with two divisions and a conversion per point;
+// the same bits).  (Rows of n/2 + 1 points taken one warp at a time left a
 // third pass over each row with one lane of 32 busy: 0.41 of the HBM
 // bandwidth at 32 grids of 128^3.)  Each term |F(m)|^2 w / |m|^2 is
 // formed in FP32 (the approximate reciprocal of |m|^2: one instruction
@@ -66,8 +69,11 @@ __device__ __forceinline__ unsigned udiv(unsigned x, FastDiv d) {
 // accumulated in FP64: FP64 work is a few operations per hundred points,
 // since FP64 runs at a small fraction of the FP32 rate on this GPU (the
 // per-point FP64 form ran at 0.39 TB/s).
+// The number of blocks sets which terms are summed together, so it is a fixed
+// kEnergyBlocks per multiprocessor.
+constexpr int kEnergyBlocks = 6;
 template <bool HALF>
-__global__ void __launch_bounds__(kRedThreads) hartree_energy_kernel(
+__global__ void __launch_bounds__(kRedThreads, kEnergyBlocks) hartree_energy_kernel(
     const float2* __restrict__ f, int n, long long npts, double half_s,
     double* __restrict__ partials, unsigned* __restrict__ counters, double* __restrict__ energy,
     FastDiv div_h, FastDiv div_n) {
@@ -76,8 +82,14 @@ __global__ void __launch_bounds__(kRedThreads) hartree_energy_kernel(
   constexpr int W = kRedThreads / 32, U = 8;  // points per thread per step
   const int h = HALF ? n / 2 + 1 : n;
   const unsigned np = (unsigned)npts, stride = gridDim.x * kRedThreads;
+  const unsigned first = blockIdx.x * kRedThreads + threadIdx.x;
+  const unsigned row = udiv(first, div_h), srow = udiv(stride, div_h);
+  const unsigned z = udiv(row, div_n), sz = udiv(srow, div_n);
+  float kx = (float)(first - row * h), ky = (float)(row - z * n), kz = (float)z;
+  const float sx = (float)(stride - srow * h), sy = (float)(srow - sz * n), szf = (float)sz;
+  const float fh = (float)h, fn = (float)n;
   double acc = 0.0;
-  for (unsigned i0 = blockIdx.x * kRedThreads + threadIdx.x; i0 < np; i0 += U * stride) {
+  for (unsigned i0 = first; i0 < np; i0 += U * stride) {
     float2 v[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -87,14 +99,23 @@ __global__ void __launch_bounds__(kRedThreads) hartree_energy_kernel(
     float part = 0.0f;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const unsigned i = i0 + u * stride;
-      const unsigned row = udiv(i, div_h), kz = udiv(row, div_n);
-      const int kx = (int)(i - row * h), ky = (int)(row - kz * n);
-      const int mx = signed_index(kx, n), my = signed_index(ky, n), mz = signed_index((int)kz, n);
-      const int m2 = mx * mx + my * my + mz * mz;
-      const float w = HALF && kx != 0 && 2 * kx != n ? 2.0f : 1.0f;
-      if (i < np && m2 > 0)
-        part = fmaf(fmaf(v[u].x, v[u].x, v[u].y * v[u].y), w * rcp_approx((float)m2), part);
+      // |m| per axis; past the last point v is 0 and so is its term
+      const float mx = HALF ? kx : fminf(kx, fn - kx), my = fminf(ky, fn - ky), mz = fminf(kz, fn - kz);
+      const float m2 = fmaf(mx, mx, fmaf(my, my, mz * mz));
+      const float w = HALF && kx != 0.0f && 2.0f * kx != fn ? 2.0f : 1.0f;
+      if (m2 > 0.0f)
+        part = fmaf(fmaf(v[u].x, v[u].x, v[u].y * v[u].y), w * rcp_approx(m2), part);
+      kx += sx;
+      ky += sy;
+      kz += szf;
+      if (kx >= fh) {
+        kx -= fh;
+        ky += 1.0f;
+      }
+      if (ky >= fn) {
+        ky -= fn;
+        kz += 1.0f;
+      }
     }
     acc += (double)part;
   }
@@ -182,7 +203,7 @@ int resident_blocks() {
       cudaGetLastError();
       return 2048;
     }
-    return sms * per_sm;
+    return sms * (SEED ? per_sm : std::min(per_sm, kEnergyBlocks));
   }();
   return r;
 }
