@@ -204,6 +204,7 @@ struct BoxKernel {
   int threads = 0;
   size_t smem = 0;  // pass 1: per row
   int split = 0;    // AX or AZ
+  int threads32 = 0;  // pass 1: threads for 32 rows
 };
 BoxKernel box1_kernel_info(int nx, int dir);         // func null: none
 BoxKernel box2_kernel_info(int A, int nz, int dir);

@@ -143,6 +143,7 @@ int AxisPasses::create(PassKind kind_, int nx_, int ny_, int nz_, int batch_, in
           cudaGetLastError();
           return FFT3D_ERR_CUDA;
         }
+      if (ny / A == 32) box[0].threads = box[0].threads32;
       BoxArgs& b = box_args;
       b = BoxArgs{};
       b.A = A;

@@ -26,7 +26,7 @@
 // two passes with padded rows of their own splits / now: 60^3 x 129 - / 140 / 123;
 // 72^3 x 75 - / 135 / 120; 80^3 x 54 - / 129 / 118; 90^3 x 38 - / 174 / 137; 108^3 x 22
 // - / 155 / 129; 100^3 x 16 94 / 86 / 79; 48^3 x 400 - / 191 / 169; 64^3 x 64 90.3 / 74.6 /
-// 72.4; 96^3 x 8 44.2 / 33.6 / 34.5; 128^3 x 8 92.7 / 78.7 / 80.5.
+// 72.4; 96^3 x 31 - / 126 / 124; 128^3 x 8 92.7 / 78.7 / 80.5.
 //
 // In place, the A groups of a plane read rows that the others write.  Where their
 // rows take at most 56 KB they are one block (four fit a multiprocessor);
@@ -52,26 +52,26 @@ using pc::transform;
 using pc::twiddle;
 
 // Splits of an edge: y into A groups of B; x and z into two register steps,
-// BX (BZ) points first, AX (AZ) apart, then AX (AZ).
+// BX (BZ) points first, AX (AZ) apart, then AX (AZ); T threads of pass 1.
 template <int L>
 struct Cfg;
-#define FFT3D_TP(L_, A_, AX_, AZ_)                                      \
+#define FFT3D_TP(L_, A_, AX_, AZ_, T_)                                  \
   template <>                                                           \
   struct Cfg<L_> {                                                      \
     static constexpr int L = L_, A = A_, B = L_ / A_;                   \
     static constexpr int AX = AX_, BX = L_ / AX_, AZ = AZ_, BZ = L_ / AZ_; \
-    static constexpr int W = 16; /* columns of a pass-2 block */        \
+    static constexpr int T1 = T_, W = 16; /* W: columns of a pass-2 block */ \
   };
-FFT3D_TP(48, 3, 8, 4)
-FFT3D_TP(60, 4, 12, 4)
-FFT3D_TP(64, 4, 16, 4)
-FFT3D_TP(72, 3, 12, 6)
-FFT3D_TP(80, 4, 16, 4)
-FFT3D_TP(90, 5, 15, 6)
-FFT3D_TP(96, 4, 16, 8)
-FFT3D_TP(100, 5, 10, 5)
-FFT3D_TP(108, 4, 12, 9)
-FFT3D_TP(128, 4, 16, 8)
+FFT3D_TP(48, 3, 8, 4, 64)
+FFT3D_TP(60, 4, 12, 4, 64)
+FFT3D_TP(64, 4, 16, 4, 64)
+FFT3D_TP(72, 3, 12, 6, 96)
+FFT3D_TP(80, 4, 16, 4, 96)
+FFT3D_TP(90, 5, 15, 6, 160)
+FFT3D_TP(96, 4, 16, 8, 192)
+FFT3D_TP(100, 5, 10, 5, 128)
+FFT3D_TP(108, 4, 12, 9, 128)
+FFT3D_TP(128, 4, 16, 8, 128)
 #undef FFT3D_TP
 
 // Rows in shared memory for an x transform in two register steps, P lanes of Q
@@ -120,7 +120,7 @@ struct Dims : Cfg<L> {
   using C = Cfg<L>;
   static constexpr Layout rows = row_layout(C::B, C::AX, C::BX, L);
   static constexpr int PD = rows.PD, RP = rows.RP;
-  static constexpr int T1 = (L + 31) / 32 * 32;
+  using C::T1;
   static constexpr size_t smem1 = sizeof(float2) * (size_t)C::B * RP;
   static constexpr bool MERGED = C::A * smem1 <= 56 * 1024;  // in place: see above
   // pass 2: point (kz2, m1, n1) of column q at kz2 * ZP + (m1 * A + n1) * W + q

@@ -2,7 +2,7 @@
 // per nx, with the points B per thread of its y step chosen at run time, pass 2
 // per (A, nz), ny = A B.  Packed batches; in place with clusters of A blocks.
 // What bounds it and why the steps are split as they are: see twopass.cuh.
-// GB300, us, two passes / three: 96 x 128 x 64, 64 grids 231 / 264; 128 x 96 x
+// GB300, us, two passes / three: 96 x 128 x 64, 64 grids 215 / 264; 128 x 96 x
 // 80 x 16 78 / 88; 75^3 x 20 46 / 59; 135 x 128 x 90 x 4 33.5 / 42; 120^3 x 16 143 /
 // 190 (two passes with tiles of 16 columns of one row k2).
 #pragma once
@@ -36,6 +36,13 @@ struct BoxX {
   static constexpr Layout rows = row_layout(32, AX, BX, LX);  // (any number of rows)
   static constexpr int PD = rows.PD, RP = rows.RP;
   static constexpr int T = LX <= 64 ? 64 : (LX + 31) / 32 * 32;
+  // threads for 32 rows, whose shared memory leaves few blocks: a warp more where
+  // that keeps the lanes of the first step busy (96 x 128 x 64 x 64 231 -> 213 us,
+  // 60 x 128 x 72 x 40 119 -> 107, 90 x 128 x 96 x 20 123 -> 112; not for 64 x 128 x 64 x
+  // 40, a ninth of them idle, 96 -> 99, nor for fewer rows, 108 x 96 x 100 104 -> 110)
+  // and BX is even (odd, 80 x 128 x 64 x 40 117 -> 120, 125 x 128 x 96 x 10 80 -> 85)
+  static constexpr int T32 =
+      AX >= 15 && BX % 2 == 0 && (32 * AX + T + 31) / (T + 32) * (T + 32) * 10 <= 32 * AX * 11 ? T + 32 : T;
 };
 constexpr int kBoxW = 16;  // columns of a pass-2 block
 template <int A, int LZ>
@@ -60,9 +67,10 @@ __device__ __forceinline__ void box_y(const float2* x, int RP, float2* o, int nx
 }
 
 template <int LX, int DIR>
-__global__ void __launch_bounds__(BoxX<LX>::T) box1_kernel(const __grid_constant__ BoxArgs a) {
+__global__ void __launch_bounds__(BoxX<LX>::T32) box1_kernel(const __grid_constant__ BoxArgs a) {
   using D = BoxX<LX>;
-  constexpr int AX = D::AX, BX = D::BX, T = D::T;
+  constexpr int AX = D::AX, BX = D::BX;
+  const int T = blockDim.x;  // D::T or D::T32
   extern __shared__ __align__(16) float2 sm[];
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int A = a.A, B = a.B;
@@ -211,7 +219,7 @@ template <int LX>
 BoxKernel box1_entry(int dir) {
   using D = BoxX<LX>;
   return BoxKernel{dir < 0 ? (const void*)&box1_kernel<LX, -1> : (const void*)&box1_kernel<LX, 1>,
-                   D::T, sizeof(float2) * (size_t)D::RP, D::AX};
+                   D::T, sizeof(float2) * (size_t)D::RP, D::AX, D::T32};
 }
 template <int A, int LZ>
 BoxKernel box2_entry(int dir) {
