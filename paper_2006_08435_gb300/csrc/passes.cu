@@ -133,16 +133,17 @@ int AxisPasses::create(PassKind kind_, int nx_, int ny_, int nz_, int batch_, in
       box[0] = box1_kernel_info(nx, dir);
       box[1] = box2_kernel_info(A, nz, dir);
     }
-    const size_t smem1 = A ? box[0].smem * (size_t)(ny / A) : 0;
-    if (!box[0].func || !box[1].func || smem1 > 72 * 1024) {
+    if (!box[0].func || !box[1].func) {
       box[0] = box[1] = BoxKernel{};
     } else {
-      for (int i = 0; i < 2; ++i)
-        if (cudaFuncSetAttribute(box[i].func, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(i ? box[1].smem : smem1)) != cudaSuccess) {
-          cudaGetLastError();
-          return FFT3D_ERR_CUDA;
-        }
+      // (the limit belongs to the kernel, which plans of several ny share: pass 1,
+      // whose rows are the plan's, stays below the default and leaves it alone)
+      if (box[1].smem > 48 * 1024 &&
+          cudaFuncSetAttribute(box[1].func, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)box[1].smem) != cudaSuccess) {
+        cudaGetLastError();
+        return FFT3D_ERR_CUDA;
+      }
       if (ny / A == 32) box[0].threads = box[0].threads32;
       BoxArgs& b = box_args;
       b = BoxArgs{};

@@ -35,6 +35,7 @@ struct BoxX {
   static constexpr int AX = box_ax(LX), BX = LX / AX;
   static constexpr Layout rows = row_layout(32, AX, BX, LX);  // (any number of rows)
   static constexpr int PD = rows.PD, RP = rows.RP;
+  static_assert(sizeof(float2) * 32 * RP <= 48 * 1024, "32 rows within the default limit");
   static constexpr int T = LX <= 64 ? 64 : (LX + 31) / 32 * 32;
   // threads for 32 rows, whose shared memory leaves few blocks: a warp more where
   // that keeps the lanes of the first step busy (96 x 128 x 64 x 64 231 -> 213 us,
