@@ -163,7 +163,8 @@ int AxisPasses::create(PassKind kind_, int nx_, int ny_, int nz_, int batch_, in
       tab.insert(tab.end(), b.tz, b.tz + nz);
     }
   }
-  for (int a = 0; a < 3 && !two.launch && !real.launch; ++a) {
+  // the pencil passes, where no two passes take their place
+  for (int a = 0; a < 3 && !two.launch && !real.launch && !box[0].func; ++a) {
     k[a] = pencil_kernel_info(len[a], dir, a == 0 ? kx : 0);
     if (!k[a].launch) return FFT3D_ERR_UNSUPPORTED_SIZE;
     if (k[a].smem > 48 * 1024 &&
@@ -287,6 +288,17 @@ cudaError_t AxisPasses::chunk_passes(long long g, const void* in, void* out, flo
     }
     return real.launch(a, (int)m, s);
   }
+  if (box[0].func) {
+    const long long m = std::min(chunk, batch - g);
+    BoxArgs a = box_args;
+    a.in = static_cast<const float2*>(in) + g * pp * nz;
+    a.out = static_cast<float2*>(out) + g * pp * nz;
+    a.in_place = in == out;
+    const cudaError_t e = launch_box(box[0], (unsigned)(m * nz * a.A), box[0].smem * a.B,
+                                     a.in_place ? a.A : 1, a, s);
+    return e != cudaSuccess ? e
+                            : launch_box(box[1], (unsigned)(m * a.tiles), box[1].smem, 1, a, s);
+  }
   // contiguous rows of `planes` planes
   auto x_pass = [&](const float2* src, float2* dst, long long planes) {
     PencilArgs a{};
@@ -341,17 +353,6 @@ cudaError_t AxisPasses::chunk_passes(long long g, const void* in, void* out, flo
     }
     return k[2].launch(a, s);
   };
-  if (box[0].func) {
-    const long long m = std::min(chunk, batch - g);
-    BoxArgs a = box_args;
-    a.in = static_cast<const float2*>(in) + g * pp * nz;
-    a.out = static_cast<float2*>(out) + g * pp * nz;
-    a.in_place = in == out;
-    const cudaError_t e = launch_box(box[0], (unsigned)(m * nz * a.A), box[0].smem * a.B,
-                                     a.in_place ? a.A : 1, a, s);
-    return e != cudaSuccess ? e
-                            : launch_box(box[1], (unsigned)(m * a.tiles), box[1].smem, 1, a, s);
-  }
   // complex points of one grid on the x pass's two sides
   const long long real_pts = (long long)nx / 2 * ny * nz, spec_pts = pp * nz;
   const long long m = std::min(chunk, batch - g);
