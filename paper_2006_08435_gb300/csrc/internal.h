@@ -135,7 +135,8 @@ struct PencilKernel {
   size_t smem = 0;
 };
 // kind: 0 strided, 1 rows, 2 real rows of 2 L points forward (dir -1), 3 the
-// same inverse (dir 1), 4 strided with weights (dir 1, even L); launch is null for an edge that is not plannable.
+// same inverse (dir 1), 4 strided with weights (dir 1, even L), 5 strided for the
+// half spectra of real grids (even L); launch is null for an edge that is not plannable.
 PencilKernel pencil_kernel_info(int L, int dir, int kind);
 
 // Two-pass transforms of cubic edges (twopass.cuh).  tx, ty, tz: W_L^(n1 k) at

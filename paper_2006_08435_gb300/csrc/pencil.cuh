@@ -55,12 +55,13 @@
 
 #include "codelets.cuh"
 #include "internal.h"
+#include "primefactor.cuh"
 
 namespace fft3d {
 namespace pc {
 
-enum { kStrided = 0, kContig = 1, kR2C = 2, kC2R = 3, kWeighted = 4 };
-constexpr bool strided(int kind) { return kind == kStrided || kind == kWeighted; }
+enum { kStrided = 0, kContig = 1, kR2C = 2, kC2R = 3, kWeighted = 4, kStridedReal = 5 };
+constexpr bool strided(int kind) { return kind == kStrided || kind == kWeighted || kind == kStridedReal; }
 
 constexpr bool smooth(int n) {
   if (n < 2) return false;
@@ -260,6 +261,14 @@ __device__ __forceinline__ void split(const float2* twr, float2* dst, const floa
   }
 }
 
+// The kinds of real grids take the prime-factor forms, whose errors are smaller;
+// those of complex grids keep the order of the sums (see split_a).
+template <int R, int DIR, int KIND>
+__device__ __forceinline__ void step(float2* v) {
+  if constexpr (KIND == kStrided || KIND == kContig) transform<R, DIR>(v);
+  else pf::transform<R, DIR>(v);
+}
+
 template <int L, int DIR, int KIND>
 __global__ void __launch_bounds__(Cfg<L, KIND>::T, Cfg<L, KIND>::blocks) pencil_kernel(const PencilArgs a) {
   using C = Cfg<L, KIND>;
@@ -318,7 +327,7 @@ __global__ void __launch_bounds__(Cfg<L, KIND>::T, Cfg<L, KIND>::blocks) pencil_
         u[j] = make_float2(s.x - t.y, s.y + t.x);
         m[j] = make_float2(s.x + t.y, t.x - s.y);
       }
-      transform<B, DIR>(u);
+      step<B, DIR, KIND>(u);
       if constexpr (A > 1) {
         float2* x = sm + c * C::RP;
 #pragma unroll
@@ -328,7 +337,7 @@ __global__ void __launch_bounds__(Cfg<L, KIND>::T, Cfg<L, KIND>::blocks) pencil_
           float2 v[B];
 #pragma unroll
           for (int j = 0; j < B; ++j) v[j] = m[B - 1 - j];
-          transform<B, DIR>(v);
+          step<B, DIR, KIND>(v);
           const int n2 = A - n1;
 #pragma unroll
           for (int k = 0; k < B; ++k)
@@ -363,7 +372,7 @@ __global__ void __launch_bounds__(Cfg<L, KIND>::T, Cfg<L, KIND>::blocks) pencil_
           }
         }
       }
-      transform<B, DIR>(v);
+      step<B, DIR, KIND>(v);
       if constexpr (A > 1) {
 #pragma unroll
         for (int k = 0; k < B; ++k) {
@@ -394,7 +403,7 @@ __global__ void __launch_bounds__(Cfg<L, KIND>::T, Cfg<L, KIND>::blocks) pencil_
 #pragma unroll
       for (int j = 0; j < A; ++j)
         v[j] = sm[strided(KIND) ? (k2 * A + j) * W + c : c * C::RP + k2 * C::AP + j];
-      transform<A, DIR>(v);
+      step<A, DIR, KIND>(v);
       if constexpr (KIND == kR2C) {
         float2* row = so + c * C::SP;
         // the mirrors of this item's outputs are those of B - k2
@@ -404,7 +413,7 @@ __global__ void __launch_bounds__(Cfg<L, KIND>::T, Cfg<L, KIND>::blocks) pencil_
           float2 w[A];
 #pragma unroll
           for (int j = 0; j < A; ++j) w[j] = sm[c * C::RP + (B - k2) * C::AP + j];
-          transform<A, DIR>(w);
+          step<A, DIR, KIND>(w);
           split<L, A>(a.twr, row, v, w, k2);
         }
       } else if constexpr (KIND == kC2R) {
@@ -461,8 +470,10 @@ PencilKernel entry() {
 template <int L>
 PencilKernel entry_of(int dir, int kind) {
   if (kind == kStrided) return dir < 0 ? entry<L, -1, kStrided>() : entry<L, 1, kStrided>();
-  if constexpr (L % 2 == 0)
+  if constexpr (L % 2 == 0) {
     if (kind == kWeighted && dir > 0) return entry<L, 1, kWeighted>();
+    if (kind == kStridedReal) return dir < 0 ? entry<L, -1, kStridedReal>() : entry<L, 1, kStridedReal>();
+  }
   if (kind == kContig) return dir < 0 ? entry<L, -1, kContig>() : entry<L, 1, kContig>();
   if constexpr (L <= 256) {
     if (kind == kR2C && dir < 0) return entry<L, -1, kR2C>();

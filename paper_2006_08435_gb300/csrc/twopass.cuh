@@ -41,6 +41,7 @@
 #include "codelets.cuh"
 #include "internal.h"
 #include "pencil.cuh"
+#include "primefactor.cuh"
 
 namespace fft3d {
 namespace tp {
@@ -48,30 +49,38 @@ namespace tp {
 using pc::l2_policy;
 using pc::ldg;
 using pc::stg;
-using pc::transform;
 using pc::twiddle;
 
+// The R-point transform of a step, by prime factors (primefactor.cuh) if PF.
+template <int R, int DIR, bool PF>
+FFT3D_HD void transform(float2* v) {
+  if constexpr (PF) pf::transform<R, DIR>(v);
+  else pc::transform<R, DIR>(v);
+}
+
 // Splits of an edge: y into A groups of B; x and z into two register steps,
-// BX (BZ) points first, AX (AZ) apart, then AX (AZ); T threads of pass 1.
+// BX (BZ) points first, AX (AZ) apart, then AX (AZ); T threads of pass 1; PF: the
+// steps by prime factors, where that is no slower.
 template <int L>
 struct Cfg;
-#define FFT3D_TP(L_, A_, AX_, AZ_, T_)                                  \
+#define FFT3D_TP(L_, A_, AX_, AZ_, T_, PF_)                             \
   template <>                                                           \
   struct Cfg<L_> {                                                      \
     static constexpr int L = L_, A = A_, B = L_ / A_;                   \
     static constexpr int AX = AX_, BX = L_ / AX_, AZ = AZ_, BZ = L_ / AZ_; \
     static constexpr int T1 = T_, W = 16; /* W: columns of a pass-2 block */ \
+    static constexpr bool PF = PF_;                                     \
   };
-FFT3D_TP(48, 3, 8, 4, 64)
-FFT3D_TP(60, 4, 12, 4, 64)
-FFT3D_TP(64, 4, 16, 4, 64)
-FFT3D_TP(72, 3, 12, 6, 96)
-FFT3D_TP(80, 4, 16, 4, 96)
-FFT3D_TP(90, 5, 15, 6, 160)
-FFT3D_TP(96, 4, 16, 8, 192)
-FFT3D_TP(100, 5, 10, 5, 128)
-FFT3D_TP(108, 4, 12, 9, 128)
-FFT3D_TP(128, 4, 16, 8, 128)
+FFT3D_TP(48, 3, 8, 4, 64, true)
+FFT3D_TP(60, 4, 12, 4, 64, false)
+FFT3D_TP(64, 4, 16, 4, 64, false)
+FFT3D_TP(72, 3, 12, 6, 96, true)
+FFT3D_TP(80, 4, 16, 4, 96, true)
+FFT3D_TP(90, 5, 15, 6, 160, false)
+FFT3D_TP(96, 4, 16, 8, 192, true)
+FFT3D_TP(100, 5, 10, 5, 128, true)
+FFT3D_TP(108, 4, 12, 9, 128, false)
+FFT3D_TP(128, 4, 16, 8, 128, false)
 #undef FFT3D_TP
 
 // Rows in shared memory for an x transform in two register steps, P lanes of Q
@@ -184,7 +193,7 @@ __global__ void __launch_bounds__(Dims<L>::T1 * (INPLACE && Dims<L>::MERGED ? Di
     float2 v[BX];
 #pragma unroll
     for (int i = 0; i < BX; ++i) v[i] = ldg(s + AX * i, once);
-    transform<BX, DIR>(v);
+    transform<BX, DIR, D::PF>(v);
     float2* x = sm + j * D::RP;
 #pragma unroll
     for (int k = 0; k < BX; ++k) x[slot(D::PD, BX * m + k)] = k ? twiddle<DIR>(v[k], __ldg(a.tx + k * AX + m)) : v[k];
@@ -206,7 +215,7 @@ __global__ void __launch_bounds__(Dims<L>::T1 * (INPLACE && Dims<L>::MERGED ? Di
     float2 v[AX];
 #pragma unroll
     for (int i = 0; i < AX; ++i) v[i] = x[slot(D::PD, BX * i + k)];
-    transform<AX, DIR>(v);
+    transform<AX, DIR, D::PF>(v);
 #pragma unroll
     for (int i = 0; i < AX; ++i) x[slot(D::PD, BX * i + k)] = v[i];
   }
@@ -222,7 +231,7 @@ __global__ void __launch_bounds__(Dims<L>::T1 * (INPLACE && Dims<L>::MERGED ? Di
     float2 v[B];
 #pragma unroll
     for (int j = 0; j < B; ++j) v[j] = x[j * D::RP];
-    transform<B, DIR>(v);
+    transform<B, DIR, D::PF>(v);
     float2* o = dst + kx;
 #pragma unroll
     for (int k = 0; k < B; ++k)
@@ -258,7 +267,7 @@ __global__ void __launch_bounds__(Dims<L>::T2) pass2_kernel(const __grid_constan
     float2 v[BZ];
 #pragma unroll
     for (int i = 0; i < BZ; ++i) v[i] = ldg(s + (long long)(AZ * i) * LL, once);
-    transform<BZ, DIR>(v);
+    transform<BZ, DIR, D::PF>(v);
     float2* x = sm + (m1 * A + n1) * W + q;
 #pragma unroll
     for (int k = 0; k < BZ; ++k)
@@ -277,7 +286,7 @@ __global__ void __launch_bounds__(Dims<L>::T2) pass2_kernel(const __grid_constan
     for (int n1 = 0; n1 < A; ++n1) {
 #pragma unroll
       for (int m = 0; m < AZ; ++m) v[n1][m] = x[(m * A + n1) * W];
-      transform<AZ, DIR>(v[n1]);
+      transform<AZ, DIR, D::PF>(v[n1]);
     }
     float2* o = base + kz2 * LL + q;
 #pragma unroll
@@ -285,7 +294,7 @@ __global__ void __launch_bounds__(Dims<L>::T2) pass2_kernel(const __grid_constan
       float2 u[A];
 #pragma unroll
       for (int n1 = 0; n1 < A; ++n1) u[n1] = v[n1][k];
-      transform<A, DIR>(u);
+      transform<A, DIR, D::PF>(u);
 #pragma unroll
       for (int k1 = 0; k1 < A; ++k1)
         stg(o + (long long)(BZ * k) * LL + k1 * NC, a.do_scale ? cscale(u[k1], a.scale) : u[k1],

@@ -62,7 +62,7 @@ __device__ __forceinline__ void box_y(const float2* x, int RP, float2* o, int nx
   float2 v[B];
 #pragma unroll
   for (int j = 0; j < B; ++j) v[j] = x[j * RP];
-  transform<B, DIR>(v);
+  pc::transform<B, DIR>(v);
 #pragma unroll
   for (int k = 0; k < B; ++k) stg(o + k * nx, k ? twiddle<DIR>(v[k], ty[k * A + n1]) : v[k], pol);
 }
@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(BoxX<LX>::T32) box1_kernel(const __grid_consta
     float2 v[BX];
 #pragma unroll
     for (int i = 0; i < BX; ++i) v[i] = ldg(s + AX * i, once);
-    transform<BX, DIR>(v);
+    pc::transform<BX, DIR>(v);
     float2* x = sm + j * D::RP;
 #pragma unroll
     for (int k = 0; k < BX; ++k) x[slot(D::PD, BX * m + k)] = k ? twiddle<DIR>(v[k], __ldg(a.tx + k * AX + m)) : v[k];
@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(BoxX<LX>::T32) box1_kernel(const __grid_consta
     float2 v[AX];
 #pragma unroll
     for (int i = 0; i < AX; ++i) v[i] = x[slot(D::PD, BX * i + k)];
-    transform<AX, DIR>(v);
+    pc::transform<AX, DIR>(v);
 #pragma unroll
     for (int i = 0; i < AX; ++i) x[slot(D::PD, BX * i + k)] = v[i];
   }
@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(BoxZ<A, LZ>::T) box2_kernel(const __grid_const
     float2 v[BZ];
 #pragma unroll
     for (int i = 0; i < BZ; ++i) v[i] = ldg(s + (long long)(AZ * i) * pl, once);
-    transform<BZ, DIR>(v);
+    pc::transform<BZ, DIR>(v);
     float2* x = sm + (m1 * A + n1) * W + q;
 #pragma unroll
     for (int k = 0; k < BZ; ++k) {
@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(BoxZ<A, LZ>::T) box2_kernel(const __grid_const
     for (int n1 = 0; n1 < A; ++n1) {
 #pragma unroll
       for (int m = 0; m < AZ; ++m) v[n1][m] = x[(m * A + n1) * W];
-      transform<AZ, DIR>(v[n1]);
+      pc::transform<AZ, DIR>(v[n1]);
     }
     float2* o = base + kz2 * pl + q;
 #pragma unroll
@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(BoxZ<A, LZ>::T) box2_kernel(const __grid_const
       float2 u[A];
 #pragma unroll
       for (int n1 = 0; n1 < A; ++n1) u[n1] = v[n1][k];
-      transform<A, DIR>(u);
+      pc::transform<A, DIR>(u);
 #pragma unroll
       for (int k1 = 0; k1 < A; ++k1)
         stg(o + (long long)(BZ * k) * pl + k1 * nc, a.do_scale ? cscale(u[k1], a.scale) : u[k1],

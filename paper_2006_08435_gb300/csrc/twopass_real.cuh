@@ -37,35 +37,37 @@ namespace tpr {
 using pc::l2_policy;
 using pc::ldg;
 using pc::stg;
-using pc::transform;
 using pc::twiddle;
 using tp::slot;
 
-// A groups of the y axis; x as P lanes of Q points, z as AZ BZ (first step BZ).
+// A groups of the y axis; x as P lanes of Q points, z as AZ BZ (first step BZ);
+// PF: the rows' steps by prime factors (the columns' always).
 template <int N>
 struct Split;
-#define FFT3D_TPR(N_, A_, P_, AZ_, T_)                    \
+#define FFT3D_TPR(N_, A_, P_, AZ_, T_, PF_)                  \
   template <>                                             \
   struct Split<N_> {                                      \
     static constexpr int A = A_, P = P_, AZ = AZ_, T = T_; \
+    static constexpr bool PF = PF_;                        \
   };
-FFT3D_TPR(48, 3, 8, 4, 32)
-FFT3D_TPR(60, 3, 6, 4, 64)
-FFT3D_TPR(64, 2, 16, 4, 64)
-FFT3D_TPR(72, 3, 6, 6, 64)
-FFT3D_TPR(80, 5, 8, 4, 64)
-FFT3D_TPR(90, 5, 9, 6, 64)
-FFT3D_TPR(96, 4, 8, 6, 64)
-FFT3D_TPR(100, 4, 10, 5, 96)
-FFT3D_TPR(108, 6, 9, 6, 64)
-FFT3D_TPR(120, 5, 12, 6, 96)
-FFT3D_TPR(128, 4, 16, 8, 96)
+FFT3D_TPR(48, 3, 8, 4, 32, true)
+FFT3D_TPR(60, 3, 6, 4, 64, true)
+FFT3D_TPR(64, 2, 16, 4, 64, true)
+FFT3D_TPR(72, 3, 6, 6, 64, true)
+FFT3D_TPR(80, 5, 8, 4, 64, true)
+FFT3D_TPR(90, 5, 9, 6, 64, false)
+FFT3D_TPR(96, 4, 8, 6, 64, true)
+FFT3D_TPR(100, 4, 10, 5, 96, true)
+FFT3D_TPR(108, 6, 9, 6, 64, true)
+FFT3D_TPR(120, 5, 12, 6, 96, true)
+FFT3D_TPR(128, 4, 16, 8, 96, true)
 #undef FFT3D_TPR
 
 template <int N>
 struct Dims {
   static constexpr int L = N / 2, HX = L + 1;
   static constexpr int A = Split<N>::A, B = N / A;
+  static constexpr bool PF = Split<N>::PF;
   static constexpr int P = Split<N>::P, Q = L / P, AZ = Split<N>::AZ, BZ = N / AZ;
   static_assert(A * B == N && P * Q == L && AZ * BZ == N, "splits");
   static constexpr tp::Layout rows = tp::row_layout(B, P, Q, HX);
@@ -102,7 +104,7 @@ __global__ void __launch_bounds__(Dims<N>::T1) rows_fwd_kernel(const __grid_cons
     float2 v[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) v[i] = ldg(s + P * i, once);
-    transform<Q, -1>(v);
+    tp::transform<Q, -1, D::PF>(v);
     float2* x = sm + j * D::RP;
 #pragma unroll
     for (int k = 0; k < Q; ++k) x[slot(PD, m * Q + k)] = k ? twiddle<-1>(v[k], __ldg(a.tx + k * P + m)) : v[k];
@@ -116,7 +118,7 @@ __global__ void __launch_bounds__(Dims<N>::T1) rows_fwd_kernel(const __grid_cons
     float2 v[P];
 #pragma unroll
     for (int i = 0; i < P; ++i) v[i] = x[slot(PD, Q * i + k)];
-    transform<P, -1>(v);
+    tp::transform<P, -1, D::PF>(v);
 #pragma unroll
     for (int i = 0; i < P; ++i) x[slot(PD, Q * i + k)] = v[i];
   }
@@ -135,7 +137,7 @@ __global__ void __launch_bounds__(Dims<N>::T1) rows_fwd_kernel(const __grid_cons
       const float2 O = make_float2(0.5f * (u.y + m.y), 0.5f * (m.x - u.x));
       v[j] = cadd(E, cmul_tw<-1>(O, w));
     }
-    transform<B, -1>(v);
+    tp::transform<B, -1, D::PF>(v);
     float2* o = dst + kx;
 #pragma unroll
     for (int i = 0; i < B; ++i)
@@ -163,7 +165,7 @@ __global__ void __launch_bounds__(Dims<N>::T1) rows_inv_kernel(const __grid_cons
     for (int i = 0; i < B; ++i) v[i] = ldg(src + i * D::HX + kx, once);
 #pragma unroll
     for (int i = 1; i < B; ++i) v[i] = twiddle<1>(v[i], a.ty[i * A + n1]);
-    transform<B, 1>(v);
+    tp::transform<B, 1, D::PF>(v);
     float2* x = sm + slot(PD, kx);
 #pragma unroll
     for (int j = 0; j < B; ++j) x[j * D::RP] = v[j];
@@ -192,7 +194,7 @@ __global__ void __launch_bounds__(Dims<N>::T1) rows_inv_kernel(const __grid_cons
       u[i] = make_float2(s.x - t.y, s.y + t.x);
       m[i] = make_float2(s.x + t.y, t.x - s.y);
     }
-    transform<P, 1>(u);
+    tp::transform<P, 1, D::PF>(u);
 #pragma unroll
     for (int k = 0; k < P; ++k)
       x[slot(PD, n + Q * k)] = k ? twiddle<1>(u[k], __ldg(a.tx + n * P + k)) : u[k];
@@ -200,7 +202,7 @@ __global__ void __launch_bounds__(Dims<N>::T1) rows_inv_kernel(const __grid_cons
       float2 v[P];
 #pragma unroll
       for (int i = 0; i < P; ++i) v[i] = m[P - 1 - i];
-      transform<P, 1>(v);
+      tp::transform<P, 1, D::PF>(v);
 #pragma unroll
       for (int k = 0; k < P; ++k)
         x[slot(PD, Q - n + Q * k)] = k ? twiddle<1>(v[k], __ldg(a.tx + (Q - n) * P + k)) : v[k];
@@ -216,7 +218,7 @@ __global__ void __launch_bounds__(Dims<N>::T1) rows_inv_kernel(const __grid_cons
     float2 v[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) v[i] = x[slot(PD, Q * k + i)];
-    transform<Q, 1>(v);
+    tp::transform<Q, 1, D::PF>(v);
     float2* o = dst + j * (A * L) + k;
 #pragma unroll
     for (int i = 0; i < Q; ++i) stg(o + P * i, cscale(v[i], sc), once);
@@ -262,7 +264,7 @@ __global__ void __launch_bounds__(Dims<N>::T2) cols_kernel(const __grid_constant
         v[i] = weighted(v[i], scale, fmaf(mz, mz, xy));
       }
     }
-    transform<BZ, DIR>(v);
+    tp::transform<BZ, DIR, true>(v);
     float2* x = sm + (m1 * A + n1) * W + q;
 #pragma unroll
     for (int k = 0; k < BZ; ++k) {
@@ -279,7 +281,7 @@ __global__ void __launch_bounds__(Dims<N>::T2) cols_kernel(const __grid_constant
     for (int n1 = 0; n1 < A; ++n1) {
 #pragma unroll
       for (int m = 0; m < AZ; ++m) v[n1][m] = x[(m * A + n1) * W];
-      transform<AZ, DIR>(v[n1]);
+      tp::transform<AZ, DIR, true>(v[n1]);
     }
     float2* o = dst + kz2 * PL + q;
 #pragma unroll
@@ -287,7 +289,7 @@ __global__ void __launch_bounds__(Dims<N>::T2) cols_kernel(const __grid_constant
       float2 u[A];
 #pragma unroll
       for (int n1 = 0; n1 < A; ++n1) u[n1] = v[n1][k];
-      transform<A, DIR>(u);
+      tp::transform<A, DIR, true>(u);
 #pragma unroll
       for (int k1 = 0; k1 < A; ++k1)
         stg(o + (long long)(BZ * k) * PL + k1 * NC,
