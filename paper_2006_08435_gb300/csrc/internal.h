@@ -269,6 +269,8 @@ int builtin_default_variant(bool mixed, int n, int batch, int precision);
 
 }  // namespace fft3d
 
+// The limits of a plan of `batch` cubic grids, as fft3d_plan_create checks them.
+int fft3d_internal_validate(int n, int batch, int precision);
 // A plan with a forced variant (plan.cu), for the autotuner.
 int fft3d_internal_create_variant(bool mixed, int nx, int batch, int precision, int direction,
                                   const int* dims, int count, int variant, fft3d_plan* out);

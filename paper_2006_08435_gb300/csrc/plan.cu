@@ -895,6 +895,10 @@ int validate_mixed(int count, const int* dims, int precision) {
 
 }  // namespace
 
+int fft3d_internal_validate(int n, int batch, int precision) {
+  return validate_uniform(n, n, n, batch, precision);
+}
+
 // Plan creation for the autotuner (tune.cu): a plan with a forced variant.
 int fft3d_internal_create_variant(bool mixed, int nx, int batch, int precision, int direction,
                                   const int* dims, int count, int variant, fft3d_plan* out) {

@@ -441,7 +441,11 @@ int fft3d_real_plan_create(int n, int batch, int precision, int direction, int n
     const fft3d::KernelInfo k = fft3d::real_kernel_info(n, direction == FFT3D_FORWARD ? -1 : 1);
     if (k.launch && !fft3d::two_pass_real(n, batch, direction))
       return fft3d::create_fused_real(n, batch, direction, norm, k, out_plan);
-    if (n > 2) return fft3d::create_pencil_real(n, batch, direction, norm, out_plan);
+    if (n > 2) {
+      // (the limits are those of the pair scheme's complex plan)
+      const int rc = k.launch ? FFT3D_SUCCESS : fft3d_internal_validate(n, (batch + 1) / 2, precision);
+      return rc ? rc : fft3d::create_pencil_real(n, batch, direction, norm, out_plan);
+    }
   }
   fft3d_plan inner = nullptr;
   const int rc = fft3d_plan_create(n, n, n, (batch + 1) / 2, precision, direction, norm, &inner);
@@ -460,7 +464,8 @@ int fft3d_real_plan_create_fixed(int n, int batch, fft3d_real_plan* out_plan) {
     return fft3d::create_fused_real(n, batch, FFT3D_FORWARD, FFT3D_NORM_NONE, k, out_plan);
   const int pairs = (batch + 1) / 2;
   fft3d_plan inner = nullptr;
-  int rc;
+  int rc = fft3d_internal_validate(n, pairs, FFT3D_FP32);
+  if (rc) return rc;
   if (k.launch) {
     rc = fft3d_plan_create(n, n, n, pairs, FFT3D_FP32, FFT3D_FORWARD, FFT3D_NORM_NONE, &inner);
   } else {
