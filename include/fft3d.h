@@ -184,6 +184,15 @@ int fft3d_plan_create(int nx, int ny, int nz, int batch, int precision,
                       int direction, int norm, fft3d_plan* out_plan);
 
 /*
+ * As fft3d_plan_create with nx = ny = nz = n, FFT3D_FP32, FFT3D_FORWARD and
+ * FFT3D_NORM_NONE, by three pencil passes of one arithmetic order at every edge
+ * without a fused kernel, also where fft3d_plan_create takes two passes
+ * (FFT3D_ERR_UNSUPPORTED_SIZE at the fused edges).  The Hartree energy of odd
+ * edges, which is returned in FP64, is taken from these spectra.
+ */
+int fft3d_plan_create_fixed(int n, int batch, fft3d_plan* out_plan);
+
+/*
  * Plan `count` cubic grids of different edges dims[g] (g < count) that are
  * transformed together in one persistent launch (mixed radix 2/3/5).
  *   count : 1..FFT3D_MAX_MIXED_GRIDS.

@@ -94,7 +94,7 @@ struct KernelInfo {
 // Passes for any edge 2..kAxisMaxLen with prime factors 2, 3, 5 (passes.cu).
 constexpr int kAxisMaxLen = 512;
 constexpr int kGeneralVariant = 10;  // plan variant of the general path
-constexpr int kFixedVariant = 11;    // the same as three passes at every edge (internal)
+constexpr int kFixedVariant = 11;    // three passes in the order of the mixed-radix plan (internal)
 constexpr int kAxisMaxStages = 12;
 
 // n / d = (hi32(n * mul) + n) >> shift for every n < 2^32 (make_fastdiv).
@@ -136,7 +136,9 @@ struct PencilKernel {
 };
 // kind: 0 strided, 1 rows, 2 real rows of 2 L points forward (dir -1), 3 the
 // same inverse (dir 1), 4 strided with weights (dir 1, even L), 5 strided for the
-// half spectra of real grids (even L); launch is null for an edge that is not plannable.
+// half spectra of real grids (even L), 6 and 7 strided and rows in the order of the
+// mixed-radix plan (dir -1, where kinds 0 and 1 have another); launch is null for an edge
+// that is not plannable.
 PencilKernel pencil_kernel_info(int L, int dir, int kind);
 
 // Two-pass transforms of cubic edges (twopass.cuh).  tx, ty, tz: W_L^(n1 k) at

@@ -165,7 +165,10 @@ int AxisPasses::create(PassKind kind_, int nx_, int ny_, int nz_, int batch_, in
   }
   // the pencil passes, where no two passes take their place
   for (int a = 0; a < 3 && !two.launch && !real.launch && !box[0].func; ++a) {
-    k[a] = pencil_kernel_info(len[a], dir, a == 0 ? kx : kind == kPassC2C ? 0 : 5);
+    k[a] = PencilKernel{};
+    if (fixed) k[a] = pencil_kernel_info(len[a], dir, a == 0 ? 7 : 6);
+    if (!k[a].launch)
+      k[a] = pencil_kernel_info(len[a], dir, a == 0 ? kx : kind == kPassC2C ? 0 : 5);
     if (!k[a].launch) return FFT3D_ERR_UNSUPPORTED_SIZE;
     if (k[a].smem > 48 * 1024 &&
         cudaFuncSetAttribute(k[a].func, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -60,8 +60,24 @@
 namespace fft3d {
 namespace pc {
 
-enum { kStrided = 0, kContig = 1, kR2C = 2, kC2R = 3, kWeighted = 4, kStridedReal = 5 };
-constexpr bool strided(int kind) { return kind == kStrided || kind == kWeighted || kind == kStridedReal; }
+enum {
+  kStrided = 0,
+  kContig = 1,
+  kR2C = 2,
+  kC2R = 3,
+  kWeighted = 4,
+  kStridedReal = 5,
+  kStridedFixed = 6,
+  kContigFixed = 7
+};
+constexpr bool strided(int kind) {
+  return kind == kStrided || kind == kWeighted || kind == kStridedReal || kind == kStridedFixed;
+}
+constexpr bool contig(int kind) { return kind == kContig || kind == kContigFixed; }
+// Complex kinds of the fixed plans, at the edges where the general ones have another
+// order of sums.
+constexpr bool fixed(int kind) { return kind == kStridedFixed || kind == kContigFixed; }
+constexpr bool fixed_edge(int L) { return L == 486 || L == 500 || L == 512; }
 
 constexpr bool smooth(int n) {
   if (n < 2) return false;
@@ -79,11 +95,12 @@ constexpr bool codelet(int r) {
 // The factor A of the split; B = L / A.
 // Edges without a fused kernel: B is the first radix of the edge's mixed-radix
 // plan (fft3d_axis_digit_map: the largest of 16, 15, 12, 10, 9, 8, ...) where
-// the rest is a codelet (all but 486 and 500).  The sums, twiddles and order
+// the rest is a codelet (all but 486, 500 and 512). The sums, twiddles and order
 // are then those of the plan's decimation-in-frequency stages, and the bits
 // those of the stage-by-stage passes before: the Hartree energy is returned
-// in FP64 and keeps its value.
-// Fused edges and 512, whose Hartree spectra come from other kernels, and real
+// in FP64 and keeps its value (486, 500 and 512: by kinds of the fixed plans' own,
+// three stages with two of them in one thread).
+// Fused edges, whose Hartree spectra come from other kernels, 486, 500, 512, and real
 // rows: the closest pair, the larger factor in the phase that holds one
 // transform per thread (64^3 x 4 12.2 us, with 16 * 4 16.8; 48^3 x 12 12.0,
 // with 16 * 3 16.2; 512^3 1060, with 16 * 2 * 16 1255).
@@ -98,7 +115,8 @@ constexpr int first_radix(int L) {
 constexpr int split_a(int L, int kind) {
   const bool real = kind == kR2C || kind == kC2R;
   const bool closest = real || L == 16 || L == 32 || L == 48 || L == 64 || L == 80 || L == 96 || L == 512;
-  if (codelet(L) && L <= (real ? 6 : kind == kContig ? 15 : 32)) return 1;
+  if (fixed(kind)) return L / first_radix(L);
+  if (codelet(L) && L <= (real ? 6 : contig(kind) ? 15 : 32)) return 1;
   int a = L / first_radix(L);
   if (!closest && codelet(a)) return a;
   int best = 0;
@@ -157,9 +175,10 @@ struct Cfg {
   static constexpr int SP = (L + 1) | 1;
   static constexpr int out_at = A == 1 ? W * SP : 0;
   static constexpr size_t smem = sizeof(float2) * (size_t)(exchange + (REAL ? out_at + W * SP : 0));
-  static constexpr int blocks = strided(KIND) || KIND == kContig ? 65536 / (T * reg_budget(A > B ? A : B)) : 1;
+  static constexpr int blocks =
+      (strided(KIND) || contig(KIND)) && !fixed(KIND) ? 65536 / (T * reg_budget(A > B ? A : B)) : 1;
   static_assert(A >= 1, "no split into two codelets");
-  static_assert(strided(KIND) || KIND == kContig || L <= 256, "real rows hold 2 L points");
+  static_assert(strided(KIND) || contig(KIND) || L <= 256, "real rows hold 2 L points");
 };
 
 // a * w (forward) or a * conj w, w a forward table twiddle.  The order of the
@@ -172,12 +191,12 @@ FFT3D_HD float2 twiddle(float2 a, float2 w) {
 }
 
 // The R-point transform of a step.  Above 16 points (but 32, which only fused
-// edges and 512 have) R = R1 * R2 with R1 = first_radix(R): the two decimation-
+// edges and 512 have, unless PLAN) R = R1 * R2 with R1 = first_radix(R): the two decimation-
 // in-frequency stages of the mixed-radix plan in registers, R1 points R2
 // apart, the twiddles W_R^(j k) as the table has them, then R2 points.
-template <int R, int DIR>
+template <int R, int DIR, bool PLAN = false>
 FFT3D_HD void transform(float2* v) {
-  if constexpr (R <= 16 || R == 32) {
+  if constexpr (R <= 16 || (R == 32 && !PLAN)) {
     DFT<R, DIR>::run(v);
   } else {
     constexpr int R1 = first_radix(R), R2 = R / R1;
@@ -265,7 +284,7 @@ __device__ __forceinline__ void split(const float2* twr, float2* dst, const floa
 // those of complex grids keep the order of the sums (see split_a).
 template <int R, int DIR, int KIND>
 __device__ __forceinline__ void step(float2* v) {
-  if constexpr (KIND == kStrided || KIND == kContig) transform<R, DIR>(v);
+  if constexpr (KIND == kStrided || contig(KIND) || fixed(KIND)) transform<R, DIR, fixed(KIND)>(v);
   else pf::transform<R, DIR>(v);
 }
 
@@ -303,7 +322,7 @@ __global__ void __launch_bounds__(Cfg<L, KIND>::T, Cfg<L, KIND>::blocks) pencil_
   for (int it = 0; it < C::I1; ++it) {
     const int e = threadIdx.x + it * T;
     if (e >= C::N1) break;
-    const int c = KIND == kContig ? e / A : e % W, n1 = KIND == kContig ? e % A : e / W;
+    const int c = contig(KIND) ? e / A : e % W, n1 = contig(KIND) ? e % A : e / W;
     if (c >= np) continue;
     if constexpr (KIND == kC2R) {
       // Z[k] = 2 E + i 2 O and Z[L-k] = conj(2 E) + i conj(2 O) with
@@ -397,7 +416,7 @@ __global__ void __launch_bounds__(Cfg<L, KIND>::T, Cfg<L, KIND>::blocks) pencil_
     for (int it = 0; it < C::I2; ++it) {
       const int e = threadIdx.x + it * T;
       if (e >= C::N2) break;
-      const int c = KIND == kContig ? e / B : e % W, k2 = KIND == kContig ? e % B : e / W;
+      const int c = contig(KIND) ? e / B : e % W, k2 = contig(KIND) ? e % B : e / W;
       if (c >= np) continue;
       float2 v[A];
 #pragma unroll
@@ -470,6 +489,10 @@ PencilKernel entry() {
 template <int L>
 PencilKernel entry_of(int dir, int kind) {
   if (kind == kStrided) return dir < 0 ? entry<L, -1, kStrided>() : entry<L, 1, kStrided>();
+  if constexpr (fixed_edge(L)) {
+    if (kind == kStridedFixed && dir < 0) return entry<L, -1, kStridedFixed>();
+    if (kind == kContigFixed && dir < 0) return entry<L, -1, kContigFixed>();
+  }
   if constexpr (L % 2 == 0) {
     if (kind == kWeighted && dir > 0) return entry<L, 1, kWeighted>();
     if (kind == kStridedReal) return dir < 0 ? entry<L, -1, kStridedReal>() : entry<L, 1, kStridedReal>();

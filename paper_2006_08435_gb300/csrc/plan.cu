@@ -1085,6 +1085,15 @@ int fft3d_plan_create(int nx, int ny, int nz, int batch, int precision, int dire
   return create_uniform(nx, ny, nz, batch, precision, direction, norm, -1, out_plan);
 }
 
+int fft3d_plan_create_fixed(int n, int batch, fft3d_plan* out_plan) {
+  int rc = validate_common(FFT3D_FP32, FFT3D_FORWARD, FFT3D_NORM_NONE, out_plan);
+  if (rc) return rc;
+  if ((rc = validate_uniform(n, n, n, batch, FFT3D_FP32))) return rc;
+  if (fused_size(n)) return FFT3D_ERR_UNSUPPORTED_SIZE;
+  return create_uniform(n, n, n, batch, FFT3D_FP32, FFT3D_FORWARD, FFT3D_NORM_NONE, kFixedVariant,
+                        out_plan);
+}
+
 int fft3d_plan_create_mixed(int count, const int* dims, int precision, int direction, int norm,
                             fft3d_plan* out_plan) {
   int rc = validate_common(precision, direction, norm, out_plan);

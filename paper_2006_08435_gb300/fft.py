@@ -102,6 +102,19 @@ class Plan:
                                           _NORM[norm], ctypes.byref(h)), "fft3d_plan_create")
         self._h = h
 
+    @classmethod
+    def fixed(cls, n: int, batch: int = 1) -> "Plan":
+        """A forward FP32 plan of cubic grids of an edge without a fused kernel, in
+        three passes of one arithmetic order (``fft3d_plan_create_fixed``)."""
+        p = cls.__new__(cls)
+        p.shape, p.batch = (int(n),) * 3, int(batch)
+        p.precision, p.inverse, p.norm = "fp32", False, "none"
+        h = ctypes.c_void_p()
+        L.check(L.lib().fft3d_plan_create_fixed(int(n), p.batch, ctypes.byref(h)),
+                "fft3d_plan_create_fixed")
+        p._h = h
+        return p
+
     @property
     def handle(self) -> int:
         return self._h.value or 0
@@ -314,6 +327,23 @@ def get_plan(nx, ny, nz, batch, precision="fp32", inverse=False, norm="none", de
                 p = Plan(nx, ny, nz, batch, precision, inverse, norm)
             _plan_cache[key] = p
     return p
+
+
+def _fixed_spectrum(x: torch.Tensor) -> torch.Tensor:
+    """fft3d(x) of cubic grids of odd edge by the plans of ``Plan.fixed``, cached
+    like those of ``get_plan``."""
+    if not x.numel() or x.dim() < 3 or not x.shape[-1] == x.shape[-2] == x.shape[-3]:
+        return fft3d(x)
+    n, dev = x.shape[-1], x.get_device()
+    out = torch.empty_like(x)
+    with _on_device(dev):
+        stream = _current_stream_handle(dev)
+        key = ("fixed", n, x.numel() // n ** 3, dev, stream)
+        with _cache_lock:
+            plan = _plan_cache.get(key)
+            if plan is None:
+                plan = _plan_cache[key] = Plan.fixed(n, key[2])
+        return plan.execute(x, out, stream)
 
 
 def fft3d(x: torch.Tensor, inverse: bool = False, norm: str = "none", precision: str = "fp32",

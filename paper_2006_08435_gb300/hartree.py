@@ -20,7 +20,8 @@ from __future__ import annotations
 import torch
 
 from . import _lib as L
-from .fft import _get_real_plan, _on_device, _rfft3d, _stream_handle, fft3d, irfft3d
+from .fft import (_fixed_spectrum, _get_real_plan, _on_device, _rfft3d, _stream_handle, fft3d,
+                  irfft3d)
 
 _ws_cache: dict = {}
 
@@ -149,7 +150,7 @@ class HartreeEnergy(torch.autograd.Function):
             rhohat = _rfft3d(rho.contiguous(), "none", "fp32", None, True)
             ctx.save_for_backward(rhohat)
             return energy_from_half_spectrum(rhohat, cell)
-        rhohat = fft3d(real_to_complex(rho))
+        rhohat = _fixed_spectrum(real_to_complex(rho))
         ctx.save_for_backward(rhohat)
         return energy_from_spectrum(rhohat, cell)
 
