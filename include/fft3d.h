@@ -306,10 +306,13 @@ int fft3d_selftest_wait_timeout(int64_t timeout_ns);
  * y axis splits into few groups of 10 to 32: two passes);
  * the launches of a batch above 40 MB alternate between the caller's stream
  * and a side stream of the plan, forked and joined by events (in a captured
- * graph, parallel branches). Mixed plans:
+ * graph, parallel branches); where 10 is the built-in default, in-place executes
+ * of 162 .. 174 and 236 .. 299 grids of 32^3, 55 .. 60 of 80^3 and 13 .. 15 of
+ * 128^3 run 13 (128^3: 6), which is faster there. Mixed plans:
  * 0 one launch of the mixed-edge kernel, 1 the launches of each distinct edge
  * in sequence (the two-pass kernels of 10 where they are the default of so
- * many grids; else the edge's kernel, the tensor-TMA kernels of 128^3 and
+ * many grids, but not packed and in place for 25 .. 27 of 96^3 and 13 .. 15 of
+ * 128^3; else the edge's kernel, the tensor-TMA kernels of 128^3 and
  * 32^3 .. 96^3 with one pair of tensor maps per grid, up to 32 grids of an edge;
  * beyond that, and for calls with pointer arrays, variant 0 at 48^3 and 96^3, 4
  * at 80^3, 3 at 32^3 and 5 at 128^3), 2 the launches of 1 on two concurrent

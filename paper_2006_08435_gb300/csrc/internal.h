@@ -265,7 +265,8 @@ cudaError_t launch_wait_selftest(unsigned* flag, unsigned* status, long long tim
 // override; else the FFT3D_TUNE_CACHE entry for this device and problem;
 // else, with FFT3D_TUNE=1, tune now (and record); else the built-in default.
 int pick_variant(bool mixed, int n, int batch, int precision, int direction, const int* dims,
-                 int count);
+                 int count,
+                 bool* is_default = nullptr);
 std::vector<int> variant_candidates(bool mixed, int n, int precision);
 int builtin_default_variant(bool mixed, int n, int batch, int precision);
 

@@ -228,29 +228,50 @@ int builtin_default_variant(bool mixed, int n, int batch, int precision) {
     // The general path (dependent launches of small blocks: three pencil
     // passes at 32^3, two passes at the others) fills the GPU where the ticket
     // kernels' large items leave it idle, and pays 4 us per launch of a chunk
-    // where they pay once.  In place it is up to 15% slower at 80^3, 96^3 and
-    // 128^3, so the lines there lie where that still costs under 4%.
+    // where they pay once.  In place it is slower (in_place_variant).
     // us, general path / the kernels before:
     // 32^3 x 16 8.5 / 10.5, x 32 13.1 / 12.2 (3), x 64 15.7 / 18.8, x 127 24.5 /
-    // 31.5, x 200 35.9 / 39.5 (13), x 400 67.6 / 66.5
-    case 32: return batch >= 300 ? 13 : batch >= 48 ? kGeneralVariant : 3;
-    // 48^3 x 1 7.2 / 11.8 (0), x 48 24.5 / 29.4 (13), x 300 128 / 152, x 2000 825 /
-    // 941 (in place 860 / 940)
+    // 31.5, x 140 26.2 / 26.7 (13), x 152 28.2 / 26.8 (one wave of its blocks), x 164
+    // 28.1 / 28.9, x 200 33.9 / 39.1, x 400 67.6 / 66.5
+    case 32:
+      return batch >= 300 || (batch >= 142 && batch < 162) ? 13 : batch >= 48 ? kGeneralVariant : 3;
+    // 48^3 x 1 7.2 / 11.8 (0), x 48 24.5 / 29.4 (13), x 300 128 / 152, x 2000 814 /
+    // 922 (in place 823 / 921)
     case 48: return kGeneralVariant;
     // 64^3 x 1 7.1 / 11.7 (5), x 4 8.7 / 18.4 (1), x 32 37.5 / 50.1 (7), x 80 90.6 /
     // 95.5 (8), x 96 107.8 / 105.4, x 1024 1100 / 957
     case 64: return batch >= 88 ? 8 : kGeneralVariant;
-    // 80^3 x 1 7.8 / 14.9 (0), x 20 47.7 / 59.3 (13), x 54 118.6 / 131.5 (in place
-    // 134.2 / 130.6), x 80 170 / 188 (196 / 188), x 400 825 / 859 (948 / 858)
+    // 80^3 x 1 7.8 / 14.9 (0), x 20 47.7 / 59.3 (13), x 54 116.3 / 130.8, x 80 169 / 189
+    // (in place 189 / 189), x 400 825 / 859 (948 / 858)
     case 80: return batch >= 64 ? 13 : kGeneralVariant;
-    // 96^3 x 1 10.8 / 17.1 (0), x 8 34.5 / 43.3 (13), x 24 98.1 / 102.5 (in place
-    // 101.1 / 101.3), x 28 113.9 / 116.9 (121.5 / 115.9), x 48 190 / 185
+    // 96^3 x 1 10.8 / 17.1 (0), x 8 34.5 / 43.3 (13), x 24 93.7 / 103.1 (in place
+    // 93.9 / 102.0), x 28 109.7 / 116.7 (112.9 / 116.0), x 48 190 / 185
     case 96: return batch >= 28 ? 13 : kGeneralVariant;
-    // 128^3 x 1 16.4 / 20.9 (5), x 2 24.3 / 32.0 (6), x 8 80.7 / 87.8, x 12 117.9 /
-    // 123.2 (in place 121.8 / 121.3), x 16 155.0 / 157.2 (163 / 155), x 32 301 / 295
+    // 128^3 x 1 16.4 / 20.9 (5), x 2 24.3 / 32.0 (6), x 8 77.9 / 87.0, x 12 114.8 /
+    // 122.4 (in place 118.1 / 121.6), x 16 151.1 / 157.0 (159 / 157), x 32 301 / 295
     case 128: return batch >= 16 ? 6 : kGeneralVariant;
     default: return 0;
   }
+}
+
+// The ticket kernel that a plan on the general path by default runs instead where
+// an execute is in place (pass 1 then stores behind its cluster's loads, or in
+// larger blocks), or -1.  us in place, general path / ticket kernel: 32^3 x 172
+// 29.5 / 28.8, x 200 34.1 / 37.0, x 232 39.0 / 39.2, x 256 42.6 / 41.2, x 299 49.4 / 46.7;
+// 80^3 x 53 126.4 / 129.6, x 55 132.3 / 131.9, x 59 141.4 / 136.6, x 63 149.9 /
+// 153.0; 96^3 x 27 109.0 / 112.4; 128^3 x 12 118.1 / 121.6, x 13 135.3 / 130.3, x 15
+// 150.6 / 148.3.
+static int in_place_variant(int n, int batch) {
+  if (n == 32 && ((batch >= 162 && batch < 175) || batch >= 236)) return 13;
+  if (n == 80 && batch >= 55 && batch < 61) return 13;
+  if (n == 128 && batch >= 13) return 6;
+  return -1;
+}
+// The same for an edge's grids in a mixed plan (packed buffers; a 16^3 grid on the
+// other branch): 96^3 x 24 108.0 / 108.4, x 26 121.4 / 114.5; 128^3 x 12 128.7 /
+// 126.4, x 13 141.9 / 136.1, x 15 160.3 / 153.9; 80^3 two passes at all of them.
+static bool in_place_unit(int n, int batch) {
+  return (n == 96 && batch >= 25) || (n == 128 && batch >= 13);
 }
 
 // The kernel of an edge's `batch` grids in a mixed plan, whose grids lie
@@ -291,8 +312,10 @@ struct Unit {
   // (KernelInfo::launch_maps) over these element offsets of the unit's grids
   bool use_maps = false;
   std::vector<long long> host_off;
-  // mixed-edge plans: the two-pass kernels (twopass.cuh) instead of `kernel`
+  // mixed-edge plans: the two-pass kernels (twopass.cuh) instead of `kernel`, or
+  // (in_place_kernel) but for packed calls in place
   TwoPassKernel two;
+  bool in_place_kernel = false;
   TwoPassArgs two_args;
   float2* d_two = nullptr;
 };
@@ -332,7 +355,7 @@ struct fft3d_plan_s {
   // device buffers shared by the units (owned)
   long long* d_off = nullptr;
   unsigned* d_status = nullptr;
-  bool general = false;  // variant kGeneralVariant
+  bool general = false;  // variant kGeneralVariant (units: in_place_variant's, if any)
   AxisPasses passes;
 };
 
@@ -435,7 +458,7 @@ int finish_unit(fft3d_plan p, Unit& u, bool identity) {
     u.two_args.do_scale = p->do_scale;
     u.two_args.off = p->d_off;
     u.two_args.map = u.d_map;
-    return rc;
+    if (rc || !u.in_place_kernel) return rc;
   }
   cudaError_t e = cudaFuncSetAttribute(u.kernel.func, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)u.kernel.smem);
@@ -512,7 +535,7 @@ int finish_unit(fft3d_plan p, Unit& u, bool identity) {
     if ((rc = upload(&u.d_frag, frag.data(), frag.size()))) return rc;
   }
   if ((rc = upload(&u.d_blocks, blocks.data(), blocks.size()))) return rc;
-  if (!identity && (rc = upload(&u.d_map, u.grids.data(), u.grids.size()))) return rc;
+  if (!identity && !u.d_map && (rc = upload(&u.d_map, u.grids.data(), u.grids.size()))) return rc;
   u.work_bytes = sizeof(unsigned) * (size_t)(1 + m);
   if (cudaMalloc(&u.d_work, u.work_bytes) != cudaSuccess) {
     cudaGetLastError();
@@ -566,10 +589,10 @@ int launch_general(fft3d_plan p, const float2* in, float2* out, cudaStream_t str
   return FFT3D_SUCCESS;
 }
 
-// Grids [first, first + count) of a unit (a unit of a ticket kernel: all).
+// Grids [first, first + count) of a unit (a ticket kernel: all, with the first).
 int launch_unit(fft3d_plan p, const Unit& u, int first, int count, const float2* in, float2* out,
                 const float2* const* in_ptrs, float2* const* out_ptrs, cudaStream_t stream) {
-  if (u.two.launch) {
+  if (u.two.launch && !(u.in_place_kernel && !in_ptrs && in == out)) {
     TwoPassArgs a = u.two_args;
     a.in = in;
     a.out = out;
@@ -583,7 +606,7 @@ int launch_unit(fft3d_plan p, const Unit& u, int first, int count, const float2*
     }
     return FFT3D_SUCCESS;
   }
-  {
+  if (first == 0) {
     // ticket kernels start from zeroed counters; cluster and whole-grid
     // kernels use none
     if (u.kernel.cluster == 0 && u.kernel.uses_work &&
@@ -622,7 +645,7 @@ int launch_unit(fft3d_plan p, const Unit& u, int first, int count, const float2*
 
 int launch(fft3d_plan p, const float2* in, float2* out, const float2* const* in_ptrs,
            float2* const* out_ptrs, cudaStream_t stream) {
-  if (p->general) return launch_general(p, in, out, stream);
+  if (p->general && (in != out || p->units.empty())) return launch_general(p, in, out, stream);
   const std::vector<Unit>& units = in_ptrs && !p->units_ptr.empty() ? p->units_ptr : p->units;
   int rc = FFT3D_SUCCESS;
   if (!p->mixed) return launch_unit(p, units[0], 0, p->batch, in, out, nullptr, nullptr, stream);
@@ -676,13 +699,15 @@ int create_uniform(int nx, int ny, int nz, int batch, int precision, int directi
   int rc;
   if ((rc = check_device())) return rc;
   const bool fused = nx == ny && ny == nz && fused_size(nx);
+  bool by_default = false;
   if (!fused) {
     // the general path is the only one for these edges
     if (precision != FFT3D_FP32) return FFT3D_ERR_UNSUPPORTED_PRECISION;
     if (variant < 0) variant = kGeneralVariant;
     if (variant != kGeneralVariant && variant != kFixedVariant) return FFT3D_ERR_INVALID_ARG;
   } else {
-    if (variant < 0) variant = pick_variant(false, nx, batch, precision, direction, nullptr, 0);
+    if (variant < 0)
+      variant = pick_variant(false, nx, batch, precision, direction, nullptr, 0, &by_default);
     const std::vector<int> cand = variant_candidates(false, nx, precision);
     if (std::find(cand.begin(), cand.end(), variant) == cand.end()) return FFT3D_ERR_INVALID_ARG;
   }
@@ -705,6 +730,15 @@ int create_uniform(int nx, int ny, int nz, int batch, int precision, int directi
       rc = FFT3D_ERR_ALLOC;
     else
       rc = create_general(p);
+    const int in_place = by_default ? in_place_variant(nx, batch) : -1;
+    if (!rc && in_place >= 0) {
+      Unit u;
+      u.kernel = fused_kernel_info(nx, direction, in_place);
+      u.grids.resize(batch);
+      for (int g = 0; g < batch; ++g) u.grids[g] = g;
+      p->units.push_back(u);
+      rc = finish_unit(p, p->units[0], true);
+    }
     if (rc) {
       cudaGetLastError();
       free_plan_buffers(p);
@@ -788,12 +822,17 @@ int create_mixed(int count, const int* dims, int direction, int norm, int varian
       const int ng = (int)u.grids.size();
       if (builtin_default_variant(false, n, ng, FFT3D_FP32) == kGeneralVariant)
         u.two = two_pass_apart_kernel_info(n, direction);
+      int v = unit_variant(n, ng);
       if (u.two.launch) {
-        p->units.push_back(u);
         ptr_units.push_back(u);
+        if (in_place_unit(n, ng) && ng <= kMixMaps) {
+          u.in_place_kernel = u.use_maps = true;
+          u.kernel = fused_kernel_info(n, direction, v);
+          for (int g : u.grids) u.host_off.push_back(p->offsets[g]);
+        }
+        p->units.push_back(u);
         continue;
       }
-      int v = unit_variant(n, ng);
       // the tensor-map kernels with per-grid maps: split-y (128^3) and the
       // thread-pair kernel (80^3, 96^3); for pointer arrays a kernel that
       // addresses grids through the plan's map

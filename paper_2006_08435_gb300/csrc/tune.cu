@@ -178,7 +178,8 @@ int run_autotune(bool mixed, int n, int batch, int precision, int direction, con
 }  // namespace
 
 int pick_variant(bool mixed, int n, int batch, int precision, int direction, const int* dims,
-                 int count) {
+                 int count, bool* is_default) {
+  if (is_default) *is_default = false;
   const std::vector<int> cand = variant_candidates(mixed, n, precision);
   auto allowed = [&](int v) { return std::find(cand.begin(), cand.end(), v) != cand.end(); };
   const char* ov = std::getenv(mixed ? "FFT3D_MIXED_VARIANT" : "FFT3D_VARIANT");
@@ -205,6 +206,7 @@ int pick_variant(bool mixed, int n, int batch, int precision, int direction, con
         allowed(v))
       return v;
   }
+  if (is_default) *is_default = true;
   return builtin_default_variant(mixed, n, batch, precision);
 }
 
