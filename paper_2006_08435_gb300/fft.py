@@ -371,7 +371,7 @@ def fft3d(x: torch.Tensor, inverse: bool = False, norm: str = "none", precision:
     # counts: the cached plan is looked up here (get_plan's key; a dict read
     # needs no lock), nothing is checked twice and the device is switched
     # only when it differs (64^3, one grid: 16.5 -> 11.9 us of host time per call).
-    if _current_device is not None and _current_device() != dev or _raw_stream is None:
+    if _raw_stream is None or _current_device is None or _current_device() != dev:
         with _on_device(dev):
             stream = _current_stream_handle(dev)
             return get_plan(nx, ny, nz, batch, precision, inverse, norm, dev,
