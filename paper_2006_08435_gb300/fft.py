@@ -359,9 +359,9 @@ def fft3d(x: torch.Tensor, inverse: bool = False, norm: str = "none", precision:
     points = x.numel()
     if out is None:
         out = torch.empty_like(x)
-    else:
+    elif points:
         _check_tensor(out, "out")
-        if points and out.numel() != points:
+        if out.numel() != points:
             raise ValueError(f"expected {points} points, got {points} and {out.numel()}")
     if points == 0:
         return out

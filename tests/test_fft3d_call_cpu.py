@@ -33,3 +33,12 @@ def test_a_missing_accessor_or_another_device_switches(stand_ins, monkeypatch, r
     x = torch.zeros(4, 4, 4, dtype=torch.complex64)
     assert fft.fft3d(x) == ("plan", 7)
     assert stand_ins == [x.get_device()]
+
+
+def test_no_grids_leave_out_unchecked(monkeypatch):
+    """An empty batch returns `out` as it is."""
+    seen = []
+    monkeypatch.setattr(fft, "_check_tensor", lambda t, name: seen.append(name))
+    x, out = torch.zeros(0, 4, 4, 4, dtype=torch.complex64), torch.zeros(3)
+    assert fft.fft3d(x, out=out) is out
+    assert seen == ["x"]
