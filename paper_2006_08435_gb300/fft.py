@@ -392,23 +392,27 @@ def fft3d(x: torch.Tensor, inverse: bool = False, norm: str = "none", precision:
 # still be executing it, and its memory is released (plan destroy, whose
 # cudaFree waits for work still using it) once the last reference to it
 # goes.  Like complex plans, real plans are kept per stream.
+# Fixed plans (of the Hartree energies) have a cache of their own, so that they
+# do not crowd out the plans of rfft3d and irfft3d at the same sizes.
 _REAL_CACHE_MAX = 4
 _real_cache: "collections.OrderedDict" = collections.OrderedDict()
+_fixed_cache: "collections.OrderedDict" = collections.OrderedDict()
 
 
 def _get_real_plan(n, batch, precision, inverse, norm, dev, stream=None, fixed=False) -> RealPlan:
-    key = (n, batch, precision, bool(inverse), norm, dev, _stream_handle(stream), fixed)
+    key = (n, batch, precision, bool(inverse), norm, dev, _stream_handle(stream))
+    cache = _fixed_cache if fixed else _real_cache
     with _cache_lock:
-        p = _real_cache.get(key)
+        p = cache.get(key)
         if p is not None:
-            _real_cache.move_to_end(key)
+            cache.move_to_end(key)
             return p
         with torch.cuda.device(dev):
             p = (RealPlan.fixed(n, batch) if fixed
                  else RealPlan(n, batch, precision, inverse, norm))
-        _real_cache[key] = p
-        while len(_real_cache) > _REAL_CACHE_MAX:
-            _real_cache.popitem(last=False)
+        cache[key] = p
+        while len(cache) > _REAL_CACHE_MAX:
+            cache.popitem(last=False)
     return p
 
 
