@@ -56,7 +56,7 @@ FFT3D_TPR(64, 2, 16, 4, 64, true)
 FFT3D_TPR(72, 3, 6, 6, 64, true)
 FFT3D_TPR(80, 5, 8, 4, 64, true)
 FFT3D_TPR(90, 5, 9, 6, 64, false)
-FFT3D_TPR(96, 4, 8, 6, 64, true)
+FFT3D_TPR(96, 4, 8, 8, 64, true)
 FFT3D_TPR(100, 4, 10, 5, 96, true)
 FFT3D_TPR(108, 6, 9, 6, 64, true)
 FFT3D_TPR(120, 5, 12, 6, 96, true)

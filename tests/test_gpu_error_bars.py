@@ -13,6 +13,8 @@ pytestmark = pytest.mark.gpu
 # edge: relative L2 error times 1e7, forward and inverse
 REAL = {36: (1.336, 1.396), 80: (1.383, 1.474), 108: (1.636, 1.705)}
 COMPLEX = {48: (1.498, 1.519), 80: (1.467, 1.469)}
+# edge: of eight densities, forth and back (the pair scheme's other kernel)
+ROUND = {96: 2.182}
 
 
 def rel(got, ref):
@@ -43,6 +45,13 @@ def complex_errors(n):
     return fwd, inv
 
 
+def round_trip_error(n):
+    from paper_2006_08435_gb300 import irfft3d, rfft3d
+    rho = np.stack([synth.hartree_density(n, seed=s)[0] for s in range(8)]).astype(np.float32)
+    back = irfft3d(rfft3d(torch.from_numpy(rho).cuda()), norm="by_n").cpu().numpy()
+    return rel(back, rho.astype(np.float64))
+
+
 @pytest.mark.parametrize("n", sorted(REAL))
 def test_real_errors(cuda, n):
     for got, bar in zip(real_errors(n), REAL[n]):
@@ -53,3 +62,8 @@ def test_real_errors(cuda, n):
 def test_complex_errors(cuda, n):
     for got, bar in zip(complex_errors(n), COMPLEX[n]):
         assert got <= bar * 1e-7
+
+
+@pytest.mark.parametrize("n", sorted(ROUND))
+def test_round_trip_errors(cuda, n):
+    assert round_trip_error(n) <= ROUND[n] * 1e-7
