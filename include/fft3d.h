@@ -488,11 +488,16 @@ int fft3d_real_plan_create(int n, int batch, int precision, int direction, int n
 
 /*
  * As fft3d_real_plan_create with FFT3D_FORWARD and FFT3D_NORM_NONE in FP32,
- * for spectra whose bits must not depend on the library's choice of kernel:
- * the dedicated kernels at n = 16, 32, 64 and 128 (at 64 and 128 with a
- * schedule, counters and batch * n * n/2 complex64 points of workspace),
- * elsewhere the pair scheme over complex transforms of one fixed arithmetic
- * order.  The Hartree energy, which is returned in FP64, is taken from these.
+ * for spectra that keep the arithmetic order, and so the bits, of the kernels
+ * that the Hartree energies (FP64 values) were first taken from, whatever
+ * fft3d_real_plan_create runs by now: the dedicated kernels at n = 16, 32, 64
+ * and 128 (at 64 and 128 with a schedule, counters and batch * n * n/2 complex64
+ * points of workspace), elsewhere the pair scheme over complex transforms, in
+ * three pencil passes but at n = 48, 80 and 96.  There it takes the persistent
+ * kernel, from 32, 8 and 4 pairs the thread-pair kernel (at 80 the
+ * double-buffered kernel from 4), or the variant that FFT3D_VARIANT or the
+ * tuning cache names (10 aside): at these three edges the bits depend on the
+ * batch, the environment and the tuning, at the others on none of them.
  */
 int fft3d_real_plan_create_fixed(int n, int batch, fft3d_real_plan* out_plan);
 

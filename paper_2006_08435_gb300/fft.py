@@ -250,8 +250,9 @@ class RealPlan:
 
     @classmethod
     def fixed(cls, n: int, batch: int = 1) -> "RealPlan":
-        """A forward FP32 plan whose spectra keep their bits from one version
-        of the kernels to the next (``fft3d_real_plan_create_fixed``)."""
+        """A forward FP32 plan whose spectra keep their bits from one version of
+        the kernels to the next (``fft3d_real_plan_create_fixed``; at 48, 80 and 96
+        they depend on the batch, the variant set and the tuning cache)."""
         p = cls.__new__(cls)
         p.n, p.batch = int(n), int(batch)
         p.precision, p.inverse, p.norm = "fp32", False, "none"
