@@ -524,8 +524,9 @@ def run_ours(args, ws, rank, local):
     # the Hartree energy and its gradient on real densities (the
     # differentiation workload: 128^3, cell of 10 bohr, densities of 64
     # Gaussians): forward = real-grid transform + FP64 reduction over the
-    # half spectrum, backward = seed on the half spectrum + real-grid
-    # inverse; a batch of `batch` densities per step, and one density alone
+    # half spectrum, backward = real-grid inverse that weights the half
+    # spectrum as it reads it; a batch of `batch` densities per step, and one
+    # density alone
     hartree = None
     if not args.no_hartree and n % 2 == 0:
         import numpy as np
@@ -552,8 +553,8 @@ def run_ours(args, ws, rank, local):
             msh = max_over_ranks(msh, ws, dev)
             half = n * n * (n // 2 + 1) * 8
             # algorithmic bytes per density: R2C (4 n^3 + half), reduction
-            # (half), seed (2 half), C2R (half + 4 n^3)
-            hbytes = 8 * n ** 3 + 5 * half
+            # (half), weighted C2R (half + 4 n^3)
+            hbytes = 8 * n ** 3 + 3 * half
             hartree[f"batch{hb}"] = {
                 "value": whole_job_rate(ws, hb, 1, msh), "unit": "densities/s (energy + gradient)",
                 "steps": kh, "ms_per_step": msh, "bytes_per_density": hbytes,
@@ -588,9 +589,9 @@ def run_ours(args, ws, rank, local):
             del rho
 
     # the general path (any edge up to 512, non-cubic grids): 256^3 x 4 and
-    # a non-cubic batch, one pencil pass per axis (three launches per chunk
-    # of grids); roofline fractions of the 16 n^3 bytes and of the passes'
-    # own traffic (three reads and writes of the grid, 48 n^3 bytes)
+    # a non-cubic batch, three passes over the grid and two; the roofline
+    # fraction of the 16 bytes per point, and the rate at which the passes' own
+    # 48 and 32 go through L2 (no fraction of HBM's: an intermediate may stay there)
     general = None
     if not args.no_general:
         general = {}
@@ -602,7 +603,7 @@ def run_ours(args, ws, rank, local):
             for _ in range(3):
                 pg.execute(xg, yg, stream)
             barrier()
-            kg = max(1, args.steps // 4)
+            kg = max(20, args.steps)  # (5 of 0.2 ms read 15% high)
             msg = max_over_ranks(timed_ms(lambda: pg.execute(xg, yg, stream), kg, stream), ws, dev)
             assert pg.device_status() == 0
             pts_g = nx_ * ny_ * nz_ * bg
@@ -610,8 +611,7 @@ def run_ours(args, ws, rank, local):
                 "value": whole_job_rate(ws, bg, 1, msg), "unit": "transforms/s", "steps": kg,
                 "ms_per_step": msg, "variant": pg.variant,
                 "roofline_frac": 16.0 * pts_g / (msg / 1e3) / 1e9 / peak,
-                # 16 bytes per point and pass: 256^3 three passes, the box two
-                "frac_of_pass_traffic": (48.0 if nx_ == 256 else 32.0) * pts_g / (msg / 1e3) / 1e9 / peak}
+                "pass_traffic_gbs": (48.0 if nx_ == 256 else 32.0) * pts_g / (msg / 1e3) / 1e9}
             del xg, yg, pg
 
     # the paper's setting: one grid per transform (Table 1), latency of
