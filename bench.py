@@ -589,7 +589,7 @@ def run_ours(args, ws, rank, local):
             del rho
 
     # the general path (any edge up to 512, non-cubic grids): 256^3 x 4 and
-    # a non-cubic batch, three passes over the grid and two; the roofline
+    # a non-cubic batch (nz x ny x nx), three passes over the grid and two; the roofline
     # fraction of the 16 bytes per point, and the rate at which the passes' own
     # 48 and 32 go through L2 (no fraction of HBM's: an intermediate may stay there)
     general = None
@@ -603,7 +603,7 @@ def run_ours(args, ws, rank, local):
             for _ in range(3):
                 pg.execute(xg, yg, stream)
             barrier()
-            kg = max(20, args.steps)  # (5 of 0.2 ms read 15% high)
+            kg = max(20, args.steps // 4)
             msg = max_over_ranks(timed_ms(lambda: pg.execute(xg, yg, stream), kg, stream), ws, dev)
             assert pg.device_status() == 0
             pts_g = nx_ * ny_ * nz_ * bg
