@@ -194,7 +194,8 @@ int fft3d_plan_create_fixed(int n, int batch, fft3d_plan* out_plan);
 
 /*
  * Plan `count` cubic grids of different edges dims[g] (g < count) that are
- * transformed together in one persistent launch (mixed radix 2/3/5).
+ * transformed together: by default the launches of each edge on two concurrent
+ * branches, or one persistent launch (mixed radix 2/3/5; fft3d_plan_variant).
  *   count : 1..FFT3D_MAX_MIXED_GRIDS.
  *   dims  : HOST array of `count` edge lengths.
  * Grid g's points live at element offset fft3d_plan_grid_offset(plan, g)
@@ -445,17 +446,15 @@ int fft3d_complex_to_real(const void* in, float* re, int64_t count, void* stream
  * and for any other input the imaginary parts of the self-mirrored bins
  * (kx, ky, kz each 0 or n/2) drop out.  `in` is not modified.
  *
- * At n = 16, 32, 64 and 128 in FP32 the transforms run as dedicated kernels:
- * each real row of n points is transformed as n/2 complex points and split
- * into its half spectrum (the even and odd samples' transforms,
- * X[k] = E[k] + W_n^k O[k]),
- * so the y and z transforms run on n/2 (+ 1) columns; at n = 16 and 32 one
- * block transforms a whole grid, at 64 and 128 one pass runs over the real
- * grids and one over the half spectra; each grid's error is relative to
- * itself.
- * At the other edges above 2 they run in FP32 as one pass per axis (x on real
- * rows, y and z on the half spectra), each grid on its own as well.  At n = 2
- * and in the tensor-core precisions two grids of the batch share one complex
+ * In FP32 above n = 2 each real row of n points is transformed as n/2 complex
+ * points and split into its half spectrum (the even and odd samples' transforms,
+ * X[k] = E[k] + W_n^k O[k]), so the y and z transforms run on n/2 (+ 1) columns,
+ * and each grid's error is relative to itself: at n = 16 and 32 one block
+ * transforms a whole grid; at n = 48, 60, 64, 72, 80, 90, 96, 100, 108, 120 and
+ * 128 two passes take x and part of y, then the rest (inverses of 100 grids and
+ * more at 64, of 48 and more at 128, and fixed plans at both: a persistent kernel
+ * of one pass over the real grids and one over the half spectra); at the other
+ * edges one pass runs per axis.  At n = 2 and in the tensor-core precisions two grids of the batch share one complex
  * transform (c = a + i b; the pair is separated with the symmetry above), so
  * a grid's rounding error is relative to the larger of its pair; cost per
  * pair: a packing pass, one complex transform of the plan's precision, a

@@ -16,9 +16,10 @@
 // there (32 bytes and more of shared-memory traffic per point, run-time
 // radices): 96 x 128 x 64, 64 grids 524 -> 412 us by the kernels alone, 261
 // with the launches and chunks of passes.cu; 256^3 x 4 827 -> 396; 100^3 x
-// 16 174 -> 94.  A pass is bound by its 16 bytes of traffic per point: 256^3
-// passes run at the HBM copy rate, L2-resident ones of 50 MB take 16 us of
-// which a copy kernel takes 12 (its ramp and drain 4).
+// 16 174 -> 94.  A pass is bound by latency and its launch: L2-resident ones of 50 MB
+// take 16 us of which a copy kernel takes 12 (its ramp and drain 4); L2 is at 17-34%,
+// L1 at 47-59%, HBM at 37% where x reads it and 58% in the z pass of 256^3, whose
+// grid exceeds L2.
 //
 // A block waits for nothing but its predecessor launch: passes are
 // programmatic dependent launches (launch_dependents at the start, wait

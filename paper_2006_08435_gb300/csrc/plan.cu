@@ -599,7 +599,9 @@ int launch_unit(fft3d_plan p, const Unit& u, int first, int count, const float2*
     a.in_ptrs = in_ptrs;
     a.out_ptrs = out_ptrs;
     a.first = first;
-    // (whether pointer arrays overlap is known on the device only)
+    // (whether pointer arrays overlap is known on the device only; 20 grids of 80^3
+    // and one of 16^3, packed 51.0 us, packed in place 49.7, pointer arrays 57.8, by
+    // the edge's ticket kernel 92.6)
     if (u.two.launch(a, count, in_ptrs || in == out, stream) != cudaSuccess) {
       cudaGetLastError();
       return FFT3D_ERR_CUDA;

@@ -12,10 +12,11 @@
 //     the z transforms and the A-point DFT over n1, and stores rows k2 + B k1, the
 //     same points it read.
 // A grid crosses L2 twice (32 bytes per point; the separate passes of
-// pencil.cuh 48), which with HBM's own fills and write-backs is what bounds
-// both: 48 and 64 bytes per point at the 13.8 TB/s that a copy from and to HBM
-// reaches there (64^3 x 106: 97 us; measured 119).  The rest is L1 and latency:
-// short runs, bank conflicts, loads in flight.  Hence runs of 64 bytes and more
+// pencil.cuh 48).  Neither HBM nor L2 bounds that: at the 12.5 TB/s of L2-resident
+// copies 64^3 x 106 would take 71 us, of HBM's one round trip 66; measured 119, with
+// L2 at 24-29% and HBM at 22-28% (pass 1) and below 1% (pass 2: the intermediate
+// stays in L2).  L1 does (50-80%), and latency: short runs, bank conflicts, loads in
+// flight, the ramp and drain of a chunk's launch.  Hence runs of 64 bytes and more
 // in the first step of pass 1, shared rows whose strided accesses do not conflict
 // (row_layout), columns taken 16 at a time across the rows k2 (whatever L is, full
 // and aligned to 128 bytes where B L is a multiple of 16), and
@@ -34,6 +35,10 @@
 // everybody's loads.  us in place, cluster / one block: 48^3 x 253 158 / 116, 60^3 x
 // 129 178 / 135, 64^3 x 106 156 / 120, 80^3 x 54 140 / 134, 96^3 x 31 139 / 144, 128^3 x
 // 32 317 / 379.
+//
+// Steps by prime factors (Cfg::PF; primefactor.cuh) for the errors: one orbital of
+// 80^3 1.52e-7 -> 1.41e-7, 48^3 1.50 -> 1.38; 48^3 x 198 in place 85.7 -> 82.1 us, x 4
+// 6.9 -> 6.5, the others within 1%.
 #pragma once
 
 #include <cuda_runtime.h>

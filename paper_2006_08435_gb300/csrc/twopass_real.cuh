@@ -11,21 +11,23 @@
 //     pass 2, block (grid, z, n1): times W_N^(-n1 k2) and the B-point DFT over k2
 //     of a column in one thread, then the rows: half bins to complex points and
 //     the x transform.
-// The spectrum crosses L2 once less than in the pencil passes: with HBM's fills
-// and write-backs 48 and 64 bytes per complex point (96^3 x 32, one direction: 50
-// and 67 us at the 13.8 TB/s that copies reach there; HBM alone 34).  What bounds
-// the row kernels is L1, in wavefronts of shared memory and of twiddles: hence
-// the row layout of twopass.cuh, which hardly an access conflicts in, and lanes
-// along the rows in the steps whose twiddles are then one address for a warp
-// (96^3 x 32, with padded runs and lanes along the columns: forward 77.5, inverse
-// 98.1 us; now 66.3 and 79.2).  The B HX columns of a group lie side by side, so a
-// block of the column kernel takes 16 of them whatever HX is.
+// The spectrum crosses L2 once less than in the pencil passes, and stays there in
+// between (HBM at 27-30% in the pass on its side, 1% in the other).  Neither HBM (96^3 x
+// 32, one direction: 34 us) nor L2 (20-32%) bounds it: the row kernels are bound by L1
+// (70-73%), in wavefronts of shared memory and of twiddles: hence the row layout of
+// twopass.cuh, which hardly an access conflicts in, and lanes along the rows in the
+// steps whose twiddles are then one address for a warp (96^3 x 32, with padded runs and
+// lanes along the columns: forward 77.5, inverse 98.1 us; now 63.8 and 77.6).  The column
+// kernels wait for loads.  The B HX columns of a group lie side by side, so a block of
+// the column kernel takes 16 of them whatever HX is.
 // Splits per edge from a sweep over A, P, AZ and threads; the next best lies 1-5%
-// behind.  us, pencil passes / two passes, forward and inverse: 48^3 x 300 114.5 /
-// 76.5, 122.2 / 85.6; 60^3 x 200 150.0 / 113.8, 165.3 / 115.1; 80^3 x 60 102.2 / 74.7,
-// 108.3 / 81.4; 96^3 x 32 93.4 / 66.3, 100.1 / 79.2; 100^3 x 40 132.3 / 106.4, 140.9 /
-// 115.2; 120^3 x 24 148.3 / 102.1, 148.0 / 117.8; one grid: within 1.5 us (48^3 8.5 /
-// 6.6, 96^3 11.5 / 10.6, 100^3 10.1 / 11.2).
+// behind.  us, pencil passes / two passes (these replayed from a graph), forward and
+// inverse: 48^3 x 300 114.5 / 74.1, 122.2 / 81.9; 60^3 x 200 150.0 / 109.2, 165.3 / 112.7;
+// 80^3 x 60 102.2 / 71.2, 108.3 / 78.6; 96^3 x 32 93.4 / 63.5, 100.1 / 77.1; 100^3 x 40
+// 132.3 / 103.6, 140.9 / 111.0; 120^3 x 24 148.3 / 100.3, 148.0 / 113.4; one grid: within
+// 1.5 us (48^3 8.5 / 6.6, 96^3 11.5 / 9.8, 100^3 10.1 / 11.2).  96^3 has AZ = 8 for its
+// errors: eight densities forth and back 2.19e-7 with 6, 2.12e-7 with 8 (forward
+// 65.1 / 63.8 us).
 #pragma once
 
 #include "hartree.cuh"
