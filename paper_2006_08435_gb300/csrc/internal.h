@@ -189,6 +189,12 @@ struct RealPassKernel {
   int A = 0, AX = 0, AZ = 0;
 };
 RealPassKernel real_pass_kernel_info(int n, int dir);  // launch null: none
+// Edges whose real grids always run on these or, at 16 and 32, on a whole grid per
+// block: no pencil passes are compiled for them.
+constexpr bool real_kernels(int n) {
+  return n == 16 || n == 32 || n == 48 || n == 60 || n == 64 || n == 72 || n == 80 || n == 90 ||
+         n == 96 || n == 100 || n == 108 || n == 120 || n == 128;
+}
 
 // Two-pass transforms of boxes (twopass_box.cuh): ny = A B.
 struct BoxArgs {

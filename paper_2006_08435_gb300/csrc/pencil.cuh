@@ -494,12 +494,12 @@ PencilKernel entry_of(int dir, int kind) {
     if (kind == kStridedFixed && dir < 0) return entry<L, -1, kStridedFixed>();
     if (kind == kContigFixed && dir < 0) return entry<L, -1, kContigFixed>();
   }
-  if constexpr (L % 2 == 0) {
+  if constexpr (L % 2 == 0 && !real_kernels(L)) {
     if (kind == kWeighted && dir > 0) return entry<L, 1, kWeighted>();
     if (kind == kStridedReal) return dir < 0 ? entry<L, -1, kStridedReal>() : entry<L, 1, kStridedReal>();
   }
   if (kind == kContig) return dir < 0 ? entry<L, -1, kContig>() : entry<L, 1, kContig>();
-  if constexpr (L <= 256) {
+  if constexpr (L <= 256 && !real_kernels(2 * L)) {
     if (kind == kR2C && dir < 0) return entry<L, -1, kR2C>();
     if (kind == kC2R && dir > 0) return entry<L, 1, kC2R>();
   }

@@ -340,6 +340,7 @@ cudaError_t launch_inv(const RealPassArgs& a, int grids, cudaStream_t s) {
 template <int N>
 RealPassKernel entry(int dir) {
   using D = Dims<N>;
+  static_assert(real_kernels(N), "the pencil passes leave this edge out");
   RealPassKernel k;
   k.launch = dir < 0 ? &launch_fwd<N> : &launch_inv<N>;
   k.func[0] = dir < 0 ? (const void*)&rows_fwd_kernel<N> : (const void*)&rows_inv_kernel<N>;
